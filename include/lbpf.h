@@ -124,7 +124,7 @@ int lbpf_get_state(lbpf_sim* sim, double* g, double* h, double* f);
  * graph captured on first use.  Returns LBPF_OK, or a sticky error. */
 int lbpf_step(lbpf_sim* sim, int64_t n_steps);
 
-/* Same as lbpf_step but without graphs: each kernel launch is bracketed by CUDA
+/* Same as lbpf_step but without graphs: the kernels of each phase are bracketed by CUDA
  * events recorded on the handle's stream, and the call returns (synchronously)
  * the summed device time of the phase-field kernels in ms_kernels[0], of the
  * U/theta kernels in ms_kernels[1], and the wall span of the n steps in
@@ -171,8 +171,11 @@ int lbpf_load(lbpf_sim* sim, const char* path);
 /* Tiling of the step kernels: node rows per block `by` (4..8; a block is
  * 32 x by threads, one node per thread and plane) and z-chunk length
  * (>= 1; the z range is split into chunks processed by separate thread
- * blocks).  0 keeps the current value.  Takes effect at the next lbpf_step
- * (the step graph is re-captured). */
+ * blocks).  Steps that run node-wise (FP64, FP16 and BF16 on 3D lattices, FP32
+ * and small 2D grids where that is faster) use blocks of 16 x by threads over
+ * consecutive nodes of a plane.  Results do not depend on the tiling.  0 keeps
+ * the current value.  Takes effect at the next lbpf_step (the step graph is
+ * re-captured). */
 int lbpf_set_tiling(lbpf_sim* sim, int32_t by, int32_t zchunk);
 int lbpf_get_tiling(const lbpf_sim* sim, int32_t* by, int32_t* zchunk);
 

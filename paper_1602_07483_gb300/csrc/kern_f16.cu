@@ -5,7 +5,8 @@ namespace lbpf {
 const KernelTable& table_f16() {
   static const KernelTable t = [] {
     KernelTable k = build_table<__half>();
-    add_fixed_kernels_f16(k);
+    add_node_kernels_f16(k);
+    add_moment_kernels_f16(k);
     add_step_kernels_f16(k);
     return k;
   }();

@@ -5,7 +5,10 @@ namespace lbpf {
 const KernelTable& table_f32() {
   static const KernelTable t = [] {
     KernelTable k = build_table<float>();
+    add_tile_kernels_f32(k);
     add_fixed_kernels_f32(k);
+    add_node_kernels_f32(k);
+    add_moment_kernels_f32(k);
     add_step_kernels_f32(k);
     return k;
   }();

@@ -5,7 +5,8 @@ namespace lbpf {
 const KernelTable& table_f64() {
   static const KernelTable t = [] {
     KernelTable k = build_table<double>();
-    add_fixed_kernels_f64(k);
+    add_node_kernels_f64(k);
+    add_moment_kernels_f64(k);
     return k;
   }();
   return t;

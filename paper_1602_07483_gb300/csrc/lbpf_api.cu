@@ -87,6 +87,7 @@ double min_effective_tau(int kind, double e1, double e2, double c_eta, double* a
 struct OneLaunch {
   OneLaunchFn fn = nullptr;   // null: no one-launch kernel for these lattices and storage
   bool on = false;            // schedule selected (lbpf_set_schedule)
+  WorkItem* d_items = nullptr;  // its tiles
   int* d_sched = nullptr;     // order[ntickets] | dep_off[nitems + 1] | dep[...]
   unsigned* d_ctl = nullptr;  // next ticket, then one done flag per work item
   size_t ctl_bytes = 0;
@@ -95,6 +96,19 @@ struct OneLaunch {
   int grid = 0;               // resident blocks on the device
   size_t smem = 0;
   unsigned polls = kWaitPolls;  // bound of each wait (lbpf_set_wait_polls)
+};
+
+// The launches of one step: the phase-field kernels, then the U/theta kernels, all over the
+// same blocks (one per work item).
+struct StepPlan {
+  int n = 0, nphi = 0;  // kernels per step; the first nphi are the phase-field phase
+  StepLaunch fn[4] = {};
+  size_t smem[4] = {};
+  int threads_y = 1, threads_x = 32;
+  bool node_wise = false;
+  const SimDev* dd = nullptr;
+  WorkItem* items = nullptr;  // device
+  int nitems = 0;
 };
 
 struct lbpf_sim {
@@ -113,9 +127,9 @@ struct lbpf_sim {
   void* th[3] = {};  // theta levels like phi (theta^{n-1} is the FP16/BF16 shift of f)
   SimDev hd{};
   SimDev* dd = nullptr;
-  WorkItem* d_items = nullptr;
-  int nitems = 0;
-  int by = MAX_BLOCK_ROWS, zchunk = 0;
+  StepPlan plan;
+  int by = MAX_BLOCK_ROWS, zchunk = 0;  // tiling in effect
+  int zreq = 0;                         // z-chunk asked for (0: the default)
   double* d_part = nullptr;  // reduction partials + 4 results
   int npart = 0;
   double* d_small = nullptr; // tip output
@@ -127,8 +141,6 @@ struct lbpf_sim {
   int64_t step_base = 0;  // step count carried in from a checkpoint
   int sticky = LBPF_OK;
   double theta0 = 0.0, U0 = 0.0;
-  StepLaunch fphi = nullptr, futh = nullptr;
-  size_t smem_phi = 0, smem_uth = 0;
   OneLaunch ol;
   const int* batch_err = nullptr;  // wait-failure flag of the batch this handle is stepped by
 };
@@ -141,14 +153,10 @@ struct lbpf_batch {
   cudaEvent_t ev = nullptr;     // orders the batch stream against the members' own streams
   SimDev* h_desc = nullptr;     // pinned copy of the member descriptors last uploaded to dd
   SimDev* dd = nullptr;
-  WorkItem* d_items = nullptr;
-  int nitems = 0;
+  StepPlan plan;
   int by = MAX_BLOCK_ROWS;
   int zchunk = 0;               // z-chunk request of the current tiling (0: each member's default)
-  StepLaunch fphi = nullptr, futh = nullptr;
-  size_t smem_phi = 0, smem_uth = 0;
   OneLaunch ol;
-  std::vector<int> zchunks;     // z-chunk of each member under the current tiling
   cudaGraphExec_t gexec = nullptr;
   bool graph_ok = false;
 };
@@ -217,8 +225,10 @@ __global__ void k_wait_probe(const unsigned* flag, const int* dep, unsigned poll
 }
 
 void free_one_launch(OneLaunch& ol) {
+  if (ol.d_items) cudaFree(ol.d_items);
   if (ol.d_sched) cudaFree(ol.d_sched);
   if (ol.d_ctl) cudaFree(ol.d_ctl);
+  ol.d_items = nullptr;
   ol.d_sched = nullptr;
   ol.d_ctl = nullptr;
   ol.sc = StepSched{};
@@ -257,13 +267,15 @@ int setup_one_launch(OneLaunch& ol, const std::vector<WorkItem>& items, const st
   all.insert(all.end(), dep_off.begin(), dep_off.end());
   all.insert(all.end(), dep.begin(), dep.end());
   ol.ctl_bytes = (n + 1) * sizeof(unsigned);
-  if (cudaMalloc(&ol.d_sched, all.size() * sizeof(int)) != cudaSuccess ||
+  if (cudaMalloc(&ol.d_items, n * sizeof(WorkItem)) != cudaSuccess ||
+      cudaMalloc(&ol.d_sched, all.size() * sizeof(int)) != cudaSuccess ||
       cudaMalloc(&ol.d_ctl, ol.ctl_bytes) != cudaSuccess) {
     cudaGetLastError();
     free_one_launch(ol);
     return LBPF_ENOMEM;
   }
-  if (cudaMemcpy(ol.d_sched, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) {
+  if (cudaMemcpy(ol.d_items, items.data(), n * sizeof(WorkItem), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(ol.d_sched, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) {
     free_one_launch(ol);
     return LBPF_ECUDA;
   }
@@ -279,72 +291,143 @@ int setup_one_launch(OneLaunch& ol, const std::vector<WorkItem>& items, const st
   return LBPF_OK;
 }
 
-int set_smem_attrs(lbpf_sim* s) {
-  const KernelTable& t = *s->kt;
-  const int a = q_index(s->lat.q_phi), b = q_index(s->lat.q_u), c = qt_index(s->lat.q_theta);
-  if (raise_smem_limit(t.phi_fn[a][0], s->device) || raise_smem_limit(t.uth_fn[b][c][0], s->device) ||
-      raise_smem_limit(t.phi_fn[a][1], s->device) || raise_smem_limit(t.uth_fn[b][c][1], s->device)) {
-    s->sticky = LBPF_ECUDA;
-    return LBPF_ECUDA;
-  }
+// Raises the limits of the tiled kernels of lattices `l` (none where the storage has none).
+int set_smem_attrs(const KernelTable& t, const lbpf_lattice& l, int device) {
+  const int a = q_index(l.q_phi), b = q_index(l.q_u), c = qt_index(l.q_theta);
+  for (int v = 0; v < 2; ++v)
+    for (const void* fn : {t.phi_fn[a][v], t.uth_fn[b][c][v]})
+      if (fn && raise_smem_limit(fn, device) != LBPF_OK) return LBPF_ECUDA;
   return LBPF_OK;
+}
+
+// Kernels of the step of lattices `l` for blocks of `by` rows, or node-wise.
+void plan_kernels(StepPlan& p, const KernelTable& t, const lbpf_lattice& l, int by, bool node_wise) {
+  const int a = q_index(l.q_phi), b = q_index(l.q_u), c = qt_index(l.q_theta);
+  p.node_wise = node_wise;
+  if (node_wise) {
+    p.n = 4;
+    p.nphi = 2;
+    p.fn[0] = t.phi_node[a];
+    p.fn[1] = t.phi_moment[a];
+    p.fn[2] = t.uth_node[b][c];
+    p.fn[3] = t.uth_moment[b][c];
+    for (size_t& m : p.smem) m = 0;
+    p.threads_x = node_threads(by);
+    p.threads_y = 1;
+    return;
+  }
+  const int v = block_variant(l.q_phi, by);
+  p.n = 2;
+  p.nphi = 1;
+  p.fn[0] = t.phi[a][v];
+  p.fn[1] = t.uth[b][c][v];
+  p.smem[0] = phi_smem_bytes(t, l.q_phi, by);
+  p.smem[1] = uth_smem_bytes(t, l.q_u, l.q_theta, by);
+  p.threads_x = 32;
+  p.threads_y = by;
+}
+
+// Copies the work items to the device (replacing the plan's).
+int plan_items(StepPlan& p, const std::vector<WorkItem>& items) {
+  if (p.items) cudaFree(p.items);
+  p.items = nullptr;
+  p.nitems = 0;
+  if (cudaMalloc(&p.items, items.size() * sizeof(WorkItem)) != cudaSuccess) {
+    cudaGetLastError();
+    p.items = nullptr;
+    return LBPF_ENOMEM;
+  }
+  if (cudaMemcpy(p.items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice) != cudaSuccess)
+    return LBPF_ECUDA;
+  p.nitems = (int)items.size();
+  return LBPF_OK;
+}
+
+// Whether simulations of `sites` nodes in all step node-wise (lbpf_nodewise.cuh) or tiled.
+// The tiled step reads the distributions once but spends 1.4 collisions per node, and small
+// grids have too few tiles for the chip; the node-wise step reads them twice.  Measured
+// (microseconds per step, tiled / node-wise):
+//   FP64, bound by its arithmetic, always node-wise: 128^3 D3Q19/D3Q19 2700 / 1340, 32^3 965 / 64,
+//   8000^2 26500 / 23400.
+//   3D FP16/BF16, bound by instructions and latency, always node-wise: 96^3 D3Q19/D3Q19/D3Q7
+//   292 / 142, 256^3 1860 / 1630, 512^3 D3Q19 x 3 15450 / 15420.
+//   3D FP32: 96^3 235 / 111, 256^3 1703 / 1683, 400^3 6220 / 6150 with theta on D3Q7; with theta on
+//   D3Q19 192^3 924 / 903 but 256^3 1994 / 2066 and 512^3 14900 / 16050.
+//   2D FP32 and FP16 are tiled once the second read leaves L2: 500^2 29 / 17, 1000^2 58 / 62,
+//   4000^2 671 / 848.
+bool steps_node_wise(const KernelTable& t, const lbpf_lattice& l, long long sites) {
+  if (t.tbytes == 8) return true;
+  if (lattice_is_2d(l.q_phi)) return sites <= 700000;
+  if (t.sbytes == 2) return true;
+  return l.q_theta + l.q_u <= 26 || sites <= 8000000;
 }
 
 int apply_tiling(lbpf_sim* s, int by, int zchunk) {
   const KernelTable& t = *s->kt;
   if (lattice_is_2d(s->lat.q_phi)) by = 1;  // 2D: one-row blocks, no y halo
   s->by = by;
-  const int v = block_variant(s->lat.q_phi, by);
-  s->fphi = t.phi[q_index(s->lat.q_phi)][v];
-  s->futh = t.uth[q_index(s->lat.q_u)][qt_index(s->lat.q_theta)][v];
-  s->zchunk = zchunk > 0 ? zchunk : default_zchunk(s->kg.nx, s->kg.ny, s->kg.nz, by);
-  s->smem_phi = phi_smem_bytes(t, s->lat.q_phi, by);
-  s->smem_uth = uth_smem_bytes(t, s->lat.q_u, s->lat.q_theta, by);
-  int maxsm = 0;
-  CK(s, cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, s->device));
-  if ((int)s->smem_phi > maxsm || (int)s->smem_uth > maxsm) return LBPF_EINVAL;
+  s->zreq = zchunk;
+  plan_kernels(s->plan, t, s->lat, by, steps_node_wise(t, s->lat, s->nsite));
+  s->plan.dd = s->dd;
+  const lbpf_grid& k = s->kg;
+  const int tile_zc = zchunk > 0 ? zchunk : default_zchunk(k.nx, k.ny, k.nz, by);
   std::vector<WorkItem> items;
-  build_items(0, s->kg.nx, s->kg.ny, s->kg.nz, by, s->zchunk, items);
-  if (s->d_items) cudaFree(s->d_items);
-  s->d_items = nullptr;
-  CK(s, cudaMalloc(&s->d_items, items.size() * sizeof(WorkItem)));
-  CK(s, cudaMemcpy(s->d_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
-  s->nitems = (int)items.size();
+  if (s->plan.node_wise) {
+    const int threads = s->plan.threads_x;
+    const int zc = zchunk > 0 ? zchunk : node_zchunk(node_blocks(k.nx, k.ny, k.nz, threads), k.nz);
+    build_node_items(0, k.nx, k.ny, k.nz, threads, zc, items);
+    s->zchunk = zc;
+  } else {
+    int maxsm = 0;
+    CK(s, cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, s->device));
+    if ((int)s->plan.smem[0] > maxsm || (int)s->plan.smem[1] > maxsm) return LBPF_EINVAL;
+    build_items(0, k.nx, k.ny, k.nz, by, tile_zc, items);
+    s->zchunk = tile_zc;
+  }
+  const int rc0 = plan_items(s->plan, items);
+  if (rc0 != LBPF_OK) {
+    if (rc0 == LBPF_ECUDA) s->sticky = rc0;
+    return rc0;
+  }
   if (s->gexec) cudaGraphExecDestroy(s->gexec);
   s->gexec = nullptr;
   s->graph_ok = false;
   if (s->ol.on) {
-    const int rc = setup_one_launch(s->ol, items, {TileGeom{s->kg.nx, s->kg.ny, s->kg.nz, s->zchunk}}, by,
+    s->zchunk = tile_zc;
+    items.clear();
+    build_items(0, k.nx, k.ny, k.nz, by, tile_zc, items);
+    const int rc = setup_one_launch(s->ol, items, {TileGeom{k.nx, k.ny, k.nz, tile_zc}}, by,
                                     step_smem_bytes(t, s->lat.q_phi, s->lat.q_u, s->lat.q_theta, by),
                                     t.step_fn[q_index(s->lat.q_phi)][q_index(s->lat.q_u)][qt_index(s->lat.q_theta)],
                                     s->device);
     if (rc != LBPF_OK) return rc;
   }
-  return set_smem_attrs(s);
+  const int rc = set_smem_attrs(t, s->lat, s->device);
+  if (rc != LBPF_OK) s->sticky = rc;
+  return rc;
 }
 
-// One step: the two kernels, or the one-launch kernel when `ol` is selected.
-int launch_step(cudaStream_t st, StepLaunch fphi, StepLaunch futh, int nitems, int by, size_t smem_phi,
-                size_t smem_uth, const SimDev* dd, const WorkItem* items, int s6, const OneLaunch* ol) {
-  if (ol && ol->on) {
-    if (cudaMemsetAsync(ol->d_ctl, 0, ol->ctl_bytes, st) != cudaSuccess) return LBPF_ECUDA;
-    return ol->fn(dim3(ol->grid), dim3(32, by), ol->smem, st, dd, items, ol->sc, s6) == cudaSuccess ? LBPF_OK
-                                                                                                 : LBPF_ECUDA;
-  }
-  cudaError_t e = fphi(dim3(nitems), dim3(32, by), smem_phi, st, dd, items, s6);
-  if (e != cudaSuccess) return LBPF_ECUDA;
-  e = futh(dim3(nitems), dim3(32, by), smem_uth, st, dd, items, s6);
-  return e == cudaSuccess ? LBPF_OK : LBPF_ECUDA;
+// Kernels first .. last-1 of a step.
+int launch_kernels(cudaStream_t st, const StepPlan& p, int first, int last, int s6) {
+  for (int k = first; k < last; ++k)
+    if (p.fn[k](dim3(p.nitems), dim3(p.threads_x, p.threads_y), p.smem[k], st, p.dd, p.items, s6) != cudaSuccess)
+      return LBPF_ECUDA;
+  return LBPF_OK;
 }
 
-int capture_graph(cudaStream_t st, StepLaunch fphi, StepLaunch futh, int nitems, int by, size_t smem_phi,
-                  size_t smem_uth, const SimDev* dd, const WorkItem* items, const OneLaunch* ol,
-                  cudaGraphExec_t* out) {
+// One step: the plan's kernels, or the one-launch kernel when `ol` is selected.
+int launch_step(cudaStream_t st, const StepPlan& p, int by, int s6, const OneLaunch& ol) {
+  if (!ol.on) return launch_kernels(st, p, 0, p.n, s6);
+  if (cudaMemsetAsync(ol.d_ctl, 0, ol.ctl_bytes, st) != cudaSuccess) return LBPF_ECUDA;
+  return ol.fn(dim3(ol.grid), dim3(32, by), ol.smem, st, p.dd, ol.d_items, ol.sc, s6) == cudaSuccess ? LBPF_OK
+                                                                                                    : LBPF_ECUDA;
+}
+
+int capture_graph(cudaStream_t st, const StepPlan& p, int by, const OneLaunch& ol, cudaGraphExec_t* out) {
   cudaGraph_t graph = nullptr;
   if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return LBPF_ECUDA;
   int rc = LBPF_OK;
-  for (int s6 = 0; s6 < kGraphSteps && rc == LBPF_OK; ++s6)
-    rc = launch_step(st, fphi, futh, nitems, by, smem_phi, smem_uth, dd, items, s6, ol);
+  for (int s6 = 0; s6 < kGraphSteps && rc == LBPF_OK; ++s6) rc = launch_step(st, p, by, s6, ol);
   cudaError_t e = cudaStreamEndCapture(st, &graph);
   if (rc != LBPF_OK || e != cudaSuccess) {
     if (graph) cudaGraphDestroy(graph);
@@ -403,33 +486,46 @@ void fill_dev(lbpf_sim* s) {
   for (int l = 0; l < 3; ++l) d.th[l] = s->th[l];
   const double e2p = lattice_e2(s->lat.q_phi), e2u = lattice_e2(s->lat.q_u);
   const double W2t = p.W0 * p.W0 / p.tau0;
-  d.inv2dx = 1.0 / (2.0 * p.dx);
-  d.c_eta = W2t * p.dt / (p.dx * p.dx) / e2p;
-  d.c_N = p.dt / p.dx * W2t / e2p;
-  d.dt_tau0 = p.dt / p.tau0;
-  d.lamM = p.lambda * p.Mc_inf;
-  d.lam = p.lambda;
-  d.eps1 = p.eps1; d.eps2 = p.eps2;
-  d.grad2_min = p.grad2_min > 0 ? p.grad2_min : 1e-12;
-  d.aniso = p.aniso;
   d.antitrapping = p.antitrapping ? 1 : 0;
-  d.k = p.k;
-  d.inv_etaU = 1.0 / (p.D * p.dt / (p.dx * p.dx) / e2u + 0.5);
-  d.c_J = p.dt / p.dx / e2u;
-  d.D_dx2 = p.D / (p.dx * p.dx);
-  d.D = p.D;
-  d.at_amp = p.W0 / (2.0 * sqrt(2.0));
-  d.dt = p.dt;
-  d.inv_dt = 1.0 / p.dt;
-  d.inv_etaT = s->lat.q_theta ? 1.0 / (p.kappa * p.dt / (p.dx * p.dx) / lattice_e2(s->lat.q_theta) + 0.5) : 0.0;
-  d.theta0 = s->theta0;
-  d.shift_h = s->U0;
-  d.shift_f = s->theta0;
+  Consts<double>& c = d.c64;
+  c.inv2dx = 1.0 / (2.0 * p.dx);
+  c.inv2dx2 = c.inv2dx * c.inv2dx;
+  c.c_eta = W2t * p.dt / (p.dx * p.dx) / e2p;
+  c.c_N = p.dt / p.dx * W2t / e2p;
+  c.dt_tau0 = p.dt / p.tau0;
+  c.lamM = p.lambda * p.Mc_inf;
+  c.lam = p.lambda;
+  if (p.aniso == 0) {  // 1 - 3 eps + 4 eps sum n^4
+    c.a0 = 1.0 - 3.0 * p.eps1;
+    c.a4 = 4.0 * p.eps1;
+    c.a6 = 0.0;
+  } else {  // 1 + eps1 (sum n^4 - 3/5) + eps2 (3 sum n^4 + 66 nx^2 ny^2 nz^2 - 17/7)
+    c.a0 = 1.0 - 0.6 * p.eps1 - 17.0 / 7.0 * p.eps2;
+    c.a4 = p.eps1 + 3.0 * p.eps2;
+    c.a6 = 66.0 * p.eps2;
+  }
+  c.grad2_min = p.grad2_min > 0 ? p.grad2_min : 1e-12;
+  c.k = p.k;
+  c.inv_etaU = 1.0 / (p.D * p.dt / (p.dx * p.dx) / e2u + 0.5);
+  c.c_J = p.dt / p.dx / e2u;
+  c.D_dx2 = p.D / (p.dx * p.dx);
+  c.D = p.D;
+  c.at_amp = p.W0 / (2.0 * sqrt(2.0));
+  c.dt = p.dt;
+  c.inv_dt = 1.0 / p.dt;
+  c.inv_etaT = s->lat.q_theta ? 1.0 / (p.kappa * p.dt / (p.dx * p.dx) / lattice_e2(s->lat.q_theta) + 0.5) : 0.0;
+  c.theta0 = s->theta0;
+  c.shift_h = s->U0;
+  c.shift_f = s->theta0;
   // codec scales: powers of two keeping the stored deviations well inside the FP16 range
   for (int f = 0; f < 3; ++f) {
-    d.scale[f] = s->kt->shifted ? 4096.0 : 1.0;
-    d.inv_scale[f] = 1.0 / d.scale[f];
+    c.scale[f] = s->kt->shifted ? 4096.0 : 1.0;
+    c.inv_scale[f] = 1.0 / c.scale[f];
   }
+  static_assert(sizeof(Consts<double>) == 2 * sizeof(Consts<float>), "Consts holds only values of its type");
+  const double* wide = reinterpret_cast<const double*>(&d.c64);
+  float* narrow = reinterpret_cast<float*>(&d.c32);
+  for (size_t i = 0; i < sizeof(Consts<double>) / sizeof(double); ++i) narrow[i] = (float)wide[i];
 }
 
 int upload_dev(lbpf_sim* s) {
@@ -448,7 +544,7 @@ void free_sim(lbpf_sim* s) {
   for (int l = 0; l < 3; ++l)
     if (s->th[l]) cudaFree(s->th[l]);
   if (s->dd) cudaFree(s->dd);
-  if (s->d_items) cudaFree(s->d_items);
+  if (s->plan.items) cudaFree(s->plan.items);
   if (s->d_part) cudaFree(s->d_part);
   if (s->d_small) cudaFree(s->d_small);
   if (s->h_small) cudaFreeHost(s->h_small);
@@ -604,8 +700,7 @@ int lbpf_step(lbpf_sim* s, int64_t n) {
       if (!s->graph_ok) {
         if (s->gexec) cudaGraphExecDestroy(s->gexec);
         s->gexec = nullptr;
-        if (capture_graph(s->stream, s->fphi, s->futh, s->nitems, s->by, s->smem_phi, s->smem_uth, s->dd,
-                          s->d_items, &s->ol, &s->gexec) != LBPF_OK) {
+        if (capture_graph(s->stream, s->plan, s->by, s->ol, &s->gexec) != LBPF_OK) {
           s->sticky = LBPF_ECUDA;
           return LBPF_ECUDA;
         }
@@ -615,8 +710,7 @@ int lbpf_step(lbpf_sim* s, int64_t n) {
       s->steps += kGraphSteps;
       n -= kGraphSteps;
     } else {
-      if (launch_step(s->stream, s->fphi, s->futh, s->nitems, s->by, s->smem_phi, s->smem_uth, s->dd, s->d_items,
-                      s6_of(s), &s->ol) != LBPF_OK) {
+      if (launch_step(s->stream, s->plan, s->by, s6_of(s), s->ol) != LBPF_OK) {
         s->sticky = LBPF_ECUDA;
         return LBPF_ECUDA;
       }
@@ -635,18 +729,14 @@ int lbpf_step_timed(lbpf_sim* s, int64_t n, double ms_kernels[3]) {
   CK(s, cudaEventRecord(ev[0], s->stream));
   for (int64_t k = 0; k < n; ++k) {
     const int s6 = s6_of(s);
-    if (s->ol.on) {
-      // one launch per step: all of its time is counted as the first phase's
-      if (launch_step(s->stream, s->fphi, s->futh, s->nitems, s->by, s->smem_phi, s->smem_uth, s->dd, s->d_items,
-                      s6, &s->ol) != LBPF_OK) {
-        s->sticky = LBPF_ECUDA;
-        return LBPF_ECUDA;
-      }
-      CK(s, cudaEventRecord(ev[2 * k + 1], s->stream));
-    } else {
-      CK(s, s->fphi(dim3(s->nitems), dim3(32, s->by), s->smem_phi, s->stream, s->dd, s->d_items, s6));
-      CK(s, cudaEventRecord(ev[2 * k + 1], s->stream));
-      CK(s, s->futh(dim3(s->nitems), dim3(32, s->by), s->smem_uth, s->stream, s->dd, s->d_items, s6));
+    // one launch per step: all of its time is counted as the first phase's
+    int rc = s->ol.on ? launch_step(s->stream, s->plan, s->by, s6, s->ol)
+                      : launch_kernels(s->stream, s->plan, 0, s->plan.nphi, s6);
+    CK(s, cudaEventRecord(ev[2 * k + 1], s->stream));
+    if (rc == LBPF_OK && !s->ol.on) rc = launch_kernels(s->stream, s->plan, s->plan.nphi, s->plan.n, s6);
+    if (rc != LBPF_OK) {
+      s->sticky = LBPF_ECUDA;
+      return LBPF_ECUDA;
     }
     CK(s, cudaEventRecord(ev[2 * k + 2], s->stream));
     s->steps += 1;
@@ -861,7 +951,7 @@ int lbpf_set_tiling(lbpf_sim* s, int32_t by, int32_t zchunk) {
   if (!s || by < 0 || zchunk < 0 || (by && (by < 4 || by > MAX_BLOCK_ROWS))) return LBPF_EINVAL;
   if (status(s)) return s->sticky;
   CK(s, cudaStreamSynchronize(s->stream));
-  return apply_tiling(s, by ? by : s->by, zchunk ? zchunk : (by ? 0 : s->zchunk));
+  return apply_tiling(s, by ? by : s->by, zchunk ? zchunk : (by ? 0 : s->zreq));
 }
 
 int lbpf_get_tiling(const lbpf_sim* s, int32_t* by, int32_t* zchunk) {
@@ -878,11 +968,12 @@ int lbpf_set_schedule(lbpf_sim* s, int32_t schedule) {
   CK(s, cudaStreamSynchronize(s->stream));
   const bool was = s->ol.on;
   s->ol.on = schedule == LBPF_SCHED_ONE_LAUNCH;
-  const int rc = apply_tiling(s, s->by, s->zchunk);
+  const int zreq = s->zreq;
+  const int rc = apply_tiling(s, s->by, zreq);
   if (rc != LBPF_OK) {
     s->ol.on = was;
     free_one_launch(s->ol);
-    apply_tiling(s, s->by, s->zchunk);
+    apply_tiling(s, s->by, zreq);
   }
   if (!s->ol.on) free_one_launch(s->ol);
   return rc;
@@ -1003,8 +1094,12 @@ int lbpf_autotune(lbpf_sim* s, int32_t steps, double* best_ms) {
   const int bys[] = {4, 6, 8};
   for (int by : bys) {
     if (by > s->kg.ny + 2 && by != bys[0]) continue;
-    const int zdef = default_zchunk(s->kg.nx, s->kg.ny, s->kg.nz, by);
-    const int zcs[] = {zdef, std::max(8, zdef / 2), std::min(s->kg.nz, zdef * 2), s->kg.nz};
+    const lbpf_grid& k = s->kg;
+    const bool node = s->plan.node_wise && !s->ol.on;
+    const int zdef = node ? node_zchunk(node_blocks(k.nx, k.ny, k.nz, node_threads(s->by == 1 ? 1 : by)), k.nz)
+                          : default_zchunk(k.nx, k.ny, k.nz, by);
+    const int zcs[] = {zdef, std::max(node ? 1 : 8, zdef / 2), std::min(k.nz, zdef * 2),
+                       node ? std::min(k.nz, zdef * 4) : k.nz};
     for (int zc : zcs) {
       if (apply_tiling(s, by, zc) != LBPF_OK) { s->sticky = LBPF_OK; continue; }
       int rc = lbpf_step(s, 1);  // warm-up
@@ -1117,40 +1212,35 @@ int lbpf_load(lbpf_sim* s, const char* path) {
 // `zchunk` planes (0: each simulation's default), large chunks first.
 static int batch_tiling(lbpf_batch* b, int by, int zchunk) {
   const KernelTable& t = *b->sims[0]->kt;
-  std::vector<WorkItem> items;
+  const lbpf_lattice& l = b->sims[0]->lat;
+  std::vector<WorkItem> items, node_items;
   std::vector<TileGeom> geo;
+  long long sites = 0;
+  for (const lbpf_sim* s : b->sims) sites += s->nsite;
+  plan_kernels(b->plan, t, l, by, steps_node_wise(t, l, sites));
+  b->plan.dd = b->dd;
+  long long blocks = 0;  // of one plane each, over all members
+  for (const lbpf_sim* s : b->sims) blocks += node_blocks(s->kg.nx, s->kg.ny, s->kg.nz, b->plan.threads_x);
   for (size_t i = 0; i < b->sims.size(); ++i) {
-    const lbpf_sim* s = b->sims[i];
-    const int zc = zchunk > 0 ? std::min(zchunk, s->kg.nz) : default_zchunk(s->kg.nx, s->kg.ny, s->kg.nz, by);
-    build_items((int)i, s->kg.nx, s->kg.ny, s->kg.nz, by, zc, items);
-    geo.push_back(TileGeom{s->kg.nx, s->kg.ny, s->kg.nz, zc});
+    const lbpf_grid& k = b->sims[i]->kg;
+    const int zc = zchunk > 0 ? std::min(zchunk, k.nz) : default_zchunk(k.nx, k.ny, k.nz, by);
+    build_items((int)i, k.nx, k.ny, k.nz, by, zc, items);
+    geo.push_back(TileGeom{k.nx, k.ny, k.nz, zc});
+    if (b->plan.node_wise)
+      build_node_items((int)i, k.nx, k.ny, k.nz, b->plan.threads_x, zchunk > 0 ? zc : node_zchunk(blocks, k.nz),
+                       node_items);
   }
   // interleave large and small simulations: sort items by descending z-chunk work
-  std::stable_sort(items.begin(), items.end(),
-                   [](const WorkItem& a, const WorkItem& c) { return (a.z1 - a.z0) > (c.z1 - c.z0); });
-  if (b->d_items) cudaFree(b->d_items);
-  b->d_items = nullptr;
-  if (cudaMalloc(&b->d_items, items.size() * sizeof(WorkItem)) != cudaSuccess ||
-      cudaMemcpy(b->d_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice) != cudaSuccess) {
-    cudaGetLastError();
-    return LBPF_ENOMEM;
-  }
-  b->nitems = (int)items.size();
+  for (std::vector<WorkItem>* v : {&items, &node_items})
+    std::stable_sort(v->begin(), v->end(),
+                     [](const WorkItem& a, const WorkItem& c) { return (a.z1 - a.z0) > (c.z1 - c.z0); });
+  if (plan_items(b->plan, b->plan.node_wise ? node_items : items) != LBPF_OK) return LBPF_ENOMEM;
   b->by = by;
   b->zchunk = zchunk;
-  {
-    const lbpf_lattice& l = b->sims[0]->lat;
-    const int v = block_variant(l.q_phi, by);
-    b->fphi = t.phi[q_index(l.q_phi)][v];
-    b->futh = t.uth[q_index(l.q_u)][qt_index(l.q_theta)][v];
-  }
-  b->smem_phi = phi_smem_bytes(t, b->sims[0]->lat.q_phi, by);
-  b->smem_uth = uth_smem_bytes(t, b->sims[0]->lat.q_u, b->sims[0]->lat.q_theta, by);
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
   b->gexec = nullptr;
   b->graph_ok = false;
   if (b->ol.on) {
-    const lbpf_lattice& l = b->sims[0]->lat;
     const int rc = setup_one_launch(b->ol, items, geo, by, step_smem_bytes(t, l.q_phi, l.q_u, l.q_theta, by),
                                     t.step_fn[q_index(l.q_phi)][q_index(l.q_u)][qt_index(l.q_theta)],
                                     b->sims[0]->device);
@@ -1179,17 +1269,13 @@ int batch_init(lbpf_batch* b) {
   if (ok) {
     for (size_t i = 0; i < n; ++i) {
       fill_dev(b->sims[i]);
-      b->h_desc[i] = b->sims[i]->hd;
+      memcpy(&b->h_desc[i], &b->sims[i]->hd, sizeof(SimDev));
     }
   }
   ok = ok && cudaMemcpy(b->dd, b->h_desc, n * sizeof(SimDev), cudaMemcpyHostToDevice) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) == cudaSuccess;
   ok = ok && batch_tiling(b, lattice_is_2d(s0->lat.q_phi) ? 1 : MAX_BLOCK_ROWS, 0) == LBPF_OK;
-  const int a = q_index(s0->lat.q_phi), qb = q_index(s0->lat.q_u), qc = qt_index(s0->lat.q_theta);
-  for (int v = 0; v < 2; ++v) {
-    ok = ok && raise_smem_limit(t.phi_fn[a][v], s0->device) == LBPF_OK;
-    ok = ok && raise_smem_limit(t.uth_fn[qb][qc][v], s0->device) == LBPF_OK;
-  }
+  ok = ok && set_smem_attrs(t, s0->lat, s0->device) == LBPF_OK;
   if (!ok) {
     cudaGetLastError();
     return LBPF_ENOMEM;
@@ -1208,7 +1294,7 @@ int batch_refresh(lbpf_batch* b) {
   if (!changed) return LBPF_OK;
   // the pinned buffer may still feed an earlier upload: let the stream drain first
   if (cudaStreamSynchronize(b->stream) != cudaSuccess) return LBPF_ECUDA;
-  for (size_t i = 0; i < b->sims.size(); ++i) b->h_desc[i] = b->sims[i]->hd;
+  for (size_t i = 0; i < b->sims.size(); ++i) memcpy(&b->h_desc[i], &b->sims[i]->hd, sizeof(SimDev));
   if (cudaMemcpyAsync(b->dd, b->h_desc, b->sims.size() * sizeof(SimDev), cudaMemcpyHostToDevice, b->stream) !=
       cudaSuccess)
     return LBPF_ECUDA;
@@ -1292,8 +1378,7 @@ int lbpf_batch_step(lbpf_batch* b, int64_t n) {
     const int s6 = (int)(steps % kGraphSteps);
     if (s6 == 0 && n >= kGraphSteps) {
       if (!b->graph_ok) {
-        if (capture_graph(b->stream, b->fphi, b->futh, b->nitems, b->by, b->smem_phi, b->smem_uth, b->dd, b->d_items,
-                          &b->ol, &b->gexec) != LBPF_OK)
+        if (capture_graph(b->stream, b->plan, b->by, b->ol, &b->gexec) != LBPF_OK)
           return LBPF_ECUDA;
         b->graph_ok = true;
       }
@@ -1301,9 +1386,7 @@ int lbpf_batch_step(lbpf_batch* b, int64_t n) {
       steps += kGraphSteps;
       n -= kGraphSteps;
     } else {
-      if (launch_step(b->stream, b->fphi, b->futh, b->nitems, b->by, b->smem_phi, b->smem_uth, b->dd, b->d_items, s6,
-                      &b->ol) !=
-          LBPF_OK)
+      if (launch_step(b->stream, b->plan, b->by, s6, b->ol) != LBPF_OK)
         return LBPF_ECUDA;
       steps += 1;
       n -= 1;
@@ -1427,7 +1510,7 @@ int lbpf_batch_destroy(lbpf_batch* b) {
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
   if (b->dd) cudaFree(b->dd);
   if (b->h_desc) cudaFreeHost(b->h_desc);
-  if (b->d_items) cudaFree(b->d_items);
+  if (b->plan.items) cudaFree(b->plan.items);
   if (b->ev) cudaEventDestroy(b->ev);
   // borrowed members outlive the batch: they keep a failure the batch saw, not its flag
   for (lbpf_sim* s : b->sims)

@@ -79,7 +79,7 @@ __global__ void k_init_pop(SimDev sd, LatRT Lp, LatRT Lu, LatRT Lt, const typena
   T* phi = (T*)sd.phi[0];
   T* U = (T*)sd.U[0];
   T* th = (T*)sd.th[0];
-  const T k = (T)sd.k;
+  const T k = consts_of<T>(sd).k;
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
     const int x = (int)(s % nx);
     const int y = (int)((s / nx) % ny);
@@ -90,7 +90,7 @@ __global__ void k_init_pop(SimDev sd, LatRT Lp, LatRT Lu, LatRT Lt, const typena
       const int a = x + Lp.e[i][0], b = y + Lp.e[i][1], c = z + Lp.e[i][2];
       const T pn = in_dom(a, b, c, nx, ny, nz) ? phi0[((long long)c * ny + b) * nx + a] : px;
       const T wi = (T)Lp.w[i];
-      g[(long long)i * n + s] = C::enc(wi * pn, wi * px, (T)sd.scale[0]);
+      g[(long long)i * n + s] = C::enc(wi * pn, wi * px, consts_of<T>(sd).scale[0]);
       mphi += wi * px;
     }
     for (int i = 0; i < Lu.q; ++i) {
@@ -99,12 +99,12 @@ __global__ void k_init_pop(SimDev sd, LatRT Lp, LatRT Lu, LatRT Lt, const typena
       const T Ai = i == 0 ? T(1) : T(0);
       const T qz = T(0.5) * (T(1) - pn) / (T(0.5) * ((T(1) + k) - (T(1) - k) * pn));
       const T qzx = T(0.5) * (T(1) - px) / (T(0.5) * ((T(1) + k) - (T(1) - k) * px));
-      h[(long long)i * n + s] = C::enc((Ai + (T)Lu.B[i] * qz) * (T)U0, (T)Lu.w[i] * (T)sd.shift_h, (T)sd.scale[1]);
+      h[(long long)i * n + s] = C::enc((Ai + (T)Lu.B[i] * qz) * (T)U0, (T)Lu.w[i] * consts_of<T>(sd).shift_h, consts_of<T>(sd).scale[1]);
       mU += (Ai + (T)Lu.B[i] * qzx) * (T)U0;
     }
     for (int i = 0; i < Lt.q; ++i) {
       const T wi = (T)Lt.w[i];
-      f[(long long)i * n + s] = C::enc(wi * (T)theta0, wi * (T)sd.shift_f, (T)sd.scale[2]);
+      f[(long long)i * n + s] = C::enc(wi * (T)theta0, wi * consts_of<T>(sd).shift_f, consts_of<T>(sd).scale[2]);
       mth += wi * (T)theta0;
     }
     phi[s] = mphi;
@@ -144,8 +144,8 @@ __global__ void k_pack(SimDev sd, int field, int par, LatRT L, int i, const doub
   S* A = (S*)sd.pop[par][field];
   const int j = L.opp[i];
   const T wi = (T)L.w[i];
-  const T cshift = field == 1 ? (T)sd.shift_h : (T)sd.shift_f;
-  const T scale = (T)sd.scale[field];
+  const T cshift = field == 1 ? consts_of<T>(sd).shift_h : consts_of<T>(sd).shift_f;
+  const T scale = consts_of<T>(sd).scale[field];
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
     const int x = (int)(s % nx);
     const int y = (int)((s / nx) % ny);
@@ -175,8 +175,8 @@ __global__ void k_unpack(SimDev sd, int field, int par, LatRT L, int i, double* 
   const S* A = (const S*)sd.pop[par][field];
   const int j = L.opp[i];
   const T wi = (T)L.w[i];
-  const T cshift = field == 1 ? (T)sd.shift_h : (T)sd.shift_f;
-  const T isc = (T)sd.inv_scale[field];
+  const T cshift = field == 1 ? consts_of<T>(sd).shift_h : consts_of<T>(sd).shift_f;
+  const T isc = consts_of<T>(sd).inv_scale[field];
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
     const int x = (int)(s % nx);
     const int y = (int)((s / nx) % ny);

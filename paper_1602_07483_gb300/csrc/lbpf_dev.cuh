@@ -1,6 +1,7 @@
 // lbpf_dev.cuh -- device code of the lattice-Boltzmann phase-field step for sm_103a.
 //
-// One time step (Sec. 3.4, "Algorithm implementation") on D3Q7/D3Q15/D3Q19, or on
+// The tiled step: the distributions are read once, at the price of halo collisions
+// (lbpf_nodewise.cuh is the form without a halo).  One time step (Sec. 3.4, "Algorithm implementation") on D3Q7/D3Q15/D3Q19, or on
 // D2Q5/D2Q9 over an nz = 1 grid, is two kernels:
 //   k_phi : phi collision (Eq. collision stage, non-local term) + streaming with
 //           bounce-back, using phi^n, U^n, theta^n; writes the post-collision
@@ -27,306 +28,10 @@
 // per node and the distributions are read once and written once.
 #pragma once
 
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-#include <cuda_runtime.h>
-#include <stdint.h>
-
-#include <type_traits>
-
+#include "lbpf_node.cuh"
 #include "lbpf_plan.h"
 
 namespace lbpf {
-
-// ---------------------------------------------------------------- lattices
-// Table 1 (e_i) and Table 2 (w_i, A_i, B_i, e^2) of Sec. 3.4.
-template <int Q>
-struct Lat;
-
-template <>
-struct Lat<7> {
-  static constexpr double e2 = 0.25;
-  static constexpr bool has_y = true;  // links along the kernel's y axis (false: a 2D lattice in the xz plane)
-  static constexpr int diag0 = 1;      // first index of the diagonal weight class (none: an axis index)
-  __host__ __device__ static constexpr int cls(int i) { return i == 0 ? 0 : 1; }  // 0 rest, 1 axis, 2 diagonal
-  __host__ __device__ static constexpr int ex(int i) { return i == 1 ? 1 : (i == 3 ? -1 : 0); }
-  __host__ __device__ static constexpr int ey(int i) { return i == 2 ? 1 : (i == 4 ? -1 : 0); }
-  __host__ __device__ static constexpr int ez(int i) { return i == 5 ? 1 : (i == 6 ? -1 : 0); }
-  __host__ __device__ static constexpr int opp(int i) {
-    return i == 0 ? 0 : (i == 1 ? 3 : (i == 2 ? 4 : (i == 3 ? 1 : (i == 4 ? 2 : (i == 5 ? 6 : 5)))));
-  }
-  __host__ __device__ static constexpr double w(int i) { return i == 0 ? 0.25 : 0.125; }
-  __host__ __device__ static constexpr double B(int i) { return i == 0 ? -0.75 : 0.125; }
-};
-
-// The accessors are switch expressions so that, with the population loops
-// unrolled, every lookup folds to an immediate.
-template <>
-struct Lat<15> {
-  static constexpr double e2 = 1.0 / 3.0;
-  static constexpr bool has_y = true;
-  static constexpr int diag0 = 7;
-  __host__ __device__ static constexpr int cls(int i) { return i == 0 ? 0 : (i <= 6 ? 1 : 2); }
-  // e_0..e_6 as D3Q7, then the cube diagonals
-  __host__ __device__ static constexpr int ex(int i) {
-    switch (i) {
-      case 1: case 7: case 10: case 11: case 14: return 1;
-      case 3: case 8: case 9: case 12: case 13: return -1;
-      default: return 0;
-    }
-  }
-  __host__ __device__ static constexpr int ey(int i) {
-    switch (i) {
-      case 2: case 7: case 8: case 11: case 12: return 1;
-      case 4: case 9: case 10: case 13: case 14: return -1;
-      default: return 0;
-    }
-  }
-  __host__ __device__ static constexpr int ez(int i) {
-    switch (i) {
-      case 5: case 7: case 8: case 9: case 10: return 1;
-      case 6: case 11: case 12: case 13: case 14: return -1;
-      default: return 0;
-    }
-  }
-  __host__ __device__ static constexpr int opp(int i) {
-    switch (i) {
-      case 1: return 3; case 2: return 4; case 3: return 1; case 4: return 2; case 5: return 6; case 6: return 5;
-      case 7: return 13; case 8: return 14; case 9: return 11; case 10: return 12;
-      case 11: return 9; case 12: return 10; case 13: return 7; case 14: return 8;
-      default: return 0;
-    }
-  }
-  __host__ __device__ static constexpr double w(int i) {
-    return i == 0 ? 2.0 / 9.0 : (i <= 6 ? 1.0 / 9.0 : 1.0 / 72.0);
-  }
-  __host__ __device__ static constexpr double B(int i) {
-    return i == 0 ? -7.0 / 9.0 : (i <= 6 ? 1.0 / 9.0 : 1.0 / 72.0);
-  }
-};
-
-template <>
-struct Lat<19> {
-  static constexpr double e2 = 1.0 / 3.0;
-  static constexpr bool has_y = true;
-  static constexpr int diag0 = 7;
-  __host__ __device__ static constexpr int cls(int i) { return i == 0 ? 0 : (i <= 6 ? 1 : 2); }
-  // e_0..e_6 as D3Q7, then the twelve edge diagonals
-  __host__ __device__ static constexpr int ex(int i) {
-    switch (i) {
-      case 1: case 7: case 9: case 11: case 13: return 1;
-      case 3: case 8: case 10: case 12: case 14: return -1;
-      default: return 0;
-    }
-  }
-  __host__ __device__ static constexpr int ey(int i) {
-    switch (i) {
-      case 2: case 7: case 8: case 15: case 17: return 1;
-      case 4: case 9: case 10: case 16: case 18: return -1;
-      default: return 0;
-    }
-  }
-  __host__ __device__ static constexpr int ez(int i) {
-    switch (i) {
-      case 5: case 11: case 12: case 15: case 16: return 1;
-      case 6: case 13: case 14: case 17: case 18: return -1;
-      default: return 0;
-    }
-  }
-  __host__ __device__ static constexpr int opp(int i) {
-    switch (i) {
-      case 1: return 3; case 2: return 4; case 3: return 1; case 4: return 2; case 5: return 6; case 6: return 5;
-      case 7: return 10; case 8: return 9; case 9: return 8; case 10: return 7;
-      case 11: return 14; case 12: return 13; case 13: return 12; case 14: return 11;
-      case 15: return 18; case 16: return 17; case 17: return 16; case 18: return 15;
-      default: return 0;
-    }
-  }
-  __host__ __device__ static constexpr double w(int i) {
-    return i == 0 ? 1.0 / 3.0 : (i <= 6 ? 1.0 / 18.0 : 1.0 / 36.0);
-  }
-  __host__ __device__ static constexpr double B(int i) {
-    return i == 0 ? -2.0 / 3.0 : (i <= 6 ? 1.0 / 18.0 : 1.0 / 36.0);
-  }
-};
-// Table 3 (e_i) and Table 4 (w_i, A_i, B_i, e^2) of Sec. 3.4: the 2D lattices.  A 2D
-// grid (nx, ny) runs as a kernel grid (nx, 1, ny): the paper's y axis becomes the
-// kernel's marching axis z, so ey() below is always 0 and ez() holds the paper's e_y.
-// Population order and memory layout are unchanged (one kernel plane row per paper row).
-template <>
-struct Lat<5> {
-  static constexpr double e2 = 1.0 / 3.0;
-  static constexpr bool has_y = false;
-  static constexpr int diag0 = 1;
-  __host__ __device__ static constexpr int cls(int i) { return i == 0 ? 0 : 1; }
-  __host__ __device__ static constexpr int ex(int i) { return i == 1 ? 1 : (i == 3 ? -1 : 0); }
-  __host__ __device__ static constexpr int ey(int) { return 0; }
-  __host__ __device__ static constexpr int ez(int i) { return i == 2 ? 1 : (i == 4 ? -1 : 0); }
-  __host__ __device__ static constexpr int opp(int i) { return i == 0 ? 0 : (i <= 2 ? i + 2 : i - 2); }
-  __host__ __device__ static constexpr double w(int i) { return i == 0 ? 1.0 / 3.0 : 1.0 / 6.0; }
-  __host__ __device__ static constexpr double B(int i) { return i == 0 ? -2.0 / 3.0 : 1.0 / 6.0; }
-};
-
-template <>
-struct Lat<9> {
-  static constexpr double e2 = 1.0 / 3.0;
-  static constexpr bool has_y = false;
-  static constexpr int diag0 = 5;
-  __host__ __device__ static constexpr int cls(int i) { return i == 0 ? 0 : (i <= 4 ? 1 : 2); }
-  // paper's e_0..e_4 as D2Q5, then (1,1), (-1,1), (-1,-1), (1,-1); second component in ez()
-  __host__ __device__ static constexpr int ex(int i) {
-    switch (i) {
-      case 1: case 5: case 8: return 1;
-      case 3: case 6: case 7: return -1;
-      default: return 0;
-    }
-  }
-  __host__ __device__ static constexpr int ey(int) { return 0; }
-  __host__ __device__ static constexpr int ez(int i) {
-    switch (i) {
-      case 2: case 5: case 6: return 1;
-      case 4: case 7: case 8: return -1;
-      default: return 0;
-    }
-  }
-  __host__ __device__ static constexpr int opp(int i) {
-    switch (i) {
-      case 1: return 3; case 2: return 4; case 3: return 1; case 4: return 2;
-      case 5: return 7; case 6: return 8; case 7: return 5; case 8: return 6;
-      default: return 0;
-    }
-  }
-  __host__ __device__ static constexpr double w(int i) {
-    return i == 0 ? 4.0 / 9.0 : (i <= 4 ? 1.0 / 9.0 : 1.0 / 36.0);
-  }
-  __host__ __device__ static constexpr double B(int i) {
-    return i == 0 ? -5.0 / 9.0 : (i <= 4 ? 1.0 / 9.0 : 1.0 / 36.0);
-  }
-};
-// A_i = 1 for the rest population and 0 otherwise on all five lattices.
-
-// Populations with e_y != 0 cross block rows during the moment gather and go
-// through shared memory; yslot(i) numbers them 0..NY-1 (-1 for e_y = 0).
-template <int Q>
-struct YSlots {
-  __host__ __device__ static constexpr int count() {
-    int c = 0;
-    for (int i = 0; i < Q; ++i) c += Lat<Q>::ey(i) != 0;
-    return c;
-  }
-  __host__ __device__ static constexpr int slot(int i) {
-    if (Lat<Q>::ey(i) == 0) return -1;
-    int c = 0;
-    for (int j = 0; j < i; ++j) c += Lat<Q>::ey(j) != 0;
-    return c;
-  }
-};
-template <int Q>
-struct NYOf {
-  static constexpr int value = YSlots<Q>::count();
-};
-template <>
-struct NYOf<0> {
-  static constexpr int value = 0;
-};
-
-// ---------------------------------------------------------------- storage codec
-// FP64/FP32: stored as is.  FP16/BF16: stored = (f - shift) * scale, decoded to
-// FP32; `shift` removes the bulk value so the stored number is the small part.
-template <typename S>
-struct Codec;
-// raw(s) / pack(v): the stored number itself as T and back (round to nearest), for
-// arithmetic done directly in the scaled units (f - shift) * scale.
-// dec64 / enc64: the same codec evaluated in FP64 for state import and export: with a
-// power-of-two scale, s / scale + shift is exact in FP64, so export then import returns
-// every stored number unchanged.
-template <>
-struct Codec<double> {
-  using T = double;
-  static constexpr bool shifted = false;
-  __device__ static __forceinline__ T dec(double s, T, T) { return s; }
-  __device__ static __forceinline__ double enc(T v, T, T) { return v; }
-  __device__ static __forceinline__ T raw(double s) { return s; }
-  __device__ static __forceinline__ double pack(T v) { return v; }
-  __device__ static __forceinline__ double dec64(double s, double, double) { return s; }
-  __device__ static __forceinline__ double enc64(double v, double, double) { return v; }
-};
-template <>
-struct Codec<float> {
-  using T = float;
-  static constexpr bool shifted = false;
-  __device__ static __forceinline__ T dec(float s, T, T) { return s; }
-  __device__ static __forceinline__ float enc(T v, T, T) { return v; }
-  __device__ static __forceinline__ T raw(float s) { return s; }
-  __device__ static __forceinline__ float pack(T v) { return v; }
-  __device__ static __forceinline__ double dec64(float s, double, double) { return (double)s; }
-  __device__ static __forceinline__ float enc64(double v, double, double) { return (float)v; }
-};
-template <>
-struct Codec<__half> {
-  using T = float;
-  static constexpr bool shifted = true;
-  __device__ static __forceinline__ T dec(__half s, T shift, T inv_scale) {
-    return fmaf(__half2float(s), inv_scale, shift);
-  }
-  __device__ static __forceinline__ __half enc(T v, T shift, T scale) { return __float2half_rn((v - shift) * scale); }
-  __device__ static __forceinline__ T raw(__half s) { return __half2float(s); }
-  __device__ static __forceinline__ __half pack(T v) { return __float2half_rn(v); }
-  __device__ static __forceinline__ double dec64(__half s, double shift, double inv_scale) {
-    return (double)__half2float(s) * inv_scale + shift;
-  }
-  __device__ static __forceinline__ __half enc64(double v, double shift, double scale) {
-    return __double2half((v - shift) * scale);
-  }
-};
-template <>
-struct Codec<__nv_bfloat16> {
-  using T = float;
-  static constexpr bool shifted = true;
-  __device__ static __forceinline__ T dec(__nv_bfloat16 s, T shift, T inv_scale) {
-    return fmaf(__bfloat162float(s), inv_scale, shift);
-  }
-  __device__ static __forceinline__ __nv_bfloat16 enc(T v, T shift, T scale) {
-    return __float2bfloat16_rn((v - shift) * scale);
-  }
-  __device__ static __forceinline__ T raw(__nv_bfloat16 s) { return __bfloat162float(s); }
-  __device__ static __forceinline__ __nv_bfloat16 pack(T v) { return __float2bfloat16_rn(v); }
-  __device__ static __forceinline__ double dec64(__nv_bfloat16 s, double shift, double inv_scale) {
-    return (double)__bfloat162float(s) * inv_scale + shift;
-  }
-  __device__ static __forceinline__ __nv_bfloat16 enc64(double v, double shift, double scale) {
-    return __double2bfloat16((v - shift) * scale);
-  }
-};
-
-// ---------------------------------------------------------------- descriptors
-// Per-simulation constants and buffers, resident in device memory.
-struct SimDev {
-  int nx, ny, nz, q_theta;
-  long long nsite;
-  void* pop[2][3];  // [buffer][g, h, f] in the storage type, [Q][z][y][x]
-  void* phi[3];     // phi levels (compute type); level s%3 is phi^n at step s
-  void* U[2];       // U^n at buffer s%2
-  void* th[3];      // theta levels (unused when q_theta == 0); level s%3 is theta^n at step s
-  double inv2dx;    // 1 / (2 dx)
-  double c_eta;     // e^-2 (W0^2/tau0) dt/dx^2: eta_phi = c_eta a_s^2 + 1/2 (Eq. LBE_RelaxationTime)
-  double c_N;       // e^-2 (dt/dx) W0^2/tau0: the N term of g^(0) (Eq. Feq_Phase)
-  double dt_tau0;   // dt / tau0
-  double lamM, lam; // lambda Mc_inf, lambda (Eq. LBE_SourceTerm)
-  double eps1, eps2, grad2_min;
-  int aniso, antitrapping;
-  double k;
-  double inv_etaU;  // 1 / eta_U (Eq. RelaxationTime_Concentration)
-  double c_J;       // e^-2 dt/dx of the U lattice (Eq. Feq_Transport)
-  double D_dx2;     // D / dx^2
-  double D;
-  double at_amp;    // W0 / (2 sqrt2), Eq. (AntiTrapping_Current)
-  double dt, inv_dt;
-  double inv_etaT;  // 1 / eta_theta (Eq. ThermalDiffusivity)
-  double theta0;
-  double shift_h, shift_f;       // FP16/BF16 codec: h shifted by w_i U0; f initially by w_i theta0
-  double scale[3], inv_scale[3]; // FP16/BF16 codec scales of g, h, f
-};
 
 #ifndef LBPF_MAX_BLOCK_ROWS
 #define LBPF_MAX_BLOCK_ROWS 8
@@ -345,74 +50,14 @@ constexpr int MAX_BLOCK_ROWS = LBPF_MAX_BLOCK_ROWS;  // blocks of at most 32 x 8
 // The 2D lattices run one-warp blocks; their launch bounds (counted in 256-thread
 // blocks) set the register budget that decides how many warps an SM holds.  Measured
 // on 8192^2 FP32: 64 registers (four 256-thread blocks) for both kernels, 21.2 -> 26.4
-// GLUPS.  FP64 has budgets of its own (at 64 registers it spills).
+// GLUPS.
 #ifndef LBPF_PHI2D_MIN_BLOCKS
 #define LBPF_PHI2D_MIN_BLOCKS 4
 #endif
 #ifndef LBPF_UTH2D_MIN_BLOCKS
 #define LBPF_UTH2D_MIN_BLOCKS 4
 #endif
-// FP64 storage and arithmetic (values take two registers)
-#ifndef LBPF_PHI64_MIN_BLOCKS
-#define LBPF_PHI64_MIN_BLOCKS 3
-#endif
-#ifndef LBPF_UTH64_MIN_BLOCKS
-#define LBPF_UTH64_MIN_BLOCKS 2
-#endif
-
-// ---------------------------------------------------------------- anisotropy
-// a_s(n) and N = |grad phi|^2 a_s d a_s / d(grad phi) (Eq. TermesAnisotropes),
-// written with n = grad phi / |grad phi| so that FP32 stays in range for small
-// gradients.  kind 0: Eq. (Anisotropic-Function_As), derivatives of
-// Eq. (Derivees_As); kind 1: Eq. (As_K41-K61) with its analytic derivatives.
-template <typename T>
-__device__ __forceinline__ T aniso_N(int kind, T e1, T e2, T gx, T gy, T gz, T G2, T& Nx, T& Ny, T& Nz) {
-  const T iG = (sizeof(T) == 8) ? T(1) / sqrt(G2) : (T)rsqrtf((float)G2);
-  const T nx = gx * iG, ny = gy * iG, nz = gz * iG;
-  const T x2 = nx * nx, y2 = ny * ny, z2 = nz * nz;
-  const T s4 = x2 * x2 + y2 * y2 + z2 * z2;
-  T as, dx, dy, dz;  // dx = G * d a_s / d(d_x phi)
-  if (kind == 0) {
-    as = T(1) - T(3) * e1 + T(4) * e1 * s4;
-    const T c = T(16) * e1;
-    dx = c * nx * (x2 - s4);
-    dy = c * ny * (y2 - s4);
-    dz = c * nz * (z2 - s4);
-  } else {
-    const T p3 = x2 * y2 * z2;
-    as = T(1) + e1 * (s4 - T(0.6)) + e2 * (T(3) * s4 + T(66) * p3 - T(17.0 / 7.0));
-    const T cs = T(4) * (e1 + T(3) * e2);
-    const T cp = T(132) * e2;
-    dx = cs * nx * (x2 - s4) + cp * nx * y2 * z2 * (T(1) - T(3) * x2);
-    dy = cs * ny * (y2 - s4) + cp * ny * x2 * z2 * (T(1) - T(3) * y2);
-    dz = cs * nz * (z2 - s4) + cp * nz * x2 * y2 * (T(1) - T(3) * z2);
-  }
-  const T G = G2 * iG;
-  const T f = G * as;  // |grad phi|^2 a_s / |grad phi|
-  Nx = f * dx;
-  Ny = f * dy;
-  Nz = f * dz;
-  return as;
-}
-
-// Read-only (non-coherent) load: the distributions read by a step kernel are
-// never written by the same launch.
-template <typename S>
-__device__ __forceinline__ S ldro(const S* p) { return __ldg(p); }
-
-__device__ __forceinline__ int slot4(int z) { return (z + 4) & 3; }  // z >= -1
-
-// Products and sums that are never fused into an FMA: the collision loops are
-// instantiated per row kind, and these keep the rounding identical in every
-// instantiation (a node recomputed as a halo equals its owner's value bit for bit).
-__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
-
-// 1/x: IEEE division in FP64, the hardware approximate reciprocal in FP32
-__device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
+inline __device__ int slot4(int z) { return (z + 4) & 3; }  // z >= -1
 
 // Scalar-field ring: four planes of (BY + 2) x 34 values around the block
 // region (mirror ghosts by clamping).  Each thread owns up to RPT elements of a
@@ -494,10 +139,8 @@ __device__ __forceinline__ void phi_tile(const SimDev* __restrict__ sims, const 
   T* ringm = ring + 4 * RS;                  // phi^{n-1} [4][BY+2][34] (codec shift only)
   T* sG = ring + (C::shifted ? 8 : 4) * RS;  // [2][NY][BY][32]
 
-  const T inv2dx = (T)sd.inv2dx, c_eta = (T)sd.c_eta, c_N = (T)sd.c_N, dt_tau0 = (T)sd.dt_tau0;
-  const T lamM = (T)sd.lamM, lam = (T)sd.lam, e1 = (T)sd.eps1, e2 = (T)sd.eps2, g2min = (T)sd.grad2_min;
-  const T theta0 = (T)sd.theta0, scale = (T)sd.scale[0], iscale = (T)sd.inv_scale[0];
-  const int kind = sd.aniso;
+  const Consts<T> P = consts_of<T>(sd);
+  const T theta0 = P.theta0, scale = P.scale[0], iscale = P.inv_scale[0];
 
   const int zlo = max(it.z0 - 1, 0), zhi = min(it.z1, nz - 1);
   RingMap rm;
@@ -559,7 +202,7 @@ __device__ __forceinline__ void phi_tile(const SimDev* __restrict__ sims, const 
             const unsigned off = (unsigned)(ez * (int)plane + ey * nx + ex);
             gpull[i] = C::raw(ldro(gin + (own - off)));
             if (C::shifted)  // stored units with the source's shift: Gp + S w phi_ref(src)
-              gpull[i] = fma(rmul(scale, (T)L::w(i)), (ringm + slot4(zc - ez) * RS)[rc - ey * RW - ex], gpull[i]);
+              gpull[i] = rfma(rmul(scale, (T)L::w(i)), (ringm + slot4(zc - ez) * RS)[rc - ey * RW - ex], gpull[i]);
             gnl[i] = C::raw(ldro(gin + own));
           }
         } else {
@@ -574,69 +217,26 @@ __device__ __forceinline__ void phi_tile(const SimDev* __restrict__ sims, const 
             const int ii = inside ? i : L::opp(i);
             gpull[i] = C::raw(ldro(gin + ((unsigned)ii * NS + src)));
             if (C::shifted)
-              gpull[i] = fma(rmul(scale, (T)L::w(i)), (ringm + slot4(inside ? sz : zc) * RS)[inside ? rc - ey * RW - ex : rc],
+              gpull[i] = rfma(rmul(scale, (T)L::w(i)), (ringm + slot4(inside ? sz : zc) * RS)[inside ? rc - ey * RW - ex : rc],
                              gpull[i]);
             gnl[i] = T(0);
           }
         }
         const T ph = R0[rc];
-        // centred gradient with mirror ghosts (clamped ring)
-        const T gx = (R0[rc + 1] - R0[rc - 1]) * inv2dx;
-        const T gy = HY ? (R0[rc + RW] - R0[rc - RW]) * inv2dx : T(0);
-        const T gz = (Rp[rc] - Rm[rc]) * inv2dx;
-        const T G2 = gx * gx + gy * gy + gz * gz;
-        T as = 1, Nx = 0, Ny = 0, Nz = 0;
-        if (G2 >= g2min) as = aniso_N<T>(kind, e1, e2, gx, gy, gz, G2, Nx, Ny, Nz);
-        const T as2 = as * as;
-        const T inv_eta = rcp(c_eta * as2 + T(0.5));
-        const T omp2 = T(1) - ph * ph;
-        const T Qdt = (ph - (lamM * Usite + lam * thsite) * omp2) * omp2 * dt_tau0;
-        const T a2 = bnd ? T(1) : as2;
-        const T inv_a2 = bnd ? T(1) : rcp(a2);
-        const T oma2 = T(1) - a2;
+        // centred differences with mirror ghosts (clamped ring)
+        const T dy = HY ? radd(R0[rc + RW], -R0[rc - RW]) : T(0);
+        PhiCoef<T> co;
+        phi_coef<QP, S, T>(P, ph, Usite, thsite, radd(R0[rc + 1], -R0[rc - 1]), dy, radd(Rp[rc], -Rm[rc]), bnd,
+                           C::shifted ? (ringm + slot4(zc) * RS)[rc] : T(0), co);
+        phi_collide<QP>(co, gpull, gnl, row_needs);
         const bool store = icol && zc >= it.z0 && zc < it.z1;
-        // g* = [g (1 - 1/eta) - (1 - a^2) g_nl + g0/eta + w Q dt/tau0] / a^2 with
-        // g0 = w (phi - e.N c_N): per weight class (rest, axis, diagonal) the terms
-        // without e_i are one constant, and the e.N part is a signed sum of scaled N
-        const T omw = T(1) - inv_eta;
-        const T kph = radd(rmul(inv_eta, ph), Qdt);
-        const T ncN = rmul(inv_eta, c_N);
-        T Kc[3], nxc[3], nyc[3], nzc[3], Sc[3];
-        // FP16/BF16: the populations stay in the stored units G = (g - w phi_ref) S, phi_ref
-        // the phi of the step before at the node that stored them (phi^{n-1}); with
-        // Gp' = Gp + S w phi_ref(src) (pulled) and G* = (g* - w phi^n) S the collision becomes
-        //   G* = [omw Gp' - oma2 Gn + S (eq - w (oma2 phi_ref(x) + a^2 phi^n))] / a^2
-        // and the value gathered for phi^{n+1} is G* + S w phi^n
-        const T phr_x = C::shifted ? (ringm + slot4(zc) * RS)[rc] : T(0);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const T wc = (T)L::w(c == 0 ? 0 : (c == 1 ? 1 : L::diag0));
-          Kc[c] = rmul(wc, kph);
-          const T nc = rmul(-wc, ncN);
-          nxc[c] = rmul(nc, Nx);
-          nyc[c] = rmul(nc, Ny);
-          nzc[c] = rmul(nc, Nz);
-          if (C::shifted) {
-            Kc[c] = rmul(scale, radd(Kc[c], -rmul(wc, radd(rmul(oma2, phr_x), rmul(a2, ph)))));
-            nxc[c] = rmul(scale, nxc[c]);
-            nyc[c] = rmul(scale, nyc[c]);
-            nzc[c] = rmul(scale, nzc[c]);
-            Sc[c] = rmul(scale, rmul(wc, ph));
-          }
-        }
 #pragma unroll
         for (int i = 0; i < QP; ++i) {
-          const int ex = L::ex(i), ey = L::ey(i), ez = L::ez(i);
+          const int ey = L::ey(i);
           if (!row_needs(ey)) continue;
-          const int c = L::cls(i);
-          T eq = Kc[c];
-          if (ex) eq = radd(eq, ex > 0 ? nxc[c] : -nxc[c]);
-          if (ey) eq = radd(eq, ey > 0 ? nyc[c] : -nyc[c]);
-          if (ez) eq = radd(eq, ez > 0 ? nzc[c] : -nzc[c]);
-          const T g = rmul(fma(-oma2, gnl[i], fma(gpull[i], omw, eq)), inv_a2);
-          const auto enc = C::pack(g);
+          const auto enc = C::pack(gpull[i]);
           if (store) gout[(unsigned)i * NS + site] = enc;
-          gs[i] = C::shifted ? radd(C::raw(enc), Sc[c]) : g;
+          gs[i] = C::shifted ? rfma(rmul(scale, (T)L::w(i)), ph, C::raw(enc)) : gpull[i];
           if (ey != 0) sGb[YS::slot(i) * PS + ly * 32 + tx] = gs[i];
         }
       }
@@ -744,10 +344,12 @@ __device__ __forceinline__ void phi_tile(const SimDev* __restrict__ sims, const 
 }
 
 template <int QP, typename S, int BYC>
-__global__ void __launch_bounds__(32 * MAX_BLOCK_ROWS, sizeof(S) == 8 ? LBPF_PHI64_MIN_BLOCKS
-                                                       : (Lat<QP>::has_y ? LBPF_PHI_MIN_BLOCKS : LBPF_PHI2D_MIN_BLOCKS)) k_phi(const SimDev* __restrict__ sims, const WorkItem* __restrict__ items,
-                                                int s6) {
-  phi_tile<QP, S, BYC>(sims, items[blockIdx.x], s6);
+__global__ void __launch_bounds__(32 * MAX_BLOCK_ROWS, Lat<QP>::has_y ? LBPF_PHI_MIN_BLOCKS : LBPF_PHI2D_MIN_BLOCKS)
+    k_phi(const SimDev* __restrict__ sims, const WorkItem* __restrict__ items, int s6) {
+  const WorkItem it = items[blockIdx.x];
+  pdl_trigger();
+  pdl_wait();
+  phi_tile<QP, S, BYC>(sims, it, s6);
 }
 
 // ---------------------------------------------------------------- U and theta
@@ -795,13 +397,9 @@ __device__ __forceinline__ void uth_tile(const SimDev* __restrict__ sims, const 
   T* sH = ring + (TSH ? 8 : 4) * RS;         // [2][NYU + NYT][BY][32]
   constexpr int NYA = NYU + NYT;
 
-  const T inv2dx = (T)sd.inv2dx, k = (T)sd.k, inv_etaU = (T)sd.inv_etaU, c_J = (T)sd.c_J;
-  const T D_dx2 = (T)sd.D_dx2, D = (T)sd.D, at_amp = (T)sd.at_amp, inv_dt = (T)sd.inv_dt, dt = (T)sd.dt;
-  const T g2min = (T)sd.grad2_min, inv_etaT = (T)sd.inv_etaT;
-  const T sh_h = (T)sd.shift_h, sc_h = (T)sd.scale[1], isc_h = (T)sd.inv_scale[1];
-  const T sc_f = (T)sd.scale[2], isc_f = (T)sd.inv_scale[2];
+  const Consts<T> P = consts_of<T>(sd);
+  const T sh_h = P.shift_h, isc_h = P.inv_scale[1], sc_f = P.scale[2], isc_f = P.inv_scale[2];
   const bool at_on = sd.antitrapping != 0;
-  const T opk = T(1) + k, omk = T(1) - k;
 
   const int zlo = max(it.z0 - 1, 0), zhi = min(it.z1, nz - 1);
   RingMap rm;
@@ -866,7 +464,7 @@ __device__ __forceinline__ void uth_tile(const SimDev* __restrict__ sims, const 
             if (!row_needs(ey)) continue;
             fs[i] = C::raw(ldro(fin + ((unsigned)i * NS + site - (unsigned)(ez * (int)plane + ey * nx + ex))));
             if (TSH)  // stored units with the source's shift: F + S w theta^{n-1}(src)
-              fs[i] = fma(rmul(sc_f, (T)LT::w(i)), (ringt + slot4(zc - ez) * RS)[rc - ey * RW - ex], fs[i]);
+              fs[i] = rfma(rmul(sc_f, (T)LT::w(i)), (ringt + slot4(zc - ez) * RS)[rc - ey * RW - ex], fs[i]);
           }
         } else {
 #pragma unroll
@@ -889,119 +487,34 @@ __device__ __forceinline__ void uth_tile(const SimDev* __restrict__ sims, const 
             const int ii = inside ? i : LT::opp(i);
             fs[i] = C::raw(ldro(fin + ((unsigned)ii * NS + src)));
             if (TSH)
-              fs[i] = fma(rmul(sc_f, (T)LT::w(i)), (ringt + slot4(inside ? sz : zc) * RS)[inside ? rc - ey * RW - ex : rc],
+              fs[i] = rfma(rmul(sc_f, (T)LT::w(i)), (ringt + slot4(inside ? sz : zc) * RS)[inside ? rc - ey * RW - ex : rc],
                           fs[i]);
           }
         }
         // phi^{n+1} at the node and its six neighbours (mirror ghosts)
         const T pc = R0[rc];
         const T pxp = R0[rc + 1], pxm = R0[rc - 1], pyp = HY ? R0[rc + RW] : pc, pym = HY ? R0[rc - RW] : pc, pzp = Rp[rc], pzm = Rm[rc];
-        // q(phi) = (1 - phi)/2, zeta(phi) = ((1+k) - (1-k) phi)/2
-        auto qf = [&](T p) { return T(0.5) * (T(1) - p); };
-        // 1/zeta at the node and its six neighbours with one division (batch inversion):
-        // 2 zeta = (1+k) - (1-k) phi
-        const T d0 = opk - omk * pc, d1 = opk - omk * pxp, d2 = opk - omk * pxm, d3 = opk - omk * pyp,
-                d4 = opk - omk * pym, d5 = opk - omk * pzp, d6 = opk - omk * pzm;
-        const T p1 = d0 * d1, p2 = p1 * d2, p3 = p2 * d3, p4 = p3 * d4, p5 = p4 * d5, p6 = p5 * d6;
-        T rr = T(2) * rcp(p6);  // 2 / (d0 ... d6)
-        const T iz_zm = rr * p5;
-        rr *= d6;
-        const T iz_zp = rr * p4;
-        rr *= d5;
-        const T iz_ym = rr * p3;
-        rr *= d4;
-        const T iz_yp = rr * p2;
-        rr *= d3;
-        const T iz_xm = rr * p1;
-        rr *= d2;
-        const T iz_xp = rr * d0;
-        const T izc = rr * d1;
-        const T qc = qf(pc), qzc = qc * izc;
-        const T gpx = (pxp - pxm) * inv2dx, gpy = (pyp - pym) * inv2dx, gpz = (pzp - pzm) * inv2dx;
-        const T Fx = (iz_xp - iz_xm) * inv2dx, Fy = (iz_yp - iz_ym) * inv2dx, Fz = (iz_zp - iz_zm) * inv2dx;
-        const T gqzx = (qf(pxp) * iz_xp - qf(pxm) * iz_xm) * inv2dx;
-        const T gqzy = (qf(pyp) * iz_yp - qf(pym) * iz_ym) * inv2dx;
-        const T gqzz = (qf(pzp) * iz_zp - qf(pzm) * iz_zm) * inv2dx;
-        // div(D q grad(1/zeta)) in compact face form, face q = mean of nodal q
-        const T divDqF =
-            D_dx2 * (T(0.5) * (qc + qf(pxp)) * (iz_xp - izc) - T(0.5) * (qc + qf(pxm)) * (izc - iz_xm) +
-                     T(0.5) * (qc + qf(pyp)) * (iz_yp - izc) - T(0.5) * (qc + qf(pym)) * (izc - iz_ym) +
-                     T(0.5) * (qc + qf(pzp)) * (iz_zp - izc) - T(0.5) * (qc + qf(pzm)) * (izc - iz_zm));
-        const T dphi = pc - phn;  // phi^{n+1} - phi^n
-        const T dphidt = dphi * inv_dt;
-        const T fU = T(1) + omk * U;
-        T jx = 0, jy = 0, jz = 0;
-        const T G2 = gpx * gpx + gpy * gpy + gpz * gpz;
-        if (at_on && G2 >= g2min) {
-          const T iG = (sizeof(T) == 8) ? T(1) / sqrt(G2) : rsqrtf((float)G2);
-          const T amp = -at_amp * fU * dphidt * iG;
-          jx = amp * gpx;
-          jy = amp * gpy;
-          jz = amp * gpz;
-        }
-        const T DqU = D * U;
-        const T Jx = DqU * (gqzx + qc * Fx) + jx * izc;
-        const T Jy = DqU * (gqzy + qc * Fy) + jy * izc;
-        const T Jz = DqU * (gqzz + qc * Fz) + jz * izc;
-        const T Ssrc = U * divDqF + (jx * Fx + jy * Fy + jz * Fz);
-        const T src_dt = (Ssrc + fU * T(0.5) * dphidt * izc) * dt;
-        const T qzU = qzc * U;
+        UthCoef<T> co;
+        uth_coef<QU, QT, S, T>(P, at_on, U, th, phn, pc, pxp, pxm, pyp, pym, pzp, pzm, co);
         const bool store = icol && zc >= it.z0 && zc < it.z1;
-        // h* = h (1 - 1/eta_U) + h0/eta_U + w (S + Q_U/zeta) dt with
-        // h0 = A U + B (q/zeta U + e.J c_J): per weight class one constant plus e.(scaled J)
-        const T omU = T(1) - inv_etaU;
-        T KU[3], jxc[3], jyc[3], jzc[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const int ic = c == 0 ? 0 : (c == 1 ? 1 : LU::diag0);
-          const T wc = (T)LU::w(ic), Bc = (T)LU::B(ic);
-          KU[c] = radd(rmul(inv_etaU, radd(c == 0 ? U : T(0), rmul(Bc, qzU))), rmul(wc, src_dt));
-          const T jc = rmul(rmul(inv_etaU, Bc), c_J);
-          jxc[c] = rmul(jc, Jx);
-          jyc[c] = rmul(jc, Jy);
-          jzc[c] = rmul(jc, Jz);
-          if (C::shifted) {
-            // FP16/BF16: the populations stay in the stored units H = (h - w U0) S, so
-            // H* = H (1 - 1/eta_U) + S (h0/eta_U + w src dt - w U0 / eta_U)
-            KU[c] = rmul(sc_h, radd(KU[c], -rmul(rmul(wc, sh_h), inv_etaU)));
-            jxc[c] = rmul(sc_h, jxc[c]);
-            jyc[c] = rmul(sc_h, jyc[c]);
-            jzc[c] = rmul(sc_h, jzc[c]);
-          }
-        }
+        u_collide<QU>(co, hs, row_needs);
 #pragma unroll
         for (int i = 0; i < QU; ++i) {
-          const int ex = LU::ex(i), ey = LU::ey(i), ez = LU::ez(i);
+          const int ey = LU::ey(i);
           if (!row_needs(ey)) continue;
-          const int c = LU::cls(i);
-          T eq = KU[c];
-          if (ex) eq = radd(eq, ex > 0 ? jxc[c] : -jxc[c]);
-          if (ey) eq = radd(eq, ey > 0 ? jyc[c] : -jyc[c]);
-          if (ez) eq = radd(eq, ez > 0 ? jzc[c] : -jzc[c]);
-          const T h = fma(hs[i], omU, eq);
-          const auto enc = C::pack(h);
+          const auto enc = C::pack(hs[i]);
           if (store) hout[(unsigned)i * NS + site] = enc;
           hs[i] = C::raw(enc);
           if (ey != 0) sHb[YU::slot(i) * PS + ly * 32 + tx] = hs[i];
         }
         if (QT > 0) {
-          // f* = f (1 - 1/eta_T) + w (theta/eta_T + Q_theta dt) with Q_theta dt = dphi / 2
-          const T omT = T(1) - inv_etaT;
-          T kT = radd(rmul(inv_etaT, th), rmul(T(0.5), dphi));
-          // FP16/BF16: f is stored as F = (f - w theta_ref) S with theta_ref the theta of the
-          // storing node one step earlier; with F' = F + S w theta^{n-1}(src) (pulled) and
-          // F* = (f* - w theta^n) S the update is F* = F' (1 - 1/eta_T) + w S (dphi/2 - theta^n (1 - 1/eta_T)),
-          // and the value gathered for theta^{n+1} is F* + S w theta^n
-          if (C::shifted) kT = rmul(sc_f, radd(rmul(T(0.5), dphi), -rmul(th, omT)));
 #pragma unroll
           for (int i = 0; i < QT; ++i) {
             const int ey = LT::ey(i);
             if (!row_needs(ey)) continue;
-            const T wi = (T)LT::w(i);
-            const T f = fma(fs[i], omT, rmul(wi, kT));
-            const auto enc = C::pack(f);
+            const auto enc = C::pack(rfma(fs[i], co.At, co.Kt[LT::cls(i)]));
             if (store) fout[(unsigned)i * NS + site] = enc;
-            fs[i] = C::shifted ? radd(C::raw(enc), rmul(rmul(sc_f, wi), th)) : C::raw(enc);
+            fs[i] = C::shifted ? rfma(rmul(sc_f, (T)LT::w(i)), th, C::raw(enc)) : C::raw(enc);
             if (ey != 0) sFb[YT::slot(i) * PS + ly * 32 + tx] = fs[i];
           }
         }
@@ -1147,7 +660,7 @@ __device__ __forceinline__ void uth_tile(const SimDev* __restrict__ sims, const 
         const int zw = zc - 1;
         // FP16/BF16: the gathered sums are in stored units; the shifts w_i U0 (w_i theta0)
         // of the populations arriving at a node add up to U0 (theta0)
-        auto mU = [&](T a) { return C::shifted ? fma(a, isc_h, sh_h) : a; };
+        auto mU = [&](T a) { return C::shifted ? rfma(a, isc_h, sh_h) : a; };
         auto mT = [&](T a) { return C::shifted ? rmul(a, isc_f) : a; };
         if (zw >= it.z0 && zw < it.z1 && zw >= 0) {
           const unsigned sw = ((unsigned)zw * ny + y) * (unsigned)nx + x;
@@ -1173,10 +686,12 @@ __device__ __forceinline__ void uth_tile(const SimDev* __restrict__ sims, const 
 }
 
 template <int QU, int QT, typename S, int BYC>
-__global__ void __launch_bounds__(32 * MAX_BLOCK_ROWS, sizeof(S) == 8 ? LBPF_UTH64_MIN_BLOCKS
-                                                       : (Lat<QU>::has_y ? LBPF_UTH_MIN_BLOCKS : LBPF_UTH2D_MIN_BLOCKS)) k_uth(const SimDev* __restrict__ sims, const WorkItem* __restrict__ items,
-                                                int s6) {
-  uth_tile<QU, QT, S, false, BYC>(sims, items[blockIdx.x], s6);
+__global__ void __launch_bounds__(32 * MAX_BLOCK_ROWS, Lat<QU>::has_y ? LBPF_UTH_MIN_BLOCKS : LBPF_UTH2D_MIN_BLOCKS)
+    k_uth(const SimDev* __restrict__ sims, const WorkItem* __restrict__ items, int s6) {
+  const WorkItem it = items[blockIdx.x];
+  pdl_trigger();
+  pdl_wait();
+  uth_tile<QU, QT, S, false, BYC>(sims, it, s6);
 }
 
 // ---------------------------------------------------------------- one launch per step
@@ -1227,8 +742,7 @@ __device__ __forceinline__ bool wait_done(const unsigned* done, const int* dep, 
 }
 
 template <int QP, int QU, int QT, typename S>
-__global__ void __launch_bounds__(32 * MAX_BLOCK_ROWS, sizeof(S) == 8 ? LBPF_UTH64_MIN_BLOCKS
-                                                       : (Lat<QU>::has_y ? LBPF_UTH_MIN_BLOCKS : LBPF_UTH2D_MIN_BLOCKS)) k_step(const SimDev* __restrict__ sims, const WorkItem* __restrict__ items,
+__global__ void __launch_bounds__(32 * MAX_BLOCK_ROWS, Lat<QU>::has_y ? LBPF_UTH_MIN_BLOCKS : LBPF_UTH2D_MIN_BLOCKS) k_step(const SimDev* __restrict__ sims, const WorkItem* __restrict__ items,
                                                 const StepSched sc, int s6) {
   __shared__ int s_ticket;
   const bool lead = threadIdx.x == 0 && threadIdx.y == 0;

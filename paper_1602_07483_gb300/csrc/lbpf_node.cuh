@@ -1,0 +1,293 @@
+// lbpf_node.cuh -- the collisions of one node (Sec. 3.2-3.4), shared by every step kernel.
+//
+// Each routine turns a node's scalars into the coefficients of its collision; the
+// kernels apply them to the populations.  All arithmetic is spelled out in fused or
+// separately rounded operations, so that every kernel (a tile's owner and its halo, the
+// tiled, the node-wise and the one-launch step) rounds a node alike and their results
+// agree bit for bit.  The coefficients are arranged for few operations per population:
+// two FMAs and one addition for phi, one FMA and one addition for U, one FMA for theta,
+// with the e_i part of the equilibrium computed once per pair of opposite links.
+#pragma once
+
+#include "lbpf_lattice.cuh"
+
+namespace lbpf {
+
+// Products and sums that the compiler does not contract.
+__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// 1/x: IEEE division in FP64, the hardware approximate reciprocal in FP32
+__device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
+__device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
+__device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
+__device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
+
+// Read-only (non-coherent) load: what a step kernel reads this way is never written by the
+// same launch.
+template <typename S>
+__device__ __forceinline__ S ldro(const S* p) { return __ldg(p); }
+
+// Programmatic dependent launch: the kernels of a step are launched so that the next one may
+// start while the last blocks of this one still run.  pdl_trigger() allows that; pdl_wait()
+// returns once the kernels before have finished and their writes are visible, and comes
+// before the first access to what they write (or read, where this kernel writes it).
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Index of the first population of weight class c (0 rest, 1 axis, 2 diagonal).
+template <int Q>
+__host__ __device__ constexpr int class_rep(int c) {
+  return c == 0 ? 0 : (c == 1 ? 1 : Lat<Q>::diag0);
+}
+
+// Signed sum of the components of (ax, ay, az) along link i, added in x, y, z order: the
+// value for the opposite link is its exact negative.  Never called for the rest link.
+template <typename L, typename T>
+__device__ __forceinline__ T along(int i, T ax, T ay, T az) {
+  const int ex = L::ex(i), ey = L::ey(i), ez = L::ez(i);
+  T d = T(0);
+  bool any = false;
+  if (ex) { d = ex > 0 ? ax : -ax; any = true; }
+  if (ey) { const T v = ey > 0 ? ay : -ay; d = any ? radd(d, v) : v; any = true; }
+  if (ez) { const T v = ez > 0 ? az : -az; d = any ? radd(d, v) : v; }
+  return d;
+}
+
+// ---------------------------------------------------------------- phase field
+// g*_i = A g_i(x) + B g_i(x + e_i) + K_c + e_i . n_c, c the weight class of link i:
+// [g (1 - 1/eta) - (1 - a^2) g_nl + g0/eta + w Q dt/tau0] / a^2 with
+// g0 = w (phi - e.N c_N), the division by a^2 multiplied into every coefficient.
+// FP16/BF16: the same in the stored units G = (g - w phi_ref) S, phi_ref the phi^{n-1} of the
+// node that stored the value; with the pulled G' = G + S w phi_ref(src) and
+// G* = (g* - w phi^n) S only K changes, by -w (oma2 phi_ref(x) + a^2 phi^n), and the value
+// gathered for phi^{n+1} is G* + S w phi^n.
+template <typename T>
+struct PhiCoef {
+  T A, B, K[3], nx[3], ny[3], nz[3];
+};
+
+// ph, U, th: the node's values; dx, dy, dz: differences of phi across the node (twice the
+// gradient in units of 1/dx, mirror ghosts at walls); wall: standard collision (a^2 := 1 in
+// the prefactor and the non-local term); phr: phi_ref(x) (FP16/BF16).
+template <int QP, typename S, typename T>
+__device__ __forceinline__ void phi_coef(const Consts<T>& P, T ph, T U, T th, T dx, T dy, T dz, bool wall, T phr,
+                                         PhiCoef<T>& c) {
+  using L = Lat<QP>;
+  constexpr bool SH = Codec<S>::shifted;
+  const T s2 = rfma(dx, dx, rfma(dy, dy, rmul(dz, dz)));
+  T as = T(1), Nx = T(0), Ny = T(0), Nz = T(0);
+  if (rmul(s2, P.inv2dx2) >= P.grad2_min) {
+    // a_s(n) = a0 + a4 sum n^4 + a6 nx^2 ny^2 nz^2 covers Eq. (Anisotropic-Function_As) and
+    // Eq. (As_K41-K61); N = |grad phi|^2 a_s d a_s / d(grad phi) (Eq. TermesAnisotropes) with
+    // n = grad phi / |grad phi|, so that FP32 stays in range for small gradients
+    const T iG = rsq(s2);
+    const T nx = rmul(dx, iG), ny = rmul(dy, iG), nz = rmul(dz, iG);
+    const T x2 = rmul(nx, nx), y2 = rmul(ny, ny), z2 = rmul(nz, nz);
+    const T s4 = rfma(x2, x2, rfma(y2, y2, rmul(z2, z2)));
+    const T c4 = rmul(T(4), P.a4);
+    as = rfma(P.a4, s4, P.a0);
+    T px = rmul(c4, radd(x2, -s4)), py = rmul(c4, radd(y2, -s4)), pz = rmul(c4, radd(z2, -s4));
+    if (P.a6 != T(0)) {
+      const T yz = rmul(y2, z2), xz = rmul(x2, z2), xy = rmul(x2, y2);
+      const T c6 = rmul(T(2), P.a6);
+      as = rfma(P.a6, rmul(x2, yz), as);
+      px = rfma(rmul(c6, yz), rfma(T(-3), x2, T(1)), px);
+      py = rfma(rmul(c6, xz), rfma(T(-3), y2, T(1)), py);
+      pz = rfma(rmul(c6, xy), rfma(T(-3), z2, T(1)), pz);
+    }
+    const T f = rmul(rmul(rmul(s2, iG), P.inv2dx), as);  // |grad phi| a_s
+    Nx = rmul(f, rmul(nx, px));
+    Ny = rmul(f, rmul(ny, py));
+    Nz = rmul(f, rmul(nz, pz));
+  }
+  const T as2 = rmul(as, as);
+  const T eta = rfma(P.c_eta, as2, T(0.5));
+  const T a2 = wall ? T(1) : as2;
+  T inv_eta, inv_a2;
+  if constexpr (sizeof(T) == 8) {
+    const T r = rcp(rmul(eta, as2));  // one division for both
+    inv_eta = rmul(r, as2);
+    inv_a2 = wall ? T(1) : rmul(r, eta);
+  } else {
+    inv_eta = rcp(eta);
+    inv_a2 = wall ? T(1) : rcp(a2);
+  }
+  const T oma2 = radd(T(1), -a2);
+  const T omp2 = rfma(-ph, ph, T(1));
+  const T Q = rmul(rfma(-rfma(P.lamM, U, rmul(P.lam, th)), omp2, ph), omp2);
+  T kk = rfma(inv_eta, ph, rmul(Q, P.dt_tau0));
+  if (SH) kk = radd(kk, -rfma(oma2, phr, rmul(a2, ph)));
+  const T sa = SH ? rmul(P.scale[0], inv_a2) : inv_a2;
+  kk = rmul(kk, sa);
+  const T nn = -rmul(rmul(inv_eta, P.c_N), sa);
+  Nx = rmul(nn, Nx);
+  Ny = rmul(nn, Ny);
+  Nz = rmul(nn, Nz);
+  c.A = rmul(radd(T(1), -inv_eta), inv_a2);
+  c.B = -rmul(oma2, inv_a2);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const T w = (T)L::w(class_rep<QP>(k));
+    c.K[k] = rmul(w, kk);
+    c.nx[k] = rmul(w, Nx);
+    c.ny[k] = rmul(w, Ny);
+    c.nz[k] = rmul(w, Nz);
+  }
+}
+
+// Post-collision populations of the links wanted(e_y) in place of the pulled ones (in the
+// stored units, before the conversion to the storage type).
+template <int QP, typename T, typename W>
+__device__ __forceinline__ void phi_collide(const PhiCoef<T>& c, T (&gp)[QP], const T (&gn)[QP], W wanted) {
+  using L = Lat<QP>;
+  if (wanted(0)) gp[0] = rfma(c.A, gp[0], rfma(c.B, gn[0], c.K[0]));
+#pragma unroll
+  for (int i = 1; i < QP; ++i) {
+    const int j = L::opp(i);
+    if (j < i) continue;
+    const int k = L::cls(i);
+    const T d = along<L>(i, c.nx[k], c.ny[k], c.nz[k]);
+    if (wanted(L::ey(i))) gp[i] = rfma(c.A, gp[i], rfma(c.B, gn[i], radd(c.K[k], d)));
+    if (wanted(L::ey(j))) gp[j] = rfma(c.A, gp[j], rfma(c.B, gn[j], radd(c.K[k], -d)));
+  }
+}
+
+// ---------------------------------------------------------------- U and theta
+// h*_i = A h_i + K_c + e_i . j_c: h (1 - 1/eta_U) + h0/eta_U + w (S + Q_U/zeta) dt with
+// h0 = A U + B (q/zeta U + e.J c_J).  FP16/BF16: in the stored units H = (h - w U0) S.
+// f*_i = At f_i + Kt_c: f (1 - 1/eta_T) + w (theta/eta_T + dphi/2).  FP16/BF16: F is stored as
+// (f - w theta_ref) S, theta_ref the theta^{n-1} of the storing node; with the pulled
+// F' = F + S w theta_ref(src) and F* = (f* - w theta^n) S, Kt = S w (dphi/2 - theta^n (1 - 1/eta_T))
+// and the value gathered for theta^{n+1} is F* + S w theta^n.
+template <typename T>
+struct UthCoef {
+  T A, K[3], jx[3], jy[3], jz[3];
+  T At, Kt[3];
+};
+
+// phn: phi^n; pc and the six neighbours: phi^{n+1} (mirror ghosts at walls); U, th: U^n, theta^n.
+template <int QU, int QT, typename S, typename T>
+__device__ __forceinline__ void uth_coef(const Consts<T>& P, bool at_on, T U, T th, T phn, T pc, T pxp, T pxm, T pyp,
+                                         T pym, T pzp, T pzm, UthCoef<T>& c) {
+  using LU = Lat<QU>;
+  using LT = Lat<(QT > 0 ? QT : 7)>;
+  constexpr bool SH = Codec<S>::shifted;
+  constexpr bool HY = LU::has_y;
+  // 2 zeta = (1+k) - (1-k) phi; 1/zeta at the node and its neighbours with one division
+  const T opk = radd(T(1), P.k), omk = radd(T(1), -P.k);
+  auto zeta2 = [&](T p) { return rfma(-omk, p, opk); };
+  const T d0 = zeta2(pc), d1 = zeta2(pxp), d2 = zeta2(pxm), d5 = zeta2(pzp), d6 = zeta2(pzm);
+  T izc, iz_xp, iz_xm, iz_yp, iz_ym, iz_zp, iz_zm;
+  {
+    const T p1 = rmul(d0, d1), p2 = rmul(p1, d2);
+    T rr;
+    if constexpr (HY) {
+      const T d3 = zeta2(pyp), d4 = zeta2(pym);
+      const T p3 = rmul(p2, d3), p4 = rmul(p3, d4), p5 = rmul(p4, d5);
+      rr = rmul(T(2), rcp(rmul(p5, d6)));
+      iz_zm = rmul(rr, p5);
+      rr = rmul(rr, d6);
+      iz_zp = rmul(rr, p4);
+      rr = rmul(rr, d5);
+      iz_ym = rmul(rr, p3);
+      rr = rmul(rr, d4);
+      iz_yp = rmul(rr, p2);
+      rr = rmul(rr, d3);
+    } else {
+      const T p5 = rmul(p2, d5);
+      rr = rmul(T(2), rcp(rmul(p5, d6)));
+      iz_zm = rmul(rr, p5);
+      rr = rmul(rr, d6);
+      iz_zp = rmul(rr, p2);
+      rr = rmul(rr, d5);
+    }
+    iz_xm = rmul(rr, p1);
+    rr = rmul(rr, d2);
+    iz_xp = rmul(rr, d0);
+    izc = rmul(rr, d1);
+    if constexpr (!HY) iz_yp = iz_ym = izc;
+  }
+  // t = 2 q = 1 - phi; unscaled differences (the factors 1/(2 dx) and 1/2 come in at the end)
+  auto t2 = [&](T p) { return radd(T(1), -p); };
+  const T tc = t2(pc), txp = t2(pxp), txm = t2(pxm), tzp = t2(pzp), tzm = t2(pzm);
+  const T tyc_p = HY ? t2(pyp) : tc, tyc_m = HY ? t2(pym) : tc;
+  const T gx = radd(pxp, -pxm), gy = HY ? radd(pyp, -pym) : T(0), gz = radd(pzp, -pzm);
+  const T Fx = radd(iz_xp, -iz_xm), Fy = HY ? radd(iz_yp, -iz_ym) : T(0), Fz = radd(iz_zp, -iz_zm);
+  const T qx = rfma(txp, iz_xp, -rmul(txm, iz_xm)), qz = rfma(tzp, iz_zp, -rmul(tzm, iz_zm));
+  const T qy = HY ? rfma(tyc_p, iz_yp, -rmul(tyc_m, iz_ym)) : T(0);
+  // div(D q grad(1/zeta)) in compact face form, face q = mean of nodal q: 1/4 of this sum
+  T dv = rmul(radd(tc, txp), radd(iz_xp, -izc));
+  dv = rfma(radd(tc, txm), radd(iz_xm, -izc), dv);
+  if (HY) {
+    dv = rfma(radd(tc, tyc_p), radd(iz_yp, -izc), dv);
+    dv = rfma(radd(tc, tyc_m), radd(iz_ym, -izc), dv);
+  }
+  dv = rfma(radd(tc, tzp), radd(iz_zp, -izc), dv);
+  dv = rfma(radd(tc, tzm), radd(iz_zm, -izc), dv);
+  const T divDqF = rmul(rmul(T(0.25), P.D_dx2), dv);
+  const T dphi = radd(pc, -phn);
+  const T rate = rmul(dphi, P.inv_dt);
+  const T fU = rfma(omk, U, T(1));
+  T jx = T(0), jy = T(0), jz = T(0);
+  const T s2 = rfma(gx, gx, rfma(gy, gy, rmul(gz, gz)));
+  if (at_on && rmul(s2, P.inv2dx2) >= P.grad2_min) {  // Eq. (AntiTrapping_Current), n = grad phi / |grad phi|
+    const T amp = rmul(rmul(rmul(-P.at_amp, fU), rate), rsq(s2));
+    jx = rmul(amp, gx);
+    jy = rmul(amp, gy);
+    jz = rmul(amp, gz);
+  }
+  const T DU = rmul(rmul(rmul(T(0.5), P.D), P.inv2dx), U);
+  const T Jx = rfma(DU, rfma(tc, Fx, qx), rmul(jx, izc));
+  const T Jy = rfma(DU, rfma(tc, Fy, qy), rmul(jy, izc));
+  const T Jz = rfma(DU, rfma(tc, Fz, qz), rmul(jz, izc));
+  const T jF = rmul(P.inv2dx, rfma(jx, Fx, rfma(jy, Fy, rmul(jz, Fz))));
+  const T Ssrc = rfma(U, divDqF, jF);
+  const T src = rmul(rfma(rmul(rmul(T(0.5), fU), rate), izc, Ssrc), P.dt);
+  const T qzU = rmul(rmul(rmul(T(0.5), tc), izc), U);
+  const T sc = SH ? P.scale[1] : T(1);
+  const T cj = rmul(rmul(P.inv_etaU, P.c_J), sc);
+  const T jsx = rmul(cj, Jx), jsy = rmul(cj, Jy), jsz = rmul(cj, Jz);
+  c.A = radd(T(1), -P.inv_etaU);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const T w = (T)LU::w(class_rep<QU>(k)), b = (T)LU::B(class_rep<QU>(k));
+    const T eq = k == 0 ? rfma(b, qzU, U) : rmul(b, qzU);
+    T K = rfma(P.inv_etaU, eq, rmul(w, src));
+    if (SH) K = rmul(sc, rfma(-rmul(w, P.inv_etaU), P.shift_h, K));
+    c.K[k] = K;
+    c.jx[k] = rmul(b, jsx);
+    c.jy[k] = rmul(b, jsy);
+    c.jz[k] = rmul(b, jsz);
+  }
+  if (QT > 0) {
+    c.At = radd(T(1), -P.inv_etaT);
+    T kt = SH ? rmul(P.scale[2], rfma(-th, c.At, rmul(T(0.5), dphi))) : rfma(P.inv_etaT, th, rmul(T(0.5), dphi));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const T w = (T)LT::w(class_rep<(QT > 0 ? QT : 7)>(k));
+      c.Kt[k] = rmul(w, kt);
+    }
+  }
+}
+
+template <int QU, typename T, typename W>
+__device__ __forceinline__ void u_collide(const UthCoef<T>& c, T (&h)[QU], W wanted) {
+  using L = Lat<QU>;
+  if (wanted(0)) h[0] = rfma(c.A, h[0], c.K[0]);
+#pragma unroll
+  for (int i = 1; i < QU; ++i) {
+    const int j = L::opp(i);
+    if (j < i) continue;
+    const int k = L::cls(i);
+    const T d = along<L>(i, c.jx[k], c.jy[k], c.jz[k]);
+    if (wanted(L::ey(i))) h[i] = rfma(c.A, h[i], radd(c.K[k], d));
+    if (wanted(L::ey(j))) h[j] = rfma(c.A, h[j], radd(c.K[k], -d));
+  }
+}
+
+}  // namespace lbpf

@@ -15,6 +15,8 @@ namespace lbpf {
 
 constexpr int TILE_X = 30;  // interior columns per block row (block x = 32)
 
+constexpr int NODE_THREADS = 128;  // largest block of the node-wise kernels
+
 struct WorkItem {
   int sim;
   int x0, y0;  // first interior column of the tile
@@ -28,6 +30,34 @@ inline void build_items(int sim_index, int nx, int ny, int nz, int by, int zchun
   for (int z0 = 0; z0 < nz; z0 += zchunk)
     for (int y0 = 0; y0 < ny; y0 += ty)
       for (int x0 = 0; x0 < nx; x0 += TILE_X) out.push_back(WorkItem{sim_index, x0, y0, z0, std::min(nz, z0 + zchunk)});
+}
+
+// Blocks of one simulation's node-wise step: `threads` consecutive nodes of a plane (x0 the first)
+// over z-chunks of `zchunk` planes, z-chunk major.
+inline void build_node_items(int sim_index, int nx, int ny, int nz, int threads, int zchunk, std::vector<WorkItem>& out) {
+  const int plane = nx * ny;
+  for (int z0 = 0; z0 < nz; z0 += zchunk)
+    for (int p0 = 0; p0 < plane; p0 += threads)
+      out.push_back(WorkItem{sim_index, p0, 0, z0, std::min(nz, z0 + zchunk)});
+}
+
+// Threads of a node-wise block for a tiling of `by` rows (1: the 2D lattices, which have no rows
+// to choose).  128 (the default, by = 8) against 256 on GB300: 32^3 FP64 64 against 69 us per
+// step, 301^3 D3Q15/D3Q7/D3Q7 FP32 1835 against 1909 us, 256^3 FP16 the same.
+inline int node_threads(int by) { return by == 1 ? NODE_THREADS : 16 * by; }
+
+// Blocks of a node-wise kernel at one plane each.
+inline long long node_blocks(int nx, int ny, int nz, int threads) {
+  return ((long long)nx * ny + threads - 1) / threads * nz;
+}
+
+// Planes per block of the node-wise step: one while `blocks` blocks of a plane each do not fill
+// the chip several times over, then more, so that a block's start is shared by up to 16 planes
+// and phi along z stays in registers.  Measured best (us per step): 48^3 1 plane 20 (4: 43),
+// 128^3 FP32 4 planes 241 (16: 267), 256^3 FP16 16 planes 1630 (8: 1660, 32: 1720).
+inline int node_zchunk(long long blocks, int nz) {
+  const long long zc = blocks / 4000;
+  return (int)std::max<long long>(1, std::min<long long>({zc, 16, (long long)nz}));
 }
 
 struct TileGeom {

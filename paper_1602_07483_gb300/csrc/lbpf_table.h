@@ -18,7 +18,8 @@ struct KernelTable {
   int sbytes;            // bytes per stored population
   int tbytes;            // bytes of the compute type
   bool shifted;          // FP16/BF16 codec
-  // indexed by lattice_slot(q): 7, 15, 19, 5, 9; theta additionally 0 (frozen) in the last slot.
+  // the tiled step (3D: FP32; 2D: all but FP64; null elsewhere), indexed by
+  // lattice_slot(q): 7, 15, 19, 5, 9; theta additionally 0 (frozen) in the last slot.
   // Only pairings of one dimension are instantiated (the others are null).  Last index: the
   // block-height variant (block_variant): 1 for blocks of the height compiled in (8 rows in
   // 3D, one row in 2D), 0 for any height (the 2D entries are the one-row kernel in both).
@@ -26,6 +27,9 @@ struct KernelTable {
   StepLaunch uth[5][6][2];
   const void* phi_fn[5][2];
   const void* uth_fn[5][6][2];
+  // the node-wise step (lbpf_nodewise.cuh): collisions and moments of phi, then of U and theta
+  StepLaunch phi_node[5], phi_moment[5];
+  StepLaunch uth_node[5][6], uth_moment[5][6];
   // one-launch step kernels (k_step) by phi, U and theta slots; null where not instantiated
   // (FP64, and lattice triples other than D3Q19 x D3Q19 x {frozen, D3Q7, D3Q19} and
   // D2Q9 x D2Q5 x D2Q5)
@@ -49,12 +53,18 @@ struct KernelTable {
                      double* out);
 };
 
-// kernels compiled in translation units of their own (parallel compilation): the
-// 8-row 3D step kernels of each storage type, and the one-launch step kernels
-void add_fixed_kernels_f64(KernelTable& t);
+// kernels compiled in translation units of their own (parallel compilation): the 3D tiled step
+// of FP32 (any block height, and 8 rows), the node-wise step and the one-launch step
+void add_tile_kernels_f32(KernelTable& t);
 void add_fixed_kernels_f32(KernelTable& t);
-void add_fixed_kernels_f16(KernelTable& t);
-void add_fixed_kernels_bf16(KernelTable& t);
+void add_node_kernels_f64(KernelTable& t);
+void add_node_kernels_f32(KernelTable& t);
+void add_node_kernels_f16(KernelTable& t);
+void add_node_kernels_bf16(KernelTable& t);
+void add_moment_kernels_f64(KernelTable& t);
+void add_moment_kernels_f32(KernelTable& t);
+void add_moment_kernels_f16(KernelTable& t);
+void add_moment_kernels_bf16(KernelTable& t);
 void add_step_kernels_f32(KernelTable& t);
 void add_step_kernels_f16(KernelTable& t);
 void add_step_kernels_bf16(KernelTable& t);

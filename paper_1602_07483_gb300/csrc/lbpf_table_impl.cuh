@@ -4,6 +4,7 @@
 #pragma once
 
 #include "lbpf_aux.cuh"
+#include "lbpf_nodewise.cuh"
 #include "lbpf_table.h"
 
 namespace lbpf {
@@ -16,18 +17,80 @@ inline int aux_blocks(long long n) {
   return (int)(b < 1 ? 1 : b);
 }
 
+// Launch that may overlap the end of the kernel before it in the stream (pdl_wait).
+inline cudaError_t launch_pdl(void (*fn)(const SimDev*, const WorkItem*, int), dim3 g, dim3 b, size_t smem,
+                              cudaStream_t st, const SimDev* sims, const WorkItem* items, int s6) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = g;
+  cfg.blockDim = b;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, sims, items, s6);
+}
+
 template <int QP, typename S, int BYC>
 cudaError_t launch_phi(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
                        int s6) {
-  k_phi<QP, S, BYC><<<g, b, smem, st>>>(sims, items, s6);
-  return cudaGetLastError();
+  return launch_pdl(k_phi<QP, S, BYC>, g, b, smem, st, sims, items, s6);
 }
 
 template <int QU, int QT, typename S, int BYC>
 cudaError_t launch_uth(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
                        int s6) {
-  k_uth<QU, QT, S, BYC><<<g, b, smem, st>>>(sims, items, s6);
-  return cudaGetLastError();
+  return launch_pdl(k_uth<QU, QT, S, BYC>, g, b, smem, st, sims, items, s6);
+}
+
+template <int QP, typename S>
+cudaError_t launch_phi_node(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
+                            int s6) {
+  return launch_pdl(k_phi_node<QP, S>, g, b, smem, st, sims, items, s6);
+}
+template <int QP, typename S>
+cudaError_t launch_phi_moment(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
+                              int s6) {
+  return launch_pdl(k_phi_moment<QP, S>, g, b, smem, st, sims, items, s6);
+}
+template <int QU, int QT, typename S>
+cudaError_t launch_uth_node(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
+                            int s6) {
+  return launch_pdl(k_uth_node<QU, QT, S>, g, b, smem, st, sims, items, s6);
+}
+template <int QU, int QT, typename S>
+cudaError_t launch_uth_moment(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
+                              int s6) {
+  return launch_pdl(k_uth_moment<QU, QT, S>, g, b, smem, st, sims, items, s6);
+}
+
+// The U and theta pairings of one dimension.
+#define LBPF_UTH_PAIRS(M)                     \
+  M(7, 0) M(7, 7) M(7, 15) M(7, 19)           \
+  M(15, 0) M(15, 7) M(15, 15) M(15, 19)       \
+  M(19, 0) M(19, 7) M(19, 15) M(19, 19)       \
+  M(5, 0) M(5, 5) M(5, 9) M(9, 0) M(9, 5) M(9, 9)
+
+// The node-wise step's kernels, in two translation units per storage type.
+template <typename S>
+void fill_node_kernels(KernelTable& t) {
+#define LBPF_N(q) t.phi_node[lattice_slot(q)] = launch_phi_node<q, S>;
+  LBPF_N(7) LBPF_N(15) LBPF_N(19) LBPF_N(5) LBPF_N(9)
+#undef LBPF_N
+#define LBPF_N(qa, qb) t.uth_node[lattice_slot(qa)][lattice_slot(qb)] = launch_uth_node<qa, qb, S>;
+  LBPF_UTH_PAIRS(LBPF_N)
+#undef LBPF_N
+}
+template <typename S>
+void fill_moment_kernels(KernelTable& t) {
+#define LBPF_N(q) t.phi_moment[lattice_slot(q)] = launch_phi_moment<q, S>;
+  LBPF_N(7) LBPF_N(15) LBPF_N(19) LBPF_N(5) LBPF_N(9)
+#undef LBPF_N
+#define LBPF_N(qa, qb) t.uth_moment[lattice_slot(qa)][lattice_slot(qb)] = launch_uth_moment<qa, qb, S>;
+  LBPF_UTH_PAIRS(LBPF_N)
+#undef LBPF_N
 }
 
 template <int QP, int QU, int QT, typename S>
@@ -95,46 +158,37 @@ struct AuxImpl {
   }
 };
 
-// The two-kernel step's kernels for blocks of any height (3D) and the one-row kernels (2D).
+// The tiled step's one-row kernels of the 2D lattices (FP32, FP16, BF16; FP64 always steps
+// node-wise).
 template <typename S>
-void fill_step_kernels_general(KernelTable& t) {
-#define LBPF_PHI3(q)                                          \
-  t.phi[lattice_slot(q)][0] = launch_phi<q, S, 0>;             \
-  t.phi_fn[lattice_slot(q)][0] = (const void*)k_phi<q, S, 0>;
+void fill_tile_kernels_2d(KernelTable& t) {
 #define LBPF_PHI2(q)                                                                       \
   t.phi[lattice_slot(q)][0] = t.phi[lattice_slot(q)][1] = launch_phi<q, S, 1>;              \
   t.phi_fn[lattice_slot(q)][0] = t.phi_fn[lattice_slot(q)][1] = (const void*)k_phi<q, S, 1>;
-  LBPF_PHI3(7) LBPF_PHI3(15) LBPF_PHI3(19) LBPF_PHI2(5) LBPF_PHI2(9)
-#undef LBPF_PHI3
+  LBPF_PHI2(5) LBPF_PHI2(9)
 #undef LBPF_PHI2
-#define LBPF_UTH3(qa, qb)                                                            \
-  t.uth[lattice_slot(qa)][lattice_slot(qb)][0] = launch_uth<qa, qb, S, 0>;            \
-  t.uth_fn[lattice_slot(qa)][lattice_slot(qb)][0] = (const void*)k_uth<qa, qb, S, 0>;
 #define LBPF_UTH2(qa, qb)                                                                              \
   t.uth[lattice_slot(qa)][lattice_slot(qb)][0] = t.uth[lattice_slot(qa)][lattice_slot(qb)][1] =         \
       launch_uth<qa, qb, S, 1>;                                                                        \
   t.uth_fn[lattice_slot(qa)][lattice_slot(qb)][0] = t.uth_fn[lattice_slot(qa)][lattice_slot(qb)][1] =   \
       (const void*)k_uth<qa, qb, S, 1>;
-  LBPF_UTH3(7, 0) LBPF_UTH3(7, 7) LBPF_UTH3(7, 15) LBPF_UTH3(7, 19)
-  LBPF_UTH3(15, 0) LBPF_UTH3(15, 7) LBPF_UTH3(15, 15) LBPF_UTH3(15, 19)
-  LBPF_UTH3(19, 0) LBPF_UTH3(19, 7) LBPF_UTH3(19, 15) LBPF_UTH3(19, 19)
   LBPF_UTH2(5, 0) LBPF_UTH2(5, 5) LBPF_UTH2(5, 9)
   LBPF_UTH2(9, 0) LBPF_UTH2(9, 5) LBPF_UTH2(9, 9)
-#undef LBPF_UTH3
 #undef LBPF_UTH2
 }
 
-// The 3D two-kernel step's kernels compiled for blocks of MAX_BLOCK_ROWS rows.
-template <typename S>
-void fill_step_kernels_fixed(KernelTable& t) {
-#define LBPF_PHI3(q)                                                         \
-  t.phi[lattice_slot(q)][1] = launch_phi<q, S, MAX_BLOCK_ROWS>;               \
-  t.phi_fn[lattice_slot(q)][1] = (const void*)k_phi<q, S, MAX_BLOCK_ROWS>;
+// The tiled step's 3D kernels (FP32), block height compiled in (BYC rows) or any (BYC = 0).
+template <typename S, int BYC>
+void fill_tile_kernels_3d(KernelTable& t) {
+  constexpr int v = BYC > 0 ? 1 : 0;
+#define LBPF_PHI3(q)                                            \
+  t.phi[lattice_slot(q)][v] = launch_phi<q, S, BYC>;             \
+  t.phi_fn[lattice_slot(q)][v] = (const void*)k_phi<q, S, BYC>;
   LBPF_PHI3(7) LBPF_PHI3(15) LBPF_PHI3(19)
 #undef LBPF_PHI3
-#define LBPF_UTH3(qa, qb)                                                                           \
-  t.uth[lattice_slot(qa)][lattice_slot(qb)][1] = launch_uth<qa, qb, S, MAX_BLOCK_ROWS>;              \
-  t.uth_fn[lattice_slot(qa)][lattice_slot(qb)][1] = (const void*)k_uth<qa, qb, S, MAX_BLOCK_ROWS>;
+#define LBPF_UTH3(qa, qb)                                                              \
+  t.uth[lattice_slot(qa)][lattice_slot(qb)][v] = launch_uth<qa, qb, S, BYC>;            \
+  t.uth_fn[lattice_slot(qa)][lattice_slot(qb)][v] = (const void*)k_uth<qa, qb, S, BYC>;
   LBPF_UTH3(7, 0) LBPF_UTH3(7, 7) LBPF_UTH3(7, 15) LBPF_UTH3(7, 19)
   LBPF_UTH3(15, 0) LBPF_UTH3(15, 7) LBPF_UTH3(15, 15) LBPF_UTH3(15, 19)
   LBPF_UTH3(19, 0) LBPF_UTH3(19, 7) LBPF_UTH3(19, 15) LBPF_UTH3(19, 19)
@@ -147,7 +201,7 @@ KernelTable build_table() {
   t.sbytes = (int)sizeof(S);
   t.tbytes = (int)sizeof(typename Codec<S>::T);
   t.shifted = Codec<S>::shifted;
-  fill_step_kernels_general<S>(t);
+  if constexpr (sizeof(S) < 8) fill_tile_kernels_2d<S>(t);
   t.init_scalar = AuxImpl<S>::init_scalar;
   t.init_pop = AuxImpl<S>::init_pop;
   t.pack = AuxImpl<S>::pack;

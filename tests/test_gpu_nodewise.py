@@ -1,0 +1,59 @@
+"""The node-wise step (collisions without a halo, moments in a pass of their own) where it can
+go wrong: against the oracle at a size where a block spans several planes, and bit for bit
+against the tiled step where a batch and its members take different forms."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1602_07483_gb300 import lbpf, workloads
+
+pytestmark = pytest.mark.gpu
+
+
+def _pair(shape, lattices, seed=3):
+    p = workloads.base_params(kappa=100.0)
+    centres = np.array([[s // 2 if s > 1 else 0 for s in shape]], np.float64)
+    radii = np.array([6.0])
+    ora = oracle.Sim(shape, lattices, params=oracle.make_params(**p))
+    ora.init_seed(centres, radii, -0.55, -0.3)
+    noise = workloads.population_noise(shape, lattices, seed=seed)
+    state = [None if n is None else ora.pops(f) + n for f, n in enumerate(noise)]
+    ora.set_state(*state, theta0=-0.3)
+    gpu = lbpf.Sim(shape, lattices, storage="f64", **p)
+    gpu.set_state(*state, theta0=-0.3)
+    return gpu, ora
+
+
+# rows and planes that are no multiple of a block, blocks of two and of three planes with a
+# ragged last one, a plane smaller than a block; one step from the same noisy state: the
+# bound of the other one-step parity tests (1e-12 of the largest value)
+@pytest.mark.parametrize("shape,lattices", [((101, 104, 99), (19, 19, 7)), ((127, 130, 101), (15, 7, 0)),
+                                            ((11, 10, 61), (7, 15, 19))])
+def test_blocks_of_several_planes_match_oracle(shape, lattices):
+    gpu, ora = _pair(shape, lattices)
+    gpu.step(1)
+    ora.step(1)
+    for a, b in zip(gpu.read_fields(), ora.fields()):
+        assert np.abs(a - b).max() <= 1e-12 * max(1.0, np.abs(b).max())
+    for f, a in enumerate(gpu.get_state()):
+        if a is not None:
+            b = ora.pops(f)
+            assert np.abs(a - b).max() <= 1e-12 * max(1.0, np.abs(b).max())
+
+
+# a batch large enough to run tiled over members that run node-wise alone: the same values
+@pytest.mark.parametrize("shapes,lattices", [([(150, 149, 151)] * 3, (19, 19, 19)), ([(701, 500, 1), (640, 700, 1)], (9, 5, 9))])
+def test_tiled_batch_equals_node_wise_members(shapes, lattices):
+    p = dict(workloads.base_params(kappa=100.0), aniso=1, eps1=-0.02, eps2=0.015, dt=0.01)
+    batch = lbpf.Batch.create(shapes, lattices, [lbpf.make_params("f32", **p) for _ in shapes])
+    alone = [lbpf.Sim(s, lattices, storage="f32", **p) for s in shapes]
+    for k, (a, b) in enumerate(zip(batch.sims, alone)):
+        c = np.array([[20.0 + k, 15.0, 0.0 if shapes[k][2] == 1 else 9.0]])
+        for s in (a, b):
+            s.init_seed(c, np.array([7.0]), -0.5, -0.3)
+    batch.step(8)
+    for a, b in zip(batch.sims, alone):
+        b.step(8)
+        for x, y in zip(a.read_fields(), b.read_fields()):
+            assert np.array_equal(x, y)
+    batch.close()

@@ -491,6 +491,7 @@ void fill_dev(lbpf_sim* s) {
   c.inv2dx = 1.0 / (2.0 * p.dx);
   c.inv2dx2 = c.inv2dx * c.inv2dx;
   c.c_eta = W2t * p.dt / (p.dx * p.dx) / e2p;
+  c.inv_eta1 = 1.0 / (c.c_eta + 0.5);
   c.c_N = p.dt / p.dx * W2t / e2p;
   c.dt_tau0 = p.dt / p.tau0;
   c.lamM = p.lambda * p.Mc_inf;

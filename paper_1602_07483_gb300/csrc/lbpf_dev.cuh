@@ -226,7 +226,7 @@ __device__ __forceinline__ void phi_tile(const SimDev* __restrict__ sims, const 
         // centred differences with mirror ghosts (clamped ring)
         const T dy = HY ? radd(R0[rc + RW], -R0[rc - RW]) : T(0);
         PhiCoef<T> co;
-        phi_coef<QP, S, T>(P, ph, Usite, thsite, radd(R0[rc + 1], -R0[rc - 1]), dy, radd(Rp[rc], -Rm[rc]), bnd,
+        phi_coef<QP, S, false>(P, ph, Usite, thsite, radd(R0[rc + 1], -R0[rc - 1]), dy, radd(Rp[rc], -Rm[rc]), bnd,
                            C::shifted ? (ringm + slot4(zc) * RS)[rc] : T(0), co);
         phi_collide<QP>(co, gpull, gnl, row_needs);
         const bool store = icol && zc >= it.z0 && zc < it.z1;
@@ -495,7 +495,7 @@ __device__ __forceinline__ void uth_tile(const SimDev* __restrict__ sims, const 
         const T pc = R0[rc];
         const T pxp = R0[rc + 1], pxm = R0[rc - 1], pyp = HY ? R0[rc + RW] : pc, pym = HY ? R0[rc - RW] : pc, pzp = Rp[rc], pzm = Rm[rc];
         UthCoef<T> co;
-        uth_coef<QU, QT, S, T>(P, at_on, U, th, phn, pc, pxp, pxm, pyp, pym, pzp, pzm, co);
+        uth_coef<QU, QT, S>(P, at_on, U, th, phn, pc, pxp, pxm, pyp, pym, pzp, pzm, co);
         const bool store = icol && zc >= it.z0 && zc < it.z1;
         u_collide<QU>(co, hs, row_needs);
 #pragma unroll

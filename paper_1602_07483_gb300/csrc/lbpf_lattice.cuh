@@ -278,6 +278,7 @@ struct Consts {
   T inv2dx;       // 1 / (2 dx)
   T inv2dx2;      // its square
   T c_eta;        // e^-2 (W0^2/tau0) dt/dx^2: eta_phi = c_eta a_s^2 + 1/2 (Eq. LBE_RelaxationTime)
+  T inv_eta1;     // 1/eta_phi at a_s = 1
   T c_N;          // e^-2 (dt/dx) W0^2/tau0: the N term of g^(0) (Eq. Feq_Phase)
   T dt_tau0;      // dt / tau0
   T lamM, lam;    // lambda Mc_inf, lambda (Eq. LBE_SourceTerm)

@@ -69,22 +69,45 @@ __device__ __forceinline__ T along(int i, T ax, T ay, T az) {
 template <typename T>
 struct PhiCoef {
   T A, B, K[3], nx[3], ny[3], nz[3];
+  bool flat;  // no gradient: a_s = 1 and N = 0, so B and n_c vanish (and are not set), which spares
+              // most nodes of a run (bulk solid and melt) the anisotropy and the non-local term
 };
+
+// |grad phi|^2 >= grad2_min from the differences of phi across the node, below which n and N are
+// taken as 0 and a_s = 1.
+template <typename T>
+__device__ __forceinline__ bool has_gradient(const Consts<T>& P, T dx, T dy, T dz) {
+  return rmul(rfma(dx, dx, rfma(dy, dy, rmul(dz, dz))), P.inv2dx2) >= P.grad2_min;
+}
 
 // ph, U, th: the node's values; dx, dy, dz: differences of phi across the node (twice the
 // gradient in units of 1/dx, mirror ghosts at walls); wall: standard collision (a^2 := 1 in
 // the prefactor and the non-local term); phr: phi_ref(x) (FP16/BF16).
-template <int QP, typename S, typename T>
+// BRANCH: nodes without a gradient return early with `flat` set; otherwise `flat` stays false and
+// they take the general form with B = n_c = 0, to the same bits.
+template <int QP, typename S, bool BRANCH, typename T>
 __device__ __forceinline__ void phi_coef(const Consts<T>& P, T ph, T U, T th, T dx, T dy, T dz, bool wall, T phr,
                                          PhiCoef<T>& c) {
   using L = Lat<QP>;
   constexpr bool SH = Codec<S>::shifted;
-  const T s2 = rfma(dx, dx, rfma(dy, dy, rmul(dz, dz)));
+  const T omp2 = rfma(-ph, ph, T(1));
+  const T Q = rmul(rmul(rfma(-rfma(P.lamM, U, rmul(P.lam, th)), omp2, ph), omp2), P.dt_tau0);
+  const bool flat = !has_gradient(P, dx, dy, dz);
+  c.flat = BRANCH && flat;
+  if (c.flat) {
+    T kk = rfma(P.inv_eta1, ph, Q);
+    if (SH) kk = rmul(P.scale[0], radd(kk, -ph));
+    c.A = radd(T(1), -P.inv_eta1);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) c.K[k] = rmul((T)L::w(class_rep<QP>(k)), kk);
+    return;
+  }
   T as = T(1), Nx = T(0), Ny = T(0), Nz = T(0);
-  if (rmul(s2, P.inv2dx2) >= P.grad2_min) {
+  if (BRANCH || !flat) {
     // a_s(n) = a0 + a4 sum n^4 + a6 nx^2 ny^2 nz^2 covers Eq. (Anisotropic-Function_As) and
     // Eq. (As_K41-K61); N = |grad phi|^2 a_s d a_s / d(grad phi) (Eq. TermesAnisotropes) with
     // n = grad phi / |grad phi|, so that FP32 stays in range for small gradients
+    const T s2 = rfma(dx, dx, rfma(dy, dy, rmul(dz, dz)));
     const T iG = rsq(s2);
     const T nx = rmul(dx, iG), ny = rmul(dy, iG), nz = rmul(dz, iG);
     const T x2 = rmul(nx, nx), y2 = rmul(ny, ny), z2 = rmul(nz, nz);
@@ -112,15 +135,15 @@ __device__ __forceinline__ void phi_coef(const Consts<T>& P, T ph, T U, T th, T 
   if constexpr (sizeof(T) == 8) {
     const T r = rcp(rmul(eta, as2));  // one division for both
     inv_eta = rmul(r, as2);
-    inv_a2 = wall ? T(1) : rmul(r, eta);
+    inv_a2 = rmul(r, eta);
   } else {
     inv_eta = rcp(eta);
-    inv_a2 = wall ? T(1) : rcp(a2);
+    inv_a2 = rcp(a2);
   }
+  if (wall || flat) inv_a2 = T(1);
+  if (flat) inv_eta = P.inv_eta1;
   const T oma2 = radd(T(1), -a2);
-  const T omp2 = rfma(-ph, ph, T(1));
-  const T Q = rmul(rfma(-rfma(P.lamM, U, rmul(P.lam, th)), omp2, ph), omp2);
-  T kk = rfma(inv_eta, ph, rmul(Q, P.dt_tau0));
+  T kk = rfma(inv_eta, ph, Q);
   if (SH) kk = radd(kk, -rfma(oma2, phr, rmul(a2, ph)));
   const T sa = SH ? rmul(P.scale[0], inv_a2) : inv_a2;
   kk = rmul(kk, sa);
@@ -145,6 +168,12 @@ __device__ __forceinline__ void phi_coef(const Consts<T>& P, T ph, T U, T th, T 
 template <int QP, typename T, typename W>
 __device__ __forceinline__ void phi_collide(const PhiCoef<T>& c, T (&gp)[QP], const T (&gn)[QP], W wanted) {
   using L = Lat<QP>;
+  if (c.flat) {
+#pragma unroll
+    for (int i = 0; i < QP; ++i)
+      if (wanted(L::ey(i))) gp[i] = rfma(c.A, gp[i], c.K[L::cls(i)]);
+    return;
+  }
   if (wanted(0)) gp[0] = rfma(c.A, gp[0], rfma(c.B, gn[0], c.K[0]));
 #pragma unroll
   for (int i = 1; i < QP; ++i) {
@@ -167,6 +196,8 @@ __device__ __forceinline__ void phi_collide(const PhiCoef<T>& c, T (&gp)[QP], co
 template <typename T>
 struct UthCoef {
   T A, K[3], jx[3], jy[3], jz[3];
+  bool flat;  // phi^{n+1} is the same at the node and its six neighbours: J = S = 0, so j_c vanish
+              // (and are not set)
   T At, Kt[3];
 };
 
@@ -181,6 +212,35 @@ __device__ __forceinline__ void uth_coef(const Consts<T>& P, bool at_on, T U, T 
   // 2 zeta = (1+k) - (1-k) phi; 1/zeta at the node and its neighbours with one division
   const T opk = radd(T(1), P.k), omk = radd(T(1), -P.k);
   auto zeta2 = [&](T p) { return rfma(-omk, p, opk); };
+  const T dphi = radd(pc, -phn);
+  const T rate = rmul(dphi, P.inv_dt);
+  const T fU = rfma(omk, U, T(1));
+  const T tc = radd(T(1), -pc);  // t = 2 q = 1 - phi
+  const T sc = SH ? P.scale[1] : T(1);
+  c.A = radd(T(1), -P.inv_etaU);
+  if (QT > 0) {
+    c.At = radd(T(1), -P.inv_etaT);
+    const T kt = SH ? rmul(P.scale[2], rfma(-th, c.At, rmul(T(0.5), dphi))) : rfma(P.inv_etaT, th, rmul(T(0.5), dphi));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) c.Kt[k] = rmul((T)LT::w(class_rep<(QT > 0 ? QT : 7)>(k)), kt);
+  }
+  // K_c from q/zeta U and (S + Q_U/zeta) dt
+  auto set_K = [&](T qzU, T src) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const T w = (T)LU::w(class_rep<QU>(k)), b = (T)LU::B(class_rep<QU>(k));
+      const T eq = k == 0 ? rfma(b, qzU, U) : rmul(b, qzU);
+      T K = rfma(P.inv_etaU, eq, rmul(w, src));
+      if (SH) K = rmul(sc, rfma(-rmul(w, P.inv_etaU), P.shift_h, K));
+      c.K[k] = K;
+    }
+  };
+  c.flat = pxp == pc && pxm == pc && pyp == pc && pym == pc && pzp == pc && pzm == pc;
+  if (c.flat) {
+    const T izc = rmul(T(2), rcp(zeta2(pc)));
+    set_K(rmul(rmul(rmul(T(0.5), tc), izc), U), rmul(rmul(rmul(rmul(T(0.5), fU), rate), izc), P.dt));
+    return;
+  }
   const T d0 = zeta2(pc), d1 = zeta2(pxp), d2 = zeta2(pxm), d5 = zeta2(pzp), d6 = zeta2(pzm);
   T izc, iz_xp, iz_xm, iz_yp, iz_ym, iz_zp, iz_zm;
   {
@@ -212,9 +272,9 @@ __device__ __forceinline__ void uth_coef(const Consts<T>& P, bool at_on, T U, T 
     izc = rmul(rr, d1);
     if constexpr (!HY) iz_yp = iz_ym = izc;
   }
-  // t = 2 q = 1 - phi; unscaled differences (the factors 1/(2 dx) and 1/2 come in at the end)
+  // unscaled differences (the factors 1/(2 dx) and 1/2 come in at the end)
   auto t2 = [&](T p) { return radd(T(1), -p); };
-  const T tc = t2(pc), txp = t2(pxp), txm = t2(pxm), tzp = t2(pzp), tzm = t2(pzm);
+  const T txp = t2(pxp), txm = t2(pxm), tzp = t2(pzp), tzm = t2(pzm);
   const T tyc_p = HY ? t2(pyp) : tc, tyc_m = HY ? t2(pym) : tc;
   const T gx = radd(pxp, -pxm), gy = HY ? radd(pyp, -pym) : T(0), gz = radd(pzp, -pzm);
   const T Fx = radd(iz_xp, -iz_xm), Fy = HY ? radd(iz_yp, -iz_ym) : T(0), Fz = radd(iz_zp, -iz_zm);
@@ -230,9 +290,6 @@ __device__ __forceinline__ void uth_coef(const Consts<T>& P, bool at_on, T U, T 
   dv = rfma(radd(tc, tzp), radd(iz_zp, -izc), dv);
   dv = rfma(radd(tc, tzm), radd(iz_zm, -izc), dv);
   const T divDqF = rmul(rmul(T(0.25), P.D_dx2), dv);
-  const T dphi = radd(pc, -phn);
-  const T rate = rmul(dphi, P.inv_dt);
-  const T fU = rfma(omk, U, T(1));
   T jx = T(0), jy = T(0), jz = T(0);
   const T s2 = rfma(gx, gx, rfma(gy, gy, rmul(gz, gz)));
   if (at_on && rmul(s2, P.inv2dx2) >= P.grad2_min) {  // Eq. (AntiTrapping_Current), n = grad phi / |grad phi|
@@ -248,36 +305,27 @@ __device__ __forceinline__ void uth_coef(const Consts<T>& P, bool at_on, T U, T 
   const T jF = rmul(P.inv2dx, rfma(jx, Fx, rfma(jy, Fy, rmul(jz, Fz))));
   const T Ssrc = rfma(U, divDqF, jF);
   const T src = rmul(rfma(rmul(rmul(T(0.5), fU), rate), izc, Ssrc), P.dt);
-  const T qzU = rmul(rmul(rmul(T(0.5), tc), izc), U);
-  const T sc = SH ? P.scale[1] : T(1);
+  set_K(rmul(rmul(rmul(T(0.5), tc), izc), U), src);
   const T cj = rmul(rmul(P.inv_etaU, P.c_J), sc);
   const T jsx = rmul(cj, Jx), jsy = rmul(cj, Jy), jsz = rmul(cj, Jz);
-  c.A = radd(T(1), -P.inv_etaU);
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const T w = (T)LU::w(class_rep<QU>(k)), b = (T)LU::B(class_rep<QU>(k));
-    const T eq = k == 0 ? rfma(b, qzU, U) : rmul(b, qzU);
-    T K = rfma(P.inv_etaU, eq, rmul(w, src));
-    if (SH) K = rmul(sc, rfma(-rmul(w, P.inv_etaU), P.shift_h, K));
-    c.K[k] = K;
+    const T b = (T)LU::B(class_rep<QU>(k));
     c.jx[k] = rmul(b, jsx);
     c.jy[k] = rmul(b, jsy);
     c.jz[k] = rmul(b, jsz);
-  }
-  if (QT > 0) {
-    c.At = radd(T(1), -P.inv_etaT);
-    T kt = SH ? rmul(P.scale[2], rfma(-th, c.At, rmul(T(0.5), dphi))) : rfma(P.inv_etaT, th, rmul(T(0.5), dphi));
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const T w = (T)LT::w(class_rep<(QT > 0 ? QT : 7)>(k));
-      c.Kt[k] = rmul(w, kt);
-    }
   }
 }
 
 template <int QU, typename T, typename W>
 __device__ __forceinline__ void u_collide(const UthCoef<T>& c, T (&h)[QU], W wanted) {
   using L = Lat<QU>;
+  if (c.flat) {
+#pragma unroll
+    for (int i = 0; i < QU; ++i)
+      if (wanted(L::ey(i))) h[i] = rfma(c.A, h[i], c.K[L::cls(i)]);
+    return;
+  }
   if (wanted(0)) h[0] = rfma(c.A, h[0], c.K[0]);
 #pragma unroll
   for (int i = 1; i < QU; ++i) {

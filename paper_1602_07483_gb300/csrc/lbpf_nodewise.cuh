@@ -101,21 +101,26 @@ __device__ __forceinline__ T moment_sum(const NodeAt<HY>& at, int z, const T (&v
   return a;
 }
 
-// Resident blocks per SM (of 128 threads) that set the register budgets: 80 registers for the
-// phi collision, 128 for U and theta, 128 in FP64.
+// Resident blocks per SM (of 128 threads) that set the register budgets.  Measured, us per
+// step: phi FP32 at 6 blocks (80 registers) 256^3 D3Q19 696 (5 blocks 716); phi FP16 at 5 (96
+// registers) 711 (6: 777, spills); U and theta at 5 256^3 D3Q19/D3Q7 FP16 834 (4: 872, 3: 959), FP32
+// 918 (4: 921); FP64 at 3 (168 registers) 128^3 921 (4: 931, spills; 2: 983), 32^3 59 (4: 64).
 #ifndef LBPF_NODE_PHI_BLOCKS
 #define LBPF_NODE_PHI_BLOCKS 6
 #endif
+#ifndef LBPF_NODE16_PHI_BLOCKS
+#define LBPF_NODE16_PHI_BLOCKS 5
+#endif
 #ifndef LBPF_NODE_UTH_BLOCKS
-#define LBPF_NODE_UTH_BLOCKS 4
+#define LBPF_NODE_UTH_BLOCKS 5
 #endif
 #ifndef LBPF_NODE64_BLOCKS
-#define LBPF_NODE64_BLOCKS 4
+#define LBPF_NODE64_BLOCKS 3
 #endif
 
 // phi collision; writes the post-collision populations
 template <int QP, typename S>
-__global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 8 ? LBPF_NODE64_BLOCKS : LBPF_NODE_PHI_BLOCKS)
+__global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 8 ? LBPF_NODE64_BLOCKS : sizeof(S) == 2 ? LBPF_NODE16_PHI_BLOCKS : LBPF_NODE_PHI_BLOCKS)
     k_phi_node(const SimDev* __restrict__ sims, const WorkItem* __restrict__ items, int s6) {
   using C = Codec<S>;
   using T = typename C::T;
@@ -154,14 +159,17 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 8 ? LBPF_NODE64_BLO
     pull<QP, S>(at, z, site, gin, gp, [&](int i, unsigned s) {
       if (C::shifted) ref[i] = ldro(phim + s);
     });
+    const bool flat = !has_gradient(P, dx, dy, radd(cp, -cm));
+    if (!flat) {  // no non-local term in the bulk
 #pragma unroll
-    for (int i = 0; i < QP; ++i) gn[i] = wall ? T(0) : C::raw(ldro(gin + ((unsigned)i * at.NS + site)));
+      for (int i = 0; i < QP; ++i) gn[i] = wall ? T(0) : C::raw(ldro(gin + ((unsigned)i * at.NS + site)));
+    }
     if (C::shifted) {
 #pragma unroll
       for (int i = 0; i < QP; ++i) gp[i] = rfma(rmul(scale, (T)L::w(i)), ref[i], gp[i]);
     }
     PhiCoef<T> co;
-    phi_coef<QP, S, T>(P, cc, U, th, dx, dy, radd(cp, -cm), wall, C::shifted ? ref[0] : T(0), co);
+    phi_coef<QP, S, true>(P, cc, U, th, dx, dy, radd(cp, -cm), wall, C::shifted ? ref[0] : T(0), co);
     phi_collide<QP>(co, gp, gn, [](int) { return true; });
 #pragma unroll
     for (int i = 0; i < QP; ++i) gout[(unsigned)i * at.NS + site] = C::pack(gp[i]);
@@ -255,7 +263,7 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 8 ? LBPF_NODE64_BLO
       }
     }
     UthCoef<T> co;
-    uth_coef<QU, QT, S, T>(P, at_on, U, th, phn, cc, pxp, pxm, pyp, pym, cp, cm, co);
+    uth_coef<QU, QT, S>(P, at_on, U, th, phn, cc, pxp, pxm, pyp, pym, cp, cm, co);
     u_collide<QU>(co, h, [](int) { return true; });
 #pragma unroll
     for (int i = 0; i < QU; ++i) hout[(unsigned)i * at.NS + site] = C::pack(h[i]);

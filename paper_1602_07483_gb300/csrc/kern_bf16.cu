@@ -7,6 +7,7 @@ const KernelTable& table_bf16() {
     KernelTable k = build_table<__nv_bfloat16>();
     add_node_kernels_bf16(k);
     add_moment_kernels_bf16(k);
+    add_pair_kernels_bf16(k);
     add_step_kernels_bf16(k);
     return k;
   }();

@@ -7,6 +7,7 @@ const KernelTable& table_f16() {
     KernelTable k = build_table<__half>();
     add_node_kernels_f16(k);
     add_moment_kernels_f16(k);
+    add_pair_kernels_f16(k);
     add_step_kernels_f16(k);
     return k;
   }();

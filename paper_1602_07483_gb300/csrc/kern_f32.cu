@@ -9,6 +9,7 @@ const KernelTable& table_f32() {
     add_fixed_kernels_f32(k);
     add_node_kernels_f32(k);
     add_moment_kernels_f32(k);
+    add_pair_kernels_f32(k);
     add_step_kernels_f32(k);
     return k;
   }();

@@ -3,5 +3,5 @@
 #include "lbpf_table_impl.cuh"
 
 namespace lbpf {
-void add_moment_kernels_f16(KernelTable& t) { fill_moment_kernels<__half>(t); }
+void add_moment_kernels_f16(KernelTable& t) { fill_moment_kernels<__half, 1>(t); }
 }  // namespace lbpf

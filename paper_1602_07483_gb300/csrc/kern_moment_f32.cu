@@ -3,5 +3,5 @@
 #include "lbpf_table_impl.cuh"
 
 namespace lbpf {
-void add_moment_kernels_f32(KernelTable& t) { fill_moment_kernels<float>(t); }
+void add_moment_kernels_f32(KernelTable& t) { fill_moment_kernels<float, 1>(t); }
 }  // namespace lbpf

@@ -3,5 +3,5 @@
 #include "lbpf_table_impl.cuh"
 
 namespace lbpf {
-void add_moment_kernels_f64(KernelTable& t) { fill_moment_kernels<double>(t); }
+void add_moment_kernels_f64(KernelTable& t) { fill_moment_kernels<double, 1>(t); }
 }  // namespace lbpf

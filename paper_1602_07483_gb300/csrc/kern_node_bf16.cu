@@ -3,5 +3,5 @@
 #include "lbpf_table_impl.cuh"
 
 namespace lbpf {
-void add_node_kernels_bf16(KernelTable& t) { fill_node_kernels<__nv_bfloat16>(t); }
+void add_node_kernels_bf16(KernelTable& t) { fill_node_kernels<__nv_bfloat16, 1>(t); }
 }  // namespace lbpf

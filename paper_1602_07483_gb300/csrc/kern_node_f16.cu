@@ -3,5 +3,5 @@
 #include "lbpf_table_impl.cuh"
 
 namespace lbpf {
-void add_node_kernels_f16(KernelTable& t) { fill_node_kernels<__half>(t); }
+void add_node_kernels_f16(KernelTable& t) { fill_node_kernels<__half, 1>(t); }
 }  // namespace lbpf

@@ -1,0 +1,10 @@
+// kern_pair_bf16.cu -- node-wise kernels of two nodes per thread with __nv_bfloat16 storage (a translation
+// unit of their own so that they compile in parallel).
+#include "lbpf_table_impl.cuh"
+
+namespace lbpf {
+void add_pair_kernels_bf16(KernelTable& t) {
+  fill_node_kernels<__nv_bfloat16, 2>(t);
+  fill_moment_kernels<__nv_bfloat16, 2>(t);
+}
+}  // namespace lbpf

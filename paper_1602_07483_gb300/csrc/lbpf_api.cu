@@ -106,6 +106,7 @@ struct StepPlan {
   size_t smem[4] = {};
   int threads_y = 1, threads_x = 32;
   bool node_wise = false;
+  int nodes = 1;  // per thread of a node-wise kernel
   const SimDev* dd = nullptr;
   WorkItem* items = nullptr;  // device
   int nitems = 0;
@@ -301,16 +302,18 @@ int set_smem_attrs(const KernelTable& t, const lbpf_lattice& l, int device) {
 }
 
 // Kernels of the step of lattices `l` for blocks of `by` rows, or node-wise.
-void plan_kernels(StepPlan& p, const KernelTable& t, const lbpf_lattice& l, int by, bool node_wise) {
+void plan_kernels(StepPlan& p, const KernelTable& t, const lbpf_lattice& l, int by, bool node_wise, bool pairs) {
   const int a = q_index(l.q_phi), b = q_index(l.q_u), c = qt_index(l.q_theta);
   p.node_wise = node_wise;
   if (node_wise) {
     p.n = 4;
     p.nphi = 2;
-    p.fn[0] = t.phi_node[a];
-    p.fn[1] = t.phi_moment[a];
-    p.fn[2] = t.uth_node[b][c];
-    p.fn[3] = t.uth_moment[b][c];
+    const int v = pairs ? 1 : 0;
+    p.nodes = pairs ? 2 : 1;
+    p.fn[0] = t.phi_node[a][v];
+    p.fn[1] = t.phi_moment[a][v];
+    p.fn[2] = t.uth_node[b][c][v];
+    p.fn[3] = t.uth_moment[b][c][v];
     for (size_t& m : p.smem) m = 0;
     p.threads_x = node_threads(by);
     p.threads_y = 1;
@@ -343,23 +346,26 @@ int plan_items(StepPlan& p, const std::vector<WorkItem>& items) {
   return LBPF_OK;
 }
 
-// Whether simulations of `sites` nodes in all step node-wise (lbpf_nodewise.cuh) or tiled.
-// The tiled step reads the distributions once but spends 1.4 collisions per node, and small
-// grids have too few tiles for the chip; the node-wise step reads them twice.  Measured
-// (microseconds per step, tiled / node-wise):
-//   FP64, bound by its arithmetic, always node-wise: 128^3 D3Q19/D3Q19 2700 / 1340, 32^3 965 / 64,
+// Whether a node-wise step takes two nodes per thread: rows of even length, so that every pair
+// lies in one row and is aligned.
+bool takes_pairs(const KernelTable& t, const lbpf_grid& k) { return t.tbytes == 4 && k.nx % 2 == 0; }
+
+// Whether simulations of `sites` nodes in all step node-wise (lbpf_nodewise.cuh; `pairs`: two nodes
+// per thread, lbpf_nodepair.cuh) or tiled.  The tiled step reads the distributions once but
+// spends 1.4 collisions per node, and small grids have too few tiles for the chip; the node-wise
+// step reads them twice.  Measured (microseconds per step, tiled / node-wise):
+//   FP64, bound by its arithmetic, always node-wise: 128^3 D3Q19/D3Q19 2700 / 816, 32^3 965 / 50,
 //   8000^2 26500 / 23400.
-//   3D FP16/BF16, bound by instructions and latency, always node-wise: 96^3 D3Q19/D3Q19/D3Q7
-//   292 / 142, 256^3 1860 / 1630, 512^3 D3Q19 x 3 15450 / 15420.
-//   3D FP32: 96^3 235 / 111, 256^3 1703 / 1683, 400^3 6220 / 6150 with theta on D3Q7; with theta on
-//   D3Q19 192^3 924 / 903 but 256^3 1994 / 2066 and 512^3 14900 / 16050.
-//   2D FP32 and FP16 are tiled once the second read leaves L2: 500^2 29 / 17, 1000^2 58 / 62,
-//   4000^2 671 / 848.
-bool steps_node_wise(const KernelTable& t, const lbpf_lattice& l, long long sites) {
+//   3D FP16/BF16, always node-wise: 96^3 D3Q19/D3Q19/D3Q7 292 / 142 alone; 256^3 1860 / 1177 with pairs.
+//   3D FP32 with pairs, always node-wise: 96^3 229 / 94, 256^3 1640 / 1465, 512^3 D3Q19 x 3 14430 /
+//   14140; with odd rows 301^3 D3Q15/D3Q7/D3Q7 2133 / 1779, but D3Q19 x 3 at 512^3 14430 / 15080.
+//   2D FP32 and FP16 are tiled once the second read leaves L2: 500^2 28 / 14, 1000^2 58 / 62,
+//   8000^2 2381 / 2708.
+bool steps_node_wise(const KernelTable& t, const lbpf_lattice& l, long long sites, bool pairs) {
   if (t.tbytes == 8) return true;
   if (lattice_is_2d(l.q_phi)) return sites <= 700000;
   if (t.sbytes == 2) return true;
-  return l.q_theta + l.q_u <= 26 || sites <= 8000000;
+  return pairs || l.q_theta + l.q_u <= 26 || sites <= 8000000;
 }
 
 int apply_tiling(lbpf_sim* s, int by, int zchunk) {
@@ -367,15 +373,16 @@ int apply_tiling(lbpf_sim* s, int by, int zchunk) {
   if (lattice_is_2d(s->lat.q_phi)) by = 1;  // 2D: one-row blocks, no y halo
   s->by = by;
   s->zreq = zchunk;
-  plan_kernels(s->plan, t, s->lat, by, steps_node_wise(t, s->lat, s->nsite));
+  const bool pairs = takes_pairs(t, s->kg);
+  plan_kernels(s->plan, t, s->lat, by, steps_node_wise(t, s->lat, s->nsite, pairs), pairs);
   s->plan.dd = s->dd;
   const lbpf_grid& k = s->kg;
   const int tile_zc = zchunk > 0 ? zchunk : default_zchunk(k.nx, k.ny, k.nz, by);
   std::vector<WorkItem> items;
   if (s->plan.node_wise) {
-    const int threads = s->plan.threads_x;
-    const int zc = zchunk > 0 ? zchunk : node_zchunk(node_blocks(k.nx, k.ny, k.nz, threads), k.nz);
-    build_node_items(0, k.nx, k.ny, k.nz, threads, zc, items);
+    const int span = s->plan.threads_x * s->plan.nodes;
+    const int zc = zchunk > 0 ? zchunk : node_zchunk(node_blocks(k.nx, k.ny, k.nz, span), k.nz);
+    build_node_items(0, k.nx, k.ny, k.nz, span, zc, items);
     s->zchunk = zc;
   } else {
     int maxsm = 0;
@@ -1097,7 +1104,7 @@ int lbpf_autotune(lbpf_sim* s, int32_t steps, double* best_ms) {
     if (by > s->kg.ny + 2 && by != bys[0]) continue;
     const lbpf_grid& k = s->kg;
     const bool node = s->plan.node_wise && !s->ol.on;
-    const int zdef = node ? node_zchunk(node_blocks(k.nx, k.ny, k.nz, node_threads(s->by == 1 ? 1 : by)), k.nz)
+    const int zdef = node ? node_zchunk(node_blocks(k.nx, k.ny, k.nz, node_threads(s->by == 1 ? 1 : by) * s->plan.nodes), k.nz)
                           : default_zchunk(k.nx, k.ny, k.nz, by);
     const int zcs[] = {zdef, std::max(node ? 1 : 8, zdef / 2), std::min(k.nz, zdef * 2),
                        node ? std::min(k.nz, zdef * 4) : k.nz};
@@ -1218,18 +1225,20 @@ static int batch_tiling(lbpf_batch* b, int by, int zchunk) {
   std::vector<TileGeom> geo;
   long long sites = 0;
   for (const lbpf_sim* s : b->sims) sites += s->nsite;
-  plan_kernels(b->plan, t, l, by, steps_node_wise(t, l, sites));
+  bool pairs = true;
+  for (const lbpf_sim* s : b->sims) pairs = pairs && takes_pairs(t, s->kg);
+  plan_kernels(b->plan, t, l, by, steps_node_wise(t, l, sites, pairs), pairs);
   b->plan.dd = b->dd;
+  const int span = b->plan.threads_x * b->plan.nodes;
   long long blocks = 0;  // of one plane each, over all members
-  for (const lbpf_sim* s : b->sims) blocks += node_blocks(s->kg.nx, s->kg.ny, s->kg.nz, b->plan.threads_x);
+  for (const lbpf_sim* s : b->sims) blocks += node_blocks(s->kg.nx, s->kg.ny, s->kg.nz, span);
   for (size_t i = 0; i < b->sims.size(); ++i) {
     const lbpf_grid& k = b->sims[i]->kg;
     const int zc = zchunk > 0 ? std::min(zchunk, k.nz) : default_zchunk(k.nx, k.ny, k.nz, by);
     build_items((int)i, k.nx, k.ny, k.nz, by, zc, items);
     geo.push_back(TileGeom{k.nx, k.ny, k.nz, zc});
     if (b->plan.node_wise)
-      build_node_items((int)i, k.nx, k.ny, k.nz, b->plan.threads_x, zchunk > 0 ? zc : node_zchunk(blocks, k.nz),
-                       node_items);
+      build_node_items((int)i, k.nx, k.ny, k.nz, span, zchunk > 0 ? zc : node_zchunk(blocks, k.nz), node_items);
   }
   // interleave large and small simulations: sort items by descending z-chunk work
   for (std::vector<WorkItem>* v : {&items, &node_items})

@@ -25,20 +25,24 @@ struct NodeAt {
   unsigned plane, NS, p;
   int x, y;
   bool in;
-  __device__ __forceinline__ NodeAt(const SimDev& sd, const WorkItem& it)
-      : nx(sd.nx), ny(sd.ny), nz(sd.nz), plane((unsigned)sd.nx * (unsigned)sd.ny), NS((unsigned)sd.nsite),
-        p((unsigned)it.x0 + threadIdx.x) {
+  __device__ __forceinline__ NodeAt(const SimDev& sd, unsigned node)
+      : nx(sd.nx), ny(sd.ny), nz(sd.nz), plane((unsigned)sd.nx * (unsigned)sd.ny), NS((unsigned)sd.nsite), p(node) {
     in = p < plane;
     y = HY ? (int)(p / (unsigned)nx) : 0;
     x = (int)(p - (unsigned)y * (unsigned)nx);
   }
-  // the node is on no wall (of an axis the lattice has links along)
-  __device__ __forceinline__ bool inner(int z) const {
-    return x >= 1 && x <= nx - 2 && (!HY || (y >= 1 && y <= ny - 2)) && z >= 1 && z <= nz - 2;
-  }
+  // off the y and z walls (of the axes the lattice has links along): such nodes, x walls among
+  // them, take the path without wall checks, in which links from beyond an x wall are chosen by
+  // selects.  Most warps of short rows hold an x wall node; branching them into the general path
+  // ran both paths (48-column boxes: every warp).
+  __device__ __forceinline__ bool core(int z) const { return (!HY || (y >= 1 && y <= ny - 2)) && z >= 1 && z <= nz - 2; }
+  __device__ __forceinline__ bool inner(int z) const { return core(z) && x >= 1 && x <= nx - 2; }
   __device__ __forceinline__ bool has(int z, int ex, int ey, int ez) const {  // x - e is inside
     const int sx = x - ex, sy = y - ey, sz = z - ez;
     return sx >= 0 && sx < nx && sy >= 0 && sy < ny && sz >= 0 && sz < nz;
+  }
+  __device__ __forceinline__ bool beyond(int ex) const {  // x - e_x lies beyond an x wall
+    return ex > 0 ? x == 0 : (ex < 0 ? x == nx - 1 : false);
   }
   template <typename L>
   __device__ __forceinline__ unsigned back(int i) const {  // site(x) - site(x - e_i), modulo 2^32
@@ -53,12 +57,13 @@ __device__ __forceinline__ void pull(const NodeAt<HY>& at, int z, unsigned site,
                                      F src) {
   using L = Lat<Q>;
   using C = Codec<S>;
-  if (at.inner(z)) {
+  if (at.core(z)) {
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      const unsigned s = site - at.template back<L>(i);
-      v[i] = C::raw(ldro(pop + ((unsigned)i * at.NS + s)));
-      src(i, s);
+      const bool out = at.beyond(L::ex(i));
+      const unsigned back = out ? 0u : at.template back<L>(i);
+      v[i] = C::raw(ldro(pop + (site + ((unsigned)(out ? L::opp(i) : i) * at.NS - back))));
+      src(i, site - back);
     }
   } else {
 #pragma unroll
@@ -78,14 +83,18 @@ template <int Q, bool HY, typename T>
 __device__ __forceinline__ T moment_sum(const NodeAt<HY>& at, int z, const T (&v)[Q]) {
   using L = Lat<Q>;
   T a = T(0);
-  if (at.inner(z)) {
+  if (at.core(z)) {
 #pragma unroll
     for (int ez = 1; ez >= -1; --ez)
 #pragma unroll
       for (int y0 = 1; y0 >= 0; --y0)
 #pragma unroll
-        for (int i = 0; i < Q; ++i)
-          if (L::ez(i) == ez && (L::ey(i) == 0) == (y0 == 1)) a = radd(a, v[i]);
+        for (int i = 0; i < Q; ++i) {
+          if ((L::ey(i) == 0) != (y0 == 1)) continue;
+          // a link from beyond an x wall counts as the own plane's
+          if (L::ez(i) == ez) a = radd(a, ez != 0 && at.beyond(L::ex(i)) ? T(0) : v[i]);
+          else if (ez == 0 && L::ex(i) != 0) a = radd(a, at.beyond(L::ex(i)) ? v[i] : T(0));
+        }
   } else {
 #pragma unroll
     for (int ez = 1; ez >= -1; --ez)
@@ -128,7 +137,7 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 8 ? LBPF_NODE64_BLO
   constexpr bool HY = L::has_y;
   const WorkItem it = items[blockIdx.x];
   const SimDev& sd = sims[it.sim];
-  const NodeAt<HY> at(sd, it);
+  const NodeAt<HY> at(sd, (unsigned)it.x0 + threadIdx.x);
   pdl_trigger();
   // held in registers in FP16/BF16 (256^3: 733 against 752 us); read where used in FP32 and FP64,
   // whose registers are full (750 against 790 us, FP64 128^3 566 against 599 us)
@@ -162,7 +171,7 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 8 ? LBPF_NODE64_BLO
     const bool flat = !has_gradient(P, dx, dy, radd(cp, -cm));
     if (!flat) {  // no non-local term in the bulk
 #pragma unroll
-      for (int i = 0; i < QP; ++i) gn[i] = wall ? T(0) : C::raw(ldro(gin + ((unsigned)i * at.NS + site)));
+      for (int i = 0; i < QP; ++i) gn[i] = C::raw(ldro(gin + ((unsigned)i * at.NS + site)));  // B = 0 at walls
     }
     if (C::shifted) {
 #pragma unroll
@@ -188,7 +197,7 @@ __global__ void __launch_bounds__(NODE_THREADS)
   constexpr bool HY = L::has_y;
   const WorkItem it = items[blockIdx.x];
   const SimDev& sd = sims[it.sim];
-  const NodeAt<HY> at(sd, it);
+  const NodeAt<HY> at(sd, (unsigned)it.x0 + threadIdx.x);
   pdl_trigger();
   const Consts<T> P = consts_of<T>(sd);
   const S* __restrict__ g = (const S*)sd.pop[(s6 & 1) ^ 1][0];
@@ -224,7 +233,7 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 8 ? LBPF_NODE64_BLO
   constexpr bool HY = Lat<QU>::has_y;
   const WorkItem it = items[blockIdx.x];
   const SimDev& sd = sims[it.sim];
-  const NodeAt<HY> at(sd, it);
+  const NodeAt<HY> at(sd, (unsigned)it.x0 + threadIdx.x);
   pdl_trigger();
   const Consts<T> P = consts_of<T>(sd);
   const int par = s6 & 1;
@@ -288,7 +297,7 @@ __global__ void __launch_bounds__(NODE_THREADS)
   constexpr bool HY = Lat<QU>::has_y;
   const WorkItem it = items[blockIdx.x];
   const SimDev& sd = sims[it.sim];
-  const NodeAt<HY> at(sd, it);
+  const NodeAt<HY> at(sd, (unsigned)it.x0 + threadIdx.x);
   pdl_trigger();
   const Consts<T> P = consts_of<T>(sd);
   const int par = s6 & 1;

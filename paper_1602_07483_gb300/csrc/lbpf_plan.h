@@ -32,12 +32,12 @@ inline void build_items(int sim_index, int nx, int ny, int nz, int by, int zchun
       for (int x0 = 0; x0 < nx; x0 += TILE_X) out.push_back(WorkItem{sim_index, x0, y0, z0, std::min(nz, z0 + zchunk)});
 }
 
-// Blocks of one simulation's node-wise step: `threads` consecutive nodes of a plane (x0 the first)
+// Blocks of one simulation's node-wise step: `span` consecutive nodes of a plane (x0 the first)
 // over z-chunks of `zchunk` planes, z-chunk major.
-inline void build_node_items(int sim_index, int nx, int ny, int nz, int threads, int zchunk, std::vector<WorkItem>& out) {
+inline void build_node_items(int sim_index, int nx, int ny, int nz, int span, int zchunk, std::vector<WorkItem>& out) {
   const int plane = nx * ny;
   for (int z0 = 0; z0 < nz; z0 += zchunk)
-    for (int p0 = 0; p0 < plane; p0 += threads)
+    for (int p0 = 0; p0 < plane; p0 += span)
       out.push_back(WorkItem{sim_index, p0, 0, z0, std::min(nz, z0 + zchunk)});
 }
 
@@ -46,9 +46,9 @@ inline void build_node_items(int sim_index, int nx, int ny, int nz, int threads,
 // step, 301^3 D3Q15/D3Q7/D3Q7 FP32 1835 against 1909 us, 256^3 FP16 the same.
 inline int node_threads(int by) { return by == 1 ? NODE_THREADS : 16 * by; }
 
-// Blocks of a node-wise kernel at one plane each.
-inline long long node_blocks(int nx, int ny, int nz, int threads) {
-  return ((long long)nx * ny + threads - 1) / threads * nz;
+// Blocks of `span` nodes of a node-wise kernel at one plane each.
+inline long long node_blocks(int nx, int ny, int nz, int span) {
+  return ((long long)nx * ny + span - 1) / span * nz;
 }
 
 // Planes per block of the node-wise step: one while `blocks` blocks of a plane each do not fill

@@ -27,9 +27,10 @@ struct KernelTable {
   StepLaunch uth[5][6][2];
   const void* phi_fn[5][2];
   const void* uth_fn[5][6][2];
-  // the node-wise step (lbpf_nodewise.cuh): collisions and moments of phi, then of U and theta
-  StepLaunch phi_node[5], phi_moment[5];
-  StepLaunch uth_node[5][6], uth_moment[5][6];
+  // the node-wise step (lbpf_nodewise.cuh): collisions and moments of phi, then of U and theta;
+  // last index: one node per thread, or two (lbpf_nodepair.cuh; null for FP64)
+  StepLaunch phi_node[5][2], phi_moment[5][2];
+  StepLaunch uth_node[5][6][2], uth_moment[5][6][2];
   // one-launch step kernels (k_step) by phi, U and theta slots; null where not instantiated
   // (FP64, and lattice triples other than D3Q19 x D3Q19 x {frozen, D3Q7, D3Q19} and
   // D2Q9 x D2Q5 x D2Q5)
@@ -58,13 +59,16 @@ struct KernelTable {
 void add_tile_kernels_f32(KernelTable& t);
 void add_fixed_kernels_f32(KernelTable& t);
 void add_node_kernels_f64(KernelTable& t);
-void add_node_kernels_f32(KernelTable& t);
-void add_node_kernels_f16(KernelTable& t);
-void add_node_kernels_bf16(KernelTable& t);
 void add_moment_kernels_f64(KernelTable& t);
+void add_node_kernels_f32(KernelTable& t);
 void add_moment_kernels_f32(KernelTable& t);
+void add_pair_kernels_f32(KernelTable& t);
+void add_node_kernels_f16(KernelTable& t);
 void add_moment_kernels_f16(KernelTable& t);
+void add_pair_kernels_f16(KernelTable& t);
+void add_node_kernels_bf16(KernelTable& t);
 void add_moment_kernels_bf16(KernelTable& t);
+void add_pair_kernels_bf16(KernelTable& t);
 void add_step_kernels_f32(KernelTable& t);
 void add_step_kernels_f16(KernelTable& t);
 void add_step_kernels_bf16(KernelTable& t);

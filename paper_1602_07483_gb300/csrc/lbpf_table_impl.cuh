@@ -4,6 +4,7 @@
 #pragma once
 
 #include "lbpf_aux.cuh"
+#include "lbpf_nodepair.cuh"
 #include "lbpf_nodewise.cuh"
 #include "lbpf_table.h"
 
@@ -45,25 +46,30 @@ cudaError_t launch_uth(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDe
   return launch_pdl(k_uth<QU, QT, S, BYC>, g, b, smem, st, sims, items, s6);
 }
 
-template <int QP, typename S>
+// V nodes per thread (1 or 2; FP64 has no pairs)
+template <int QP, typename S, int V>
 cudaError_t launch_phi_node(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
                             int s6) {
-  return launch_pdl(k_phi_node<QP, S>, g, b, smem, st, sims, items, s6);
+  if constexpr (V == 2) return launch_pdl(k_phi_pair<QP, S>, g, b, smem, st, sims, items, s6);
+  else return launch_pdl(k_phi_node<QP, S>, g, b, smem, st, sims, items, s6);
 }
-template <int QP, typename S>
+template <int QP, typename S, int V>
 cudaError_t launch_phi_moment(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
                               int s6) {
-  return launch_pdl(k_phi_moment<QP, S>, g, b, smem, st, sims, items, s6);
+  if constexpr (V == 2) return launch_pdl(k_phi_moment2<QP, S>, g, b, smem, st, sims, items, s6);
+  else return launch_pdl(k_phi_moment<QP, S>, g, b, smem, st, sims, items, s6);
 }
-template <int QU, int QT, typename S>
+template <int QU, int QT, typename S, int V>
 cudaError_t launch_uth_node(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
                             int s6) {
-  return launch_pdl(k_uth_node<QU, QT, S>, g, b, smem, st, sims, items, s6);
+  if constexpr (V == 2) return launch_pdl(k_uth_pair<QU, QT, S>, g, b, smem, st, sims, items, s6);
+  else return launch_pdl(k_uth_node<QU, QT, S>, g, b, smem, st, sims, items, s6);
 }
-template <int QU, int QT, typename S>
+template <int QU, int QT, typename S, int V>
 cudaError_t launch_uth_moment(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
                               int s6) {
-  return launch_pdl(k_uth_moment<QU, QT, S>, g, b, smem, st, sims, items, s6);
+  if constexpr (V == 2) return launch_pdl(k_uth_moment2<QU, QT, S>, g, b, smem, st, sims, items, s6);
+  else return launch_pdl(k_uth_moment<QU, QT, S>, g, b, smem, st, sims, items, s6);
 }
 
 // The U and theta pairings of one dimension.
@@ -73,22 +79,22 @@ cudaError_t launch_uth_moment(dim3 g, dim3 b, size_t smem, cudaStream_t st, cons
   M(19, 0) M(19, 7) M(19, 15) M(19, 19)       \
   M(5, 0) M(5, 5) M(5, 9) M(9, 0) M(9, 5) M(9, 9)
 
-// The node-wise step's kernels, in two translation units per storage type.
-template <typename S>
+// The node-wise step's kernels with V nodes per thread, in translation units of their own.
+template <typename S, int V>
 void fill_node_kernels(KernelTable& t) {
-#define LBPF_N(q) t.phi_node[lattice_slot(q)] = launch_phi_node<q, S>;
+#define LBPF_N(q) t.phi_node[lattice_slot(q)][V - 1] = launch_phi_node<q, S, V>;
   LBPF_N(7) LBPF_N(15) LBPF_N(19) LBPF_N(5) LBPF_N(9)
 #undef LBPF_N
-#define LBPF_N(qa, qb) t.uth_node[lattice_slot(qa)][lattice_slot(qb)] = launch_uth_node<qa, qb, S>;
+#define LBPF_N(qa, qb) t.uth_node[lattice_slot(qa)][lattice_slot(qb)][V - 1] = launch_uth_node<qa, qb, S, V>;
   LBPF_UTH_PAIRS(LBPF_N)
 #undef LBPF_N
 }
-template <typename S>
+template <typename S, int V>
 void fill_moment_kernels(KernelTable& t) {
-#define LBPF_N(q) t.phi_moment[lattice_slot(q)] = launch_phi_moment<q, S>;
+#define LBPF_N(q) t.phi_moment[lattice_slot(q)][V - 1] = launch_phi_moment<q, S, V>;
   LBPF_N(7) LBPF_N(15) LBPF_N(19) LBPF_N(5) LBPF_N(9)
 #undef LBPF_N
-#define LBPF_N(qa, qb) t.uth_moment[lattice_slot(qa)][lattice_slot(qb)] = launch_uth_moment<qa, qb, S>;
+#define LBPF_N(qa, qb) t.uth_moment[lattice_slot(qa)][lattice_slot(qb)][V - 1] = launch_uth_moment<qa, qb, S, V>;
   LBPF_UTH_PAIRS(LBPF_N)
 #undef LBPF_N
 }

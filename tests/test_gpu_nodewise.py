@@ -42,7 +42,7 @@ def test_blocks_of_several_planes_match_oracle(shape, lattices):
 
 
 # a batch large enough to run tiled over members that run node-wise alone: the same values
-@pytest.mark.parametrize("shapes,lattices", [([(150, 149, 151)] * 3, (19, 19, 19)), ([(701, 500, 1), (640, 700, 1)], (9, 5, 9))])
+@pytest.mark.parametrize("shapes,lattices", [([(151, 149, 150)] * 3, (19, 19, 19)), ([(701, 500, 1), (640, 700, 1)], (9, 5, 9))])
 def test_tiled_batch_equals_node_wise_members(shapes, lattices):
     p = dict(workloads.base_params(kappa=100.0), aniso=1, eps1=-0.02, eps2=0.015, dt=0.01)
     batch = lbpf.Batch.create(shapes, lattices, [lbpf.make_params("f32", **p) for _ in shapes])
@@ -56,4 +56,31 @@ def test_tiled_batch_equals_node_wise_members(shapes, lattices):
         b.step(8)
         for x, y in zip(a.read_fields(), b.read_fields()):
             assert np.array_equal(x, y)
+    batch.close()
+
+
+# rows of even length step two nodes per thread; in a batch with one odd row length every member
+# takes one node per thread: the same values.  Rows shorter and longer than a warp's span, one and
+# two pairs long, thin boxes, D3Q7 to D3Q19, and both 2D lattices.
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("shapes,lattices", [([(48, 20, 18), (2, 9, 7), (66, 5, 3), (33, 12, 10)], (19, 19, 19)),
+                                             ([(4, 31, 6), (130, 7, 9), (31, 12, 10)], (15, 7, 15)),
+                                             ([(40, 1, 5), (62, 17, 16), (25, 12, 10)], (7, 15, 0)),
+                                             ([(258, 40, 1), (2, 77, 1), (91, 33, 1)], (9, 9, 5)),
+                                             ([(64, 50, 1), (91, 33, 1)], (5, 5, 9))])
+def test_pairs_equal_single_nodes(storage, shapes, lattices):
+    p = dict(workloads.base_params(kappa=100.0))
+    batch = lbpf.Batch.create(shapes, lattices, [lbpf.make_params(storage, **p) for _ in shapes])
+    alone = [lbpf.Sim(s, lattices, storage=storage, **p) for s in shapes]
+    for k, (a, b) in enumerate(zip(batch.sims, alone)):
+        c = np.array([[0.4 * shapes[k][0], 0.6 * shapes[k][1], 0.4 * (shapes[k][2] - 1)]])
+        for s in (a, b):
+            s.init_seed(c, np.array([4.0]), -0.55, -0.3)
+    batch.step(13)
+    for a, b in zip(batch.sims, alone):
+        b.step(13)
+        for x, y in zip(a.read_fields(), b.read_fields()):
+            assert np.isfinite(x).all() and np.array_equal(x, y)
+        for x, y in zip(a.get_state(), b.get_state()):
+            assert x is None or np.array_equal(x, y)
     batch.close()

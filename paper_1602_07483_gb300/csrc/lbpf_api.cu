@@ -512,6 +512,9 @@ void fill_dev(lbpf_sim* s) {
     c.a4 = p.eps1 + 3.0 * p.eps2;
     c.a6 = 66.0 * p.eps2;
   }
+  c.aniso = p.aniso;
+  c.eps1 = p.eps1;
+  c.eps2 = p.eps2;
   c.grad2_min = p.grad2_min > 0 ? p.grad2_min : 1e-12;
   c.k = p.k;
   c.inv_etaU = 1.0 / (p.D * p.dt / (p.dx * p.dx) / e2u + 0.5);

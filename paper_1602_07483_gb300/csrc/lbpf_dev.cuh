@@ -236,7 +236,7 @@ __device__ __forceinline__ void phi_tile(const SimDev* __restrict__ sims, const 
           if (!row_needs(ey)) continue;
           const auto enc = C::pack(gpull[i]);
           if (store) gout[(unsigned)i * NS + site] = enc;
-          gs[i] = C::shifted ? rfma(rmul(scale, (T)L::w(i)), ph, C::raw(enc)) : gpull[i];
+          gs[i] = C::shifted ? radd(C::raw(enc), shift_of<L>(scale, i, ph)) : gpull[i];
           if (ey != 0) sGb[YS::slot(i) * PS + ly * 32 + tx] = gs[i];
         }
       }
@@ -514,7 +514,7 @@ __device__ __forceinline__ void uth_tile(const SimDev* __restrict__ sims, const 
             if (!row_needs(ey)) continue;
             const auto enc = C::pack(rfma(fs[i], co.At, co.Kt[LT::cls(i)]));
             if (store) fout[(unsigned)i * NS + site] = enc;
-            fs[i] = C::shifted ? rfma(rmul(sc_f, (T)LT::w(i)), th, C::raw(enc)) : C::raw(enc);
+            fs[i] = C::shifted ? radd(C::raw(enc), shift_of<LT>(sc_f, i, th)) : C::raw(enc);
             if (ey != 0) sFb[YT::slot(i) * PS + ly * 32 + tx] = fs[i];
           }
         }

@@ -283,6 +283,7 @@ struct Consts {
   T dt_tau0;      // dt / tau0
   T lamM, lam;    // lambda Mc_inf, lambda (Eq. LBE_SourceTerm)
   T a0, a4, a6;   // a_s = a0 + a4 sum n^4 + a6 nx^2 ny^2 nz^2 (Eq. Anisotropic-Function_As, As_K41-K61)
+  T aniso, eps1, eps2;  // 0: Eq. Anisotropic-Function_As, 1: Eq. As_K41-K61, and its parameters
   T grad2_min;
   T k;
   T inv_etaU;     // 1 / eta_U (Eq. RelaxationTime_Concentration)

@@ -19,10 +19,11 @@ struct alignas(8) F2 {
 __device__ __forceinline__ F2 both(float a) { return F2{a, a}; }
 __device__ __forceinline__ F2 as_f2(float2 a) { return F2{a.x, a.y}; }
 __device__ __forceinline__ float2 as_v(F2 a) { return make_float2(a.x, a.y); }
+// Packed operations.  A sum of a packed product would be contracted, so no routine adds one.
 __device__ __forceinline__ F2 rmul(F2 a, F2 b) { return as_f2(__fmul2_rn(as_v(a), as_v(b))); }
 __device__ __forceinline__ F2 radd(F2 a, F2 b) { return as_f2(__fadd2_rn(as_v(a), as_v(b))); }
 __device__ __forceinline__ F2 rfma(F2 a, F2 b, F2 c) { return as_f2(__ffma2_rn(as_v(a), as_v(b), as_v(c))); }
-// a - b, rounded once
+// a - b
 __device__ __forceinline__ F2 rsub(F2 a, F2 b) { return rfma(b, both(-1.0f), a); }
 
 // Two consecutive stored numbers (the first at an even index), as raw FP32 values and back.
@@ -33,7 +34,7 @@ __device__ __forceinline__ F2 ld2(const __half* p) {
 __device__ __forceinline__ F2 ld2(const __nv_bfloat16* p) {
   return as_f2(__bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162*>(p))));
 }
-__device__ __forceinline__ void st2(float* p, F2 v) { *reinterpret_cast<float2*>(p) = as_v(v); }
+__device__ __forceinline__ void st2(float* p, F2 v) { *reinterpret_cast<float2*>(p) = make_float2(v.x, v.y); }
 __device__ __forceinline__ void st2(__half* p, F2 v) { *reinterpret_cast<__half2*>(p) = __floats2half2_rn(v.x, v.y); }
 __device__ __forceinline__ void st2(__nv_bfloat16* p, F2 v) {
   *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(v.x, v.y);
@@ -51,10 +52,23 @@ struct PairAt {
   __device__ __forceinline__ bool core(int z) const { return a.core(z); }
 };
 
-// Pulled populations of a pair; with REF, G + S w ref(source) in place of the raw stored number G
+// The FP16/BF16 shift on a raw stored number: fused for the pulled populations of a collision, rounded
+// on its own (shift_of) for the moments; there the products are scalar, since a packed product and
+// sum are contracted whatever their rounding says.
+template <bool FUSED>
+__device__ __forceinline__ float shifted(float ws, float ref, float raw) {
+  return FUSED ? rfma(ws, ref, raw) : radd(raw, rmul(ws, ref));
+}
+template <bool FUSED>
+__device__ __forceinline__ F2 shifted(float ws, F2 ref, F2 raw) {
+  if (FUSED) return rfma(both(ws), ref, raw);
+  return radd(raw, F2{rmul(ws, ref.x), rmul(ws, ref.y)});
+}
+
+// Pulled populations of a pair; with REF, the raw stored number G plus the shift S w ref(source)
 // (FP16/BF16; ref: phi or theta of the step that stored it).  Off the y and z walls a link from
 // beyond an x wall is chosen by selects (NodeAt::core).
-template <int Q, typename S, bool HY, bool REF>
+template <int Q, typename S, bool HY, bool REF, bool FUSED>
 __device__ __forceinline__ void pull2(const PairAt<HY>& at, int z, unsigned site, const S* __restrict__ pop,
                                       const float* __restrict__ ref, float scale, F2 (&v)[Q]) {
   using L = Lat<Q>;
@@ -94,8 +108,8 @@ __device__ __forceinline__ void pull2(const PairAt<HY>& at, int z, unsigned site
 #pragma unroll
           for (int i = 0; i < Q; ++i)
             if (L::ey(i) == ey && L::ez(i) == ez)
-              v[i] = rfma(both(rmul(scale, (float)L::w(i))),
-                          L::ex(i) == 0 ? m : (L::ex(i) > 0 ? F2{l, m.x} : F2{m.y, r}), v[i]);
+              v[i] = shifted<FUSED>(rmul(scale, (float)L::w(i)),
+                                    L::ex(i) == 0 ? m : (L::ex(i) > 0 ? F2{l, m.x} : F2{m.y, r}), v[i]);
         }
     }
   } else {
@@ -107,7 +121,7 @@ __device__ __forceinline__ void pull2(const PairAt<HY>& at, int z, unsigned site
         const bool inside = at1.has(z, L::ex(i), L::ey(i), L::ez(i));
         const unsigned s = inside ? site + n - at1.template back<L>(i) : site + n;
         float g = C::raw(ldro(pop + ((unsigned)(inside ? i : L::opp(i)) * at1.NS + s)));
-        if (REF) g = rfma(rmul(scale, (float)L::w(i)), ldro(ref + s), g);
+        if (REF) g = shifted<FUSED>(rmul(scale, (float)L::w(i)), ldro(ref + s), g);
         (n == 0 ? v[i].x : v[i].y) = g;
       }
     }
@@ -150,27 +164,6 @@ __device__ __forceinline__ F2 moment_sum2(const PairAt<HY>& at, int z, const F2 
     s.y = moment_sum<Q>(at.b, z, one);
   }
   return s;
-}
-
-// K_c + e_i . n_c and K_c - e_i . n_c for a link i and its opposite.
-template <typename L>
-__device__ __forceinline__ void eq_pair(int i, F2 K, F2 ax, F2 ay, F2 az, F2& eqi, F2& eqj) {
-  const int e[3] = {L::ex(i), L::ey(i), L::ez(i)};
-  const F2 a[3] = {ax, ay, az};
-  F2 d = both(0.0f);
-  int sign = 0;  // e_i . n = sign d
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    if (e[k] == 0) continue;
-    if (sign == 0) {
-      d = a[k];
-      sign = e[k];
-    } else {
-      d = e[k] == sign ? radd(d, a[k]) : rsub(d, a[k]);
-    }
-  }
-  eqi = sign > 0 ? radd(K, d) : rsub(K, d);
-  eqj = sign > 0 ? rsub(K, d) : radd(K, d);
 }
 
 // Resident blocks per SM (of 128 threads) that set the register budgets.  Measured, us per step:
@@ -232,7 +225,7 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_PHI
     const F2 dz = rsub(cp, cm);
     const F2 U = ld2(Un + site), th = has_th ? ld2(thn + site) : theta0;
     F2 g[QP];
-    pull2<QP, S, HY, C::shifted>(at, z, site, gin, phim, scale, g);
+    pull2<QP, S, HY, C::shifted, true>(at, z, site, gin, phim, scale, g);
     const bool fa = !has_gradient(P, dx.x, dy.x, dz.x), fb = !has_gradient(P, dx.y, dy.y, dz.y);
     if (fa && fb) {  // bulk: no non-local term
       PhiCoef<float> ca, cb;
@@ -240,7 +233,7 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_PHI
       phi_coef<QP, S, true>(P, cc.y, U.y, th.y, dx.y, dy.y, dz.y, false, 0.0f, cb);
 #pragma unroll
       for (int i = 0; i < QP; ++i)
-        st2(gout + ((unsigned)i * a.NS + site), rfma(F2{ca.A, cb.A}, g[i], F2{ca.K[L::cls(i)], cb.K[L::cls(i)]}));
+        st2(gout + ((unsigned)i * a.NS + site), rfma(g[i], F2{ca.omw, cb.omw}, F2{ca.K[L::cls(i)], cb.K[L::cls(i)]}));
     } else {
       F2 gn[QP];
       const bool wa = !a.inner(z), wb = !at.b.inner(z);
@@ -251,17 +244,13 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_PHI
       PhiCoef<float> ca, cb;
       phi_coef<QP, S, false>(P, cc.x, U.x, th.x, dx.x, dy.x, dz.x, wa, ref.x, ca);
       phi_coef<QP, S, false>(P, cc.y, U.y, th.y, dx.y, dy.y, dz.y, wb, ref.y, cb);
-      const F2 A{ca.A, cb.A}, B{ca.B, cb.B};
-      st2(gout + site, rfma(A, g[0], rfma(B, gn[0], F2{ca.K[0], cb.K[0]})));
+      const F2 omw{ca.omw, cb.omw}, noma2{-ca.oma2, -cb.oma2}, inv_a2{ca.inv_a2, cb.inv_a2};
 #pragma unroll
-      for (int i = 1; i < QP; ++i) {
-        const int j = L::opp(i), k = L::cls(i);
-        if (j < i) continue;
-        F2 ei, ej;
-        eq_pair<L>(i, F2{ca.K[k], cb.K[k]}, F2{ca.nx[k], cb.nx[k]}, F2{ca.ny[k], cb.ny[k]}, F2{ca.nz[k], cb.nz[k]}, ei,
-                   ej);
-        st2(gout + ((unsigned)i * a.NS + site), rfma(A, g[i], rfma(B, gn[i], ei)));
-        st2(gout + ((unsigned)j * a.NS + site), rfma(A, g[j], rfma(B, gn[j], ej)));
+      for (int i = 0; i < QP; ++i) {
+        const int k = L::cls(i);
+        const F2 eq = eq_of<L>(i, F2{ca.K[k], cb.K[k]}, F2{ca.nx[k], cb.nx[k]}, F2{ca.ny[k], cb.ny[k]},
+                               F2{ca.nz[k], cb.nz[k]});
+        st2(gout + ((unsigned)i * a.NS + site), rmul(rfma(noma2, gn[i], rfma(g[i], omw, eq)), inv_a2));
       }
     }
     cm = cc;
@@ -288,7 +277,7 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_MOM
   unsigned site = (unsigned)it.z0 * at.a.plane + at.a.p;
   for (int z = it.z0; z < it.z1; ++z, site += at.a.plane) {
     F2 v[QP];
-    pull2<QP, S, HY, C::shifted>(at, z, site, g, phin, scale, v);
+    pull2<QP, S, HY, C::shifted, false>(at, z, site, g, phin, scale, v);
     const F2 m = moment_sum2<QP>(at, z, v);
     st2(phinew + site, C::shifted ? rmul(m, both(iscale)) : m);
   }
@@ -332,33 +321,18 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_UTH
     const F2 yu = HY ? ld2(phi1 + (site + yp)) : cc, yd = HY ? ld2(phi1 + (site - ym)) : cc;
     const F2 U = ld2(Un + site), pn = ld2(phin + site), th = QT > 0 ? ld2(thn + site) : both(0.0f);
     F2 h[QU], f[QTL];
-    pull2<QU, S, HY, false>(at, z, site, hin, nullptr, 0.0f, h);
-    if (QT > 0) pull2<QTL, S, HY, C::shifted>(at, z, site, fin, thm, P.scale[2], f);
+    pull2<QU, S, HY, false, true>(at, z, site, hin, nullptr, 0.0f, h);
+    if (QT > 0) pull2<QTL, S, HY, C::shifted, true>(at, z, site, fin, thm, P.scale[2], f);
     UthCoef<float> ca, cb;
     uth_coef<QU, QT, S>(P, at_on, U.x, th.x, pn.x, cc.x, cc.y, l, yu.x, yd.x, cp.x, cm.x, ca);
     uth_coef<QU, QT, S>(P, at_on, U.y, th.y, pn.y, cc.y, r, cc.x, yu.y, yd.y, cp.y, cm.y, cb);
     const F2 A = both(ca.A);
-    if (ca.flat && cb.flat) {
 #pragma unroll
-      for (int i = 0; i < QU; ++i)
-        st2(hout + ((unsigned)i * a.NS + site), rfma(A, h[i], F2{ca.K[L::cls(i)], cb.K[L::cls(i)]}));
-    } else {
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        if (ca.flat) ca.jx[k] = ca.jy[k] = ca.jz[k] = 0.0f;
-        if (cb.flat) cb.jx[k] = cb.jy[k] = cb.jz[k] = 0.0f;
-      }
-      st2(hout + site, rfma(A, h[0], F2{ca.K[0], cb.K[0]}));
-#pragma unroll
-      for (int i = 1; i < QU; ++i) {
-        const int j = L::opp(i), k = L::cls(i);
-        if (j < i) continue;
-        F2 ei, ej;
-        eq_pair<L>(i, F2{ca.K[k], cb.K[k]}, F2{ca.jx[k], cb.jx[k]}, F2{ca.jy[k], cb.jy[k]}, F2{ca.jz[k], cb.jz[k]}, ei,
-                   ej);
-        st2(hout + ((unsigned)i * a.NS + site), rfma(A, h[i], ei));
-        st2(hout + ((unsigned)j * a.NS + site), rfma(A, h[j], ej));
-      }
+    for (int i = 0; i < QU; ++i) {
+      const int k = L::cls(i);
+      st2(hout + ((unsigned)i * a.NS + site),
+          rfma(h[i], A, eq_of<L>(i, F2{ca.K[k], cb.K[k]}, F2{ca.jx[k], cb.jx[k]}, F2{ca.jy[k], cb.jy[k]},
+                                 F2{ca.jz[k], cb.jz[k]})));
     }
     if (QT > 0) {
       const F2 At = both(ca.At);
@@ -395,13 +369,13 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_MOM
   for (int z = it.z0; z < it.z1; ++z, site += at.a.plane) {
     {
       F2 v[QU];
-      pull2<QU, S, HY, false>(at, z, site, h, nullptr, 0.0f, v);
+      pull2<QU, S, HY, false, false>(at, z, site, h, nullptr, 0.0f, v);
       const F2 m = moment_sum2<QU>(at, z, v);
       st2(Unew + site, C::shifted ? rfma(m, both(P.inv_scale[1]), both(P.shift_h)) : m);
     }
     if (QT > 0) {
       F2 v[QTL];
-      pull2<QTL, S, HY, C::shifted>(at, z, site, f, thn, P.scale[2], v);
+      pull2<QTL, S, HY, C::shifted, false>(at, z, site, f, thn, P.scale[2], v);
       const F2 m = moment_sum2<QTL>(at, z, v);
       st2(thnew + site, C::shifted ? rmul(m, both(P.inv_scale[2])) : m);
     }

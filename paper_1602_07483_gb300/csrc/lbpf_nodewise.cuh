@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(NODE_THREADS)
     });
     if (C::shifted) {
 #pragma unroll
-      for (int i = 0; i < QP; ++i) v[i] = rfma(rmul(scale, (T)L::w(i)), ref[i], v[i]);
+      for (int i = 0; i < QP; ++i) v[i] = radd(v[i], shift_of<L>(scale, i, ref[i]));
     }
     const T a = moment_sum<QP>(at, z, v);
     phinew[site] = C::shifted ? rmul(a, iscale) : a;
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(NODE_THREADS)
       });
       if (C::shifted) {
 #pragma unroll
-        for (int i = 0; i < QTL; ++i) v[i] = rfma(rmul(P.scale[2], (T)LT::w(i)), ref[i], v[i]);
+        for (int i = 0; i < QTL; ++i) v[i] = radd(v[i], shift_of<LT>(P.scale[2], i, ref[i]));
       }
       const T a = moment_sum<QTL>(at, z, v);
       thnew[site] = C::shifted ? rmul(a, P.inv_scale[2]) : a;

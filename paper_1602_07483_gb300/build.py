@@ -23,7 +23,7 @@ SOURCES = ["lbpf_api.cu", "kern_f64.cu", "kern_f32.cu", "kern_f16.cu", "kern_bf1
            "kern_moment_f64.cu", "kern_moment_f32.cu", "kern_moment_f16.cu", "kern_moment_bf16.cu",
            "kern_pair_f32.cu", "kern_pair_f16.cu", "kern_pair_bf16.cu",
            "lbpf_noalloc.cu"]
-HEADERS = ["lbpf_lattice.cuh", "lbpf_node.cuh", "lbpf_dev.cuh", "lbpf_nodewise.cuh", "lbpf_nodepair.cuh", "lbpf_aux.cuh", "lbpf_table.h", "lbpf_table_impl.cuh", "lbpf_plan.h"]
+HEADERS = ["lbpf_lattice.cuh", "lbpf_node.cuh", "lbpf_dev.cuh", "lbpf_nodewise.cuh", "lbpf_nodepair.cuh", "lbpf_plane.cuh", "lbpf_aux.cuh", "lbpf_table.h", "lbpf_table_impl.cuh", "lbpf_plan.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall"]
 

@@ -98,18 +98,31 @@ struct OneLaunch {
   unsigned polls = kWaitPolls;  // bound of each wait (lbpf_set_wait_polls)
 };
 
-// The launches of one step: the phase-field kernels, then the U/theta kernels, all over the
-// same blocks (one per work item).
-struct StepPlan {
-  int n = 0, nphi = 0;  // kernels per step; the first nphi are the phase-field phase
-  StepLaunch fn[4] = {};
-  size_t smem[4] = {};
-  int threads_y = 1, threads_x = 32;
-  bool node_wise = false;
-  int nodes = 1;  // per thread of a node-wise kernel
-  const SimDev* dd = nullptr;
+// The forms of a phase of the step: tiles with recomputed halos (lbpf_dev.cuh; planes with two nodes
+// per thread, lbpf_plane.cuh), or node-wise (lbpf_nodewise.cuh; lbpf_nodepair.cuh with two nodes per
+// thread).  All give the same bits, and the phases of a step choose independently.
+enum class StepForm { tile, plane, node, node_pairs };
+
+// The launches of one phase (phi, or U and theta): one or two kernels over the same blocks, one per
+// work item.
+struct PhasePlan {
+  StepForm form = StepForm::node;
+  int n = 0;
+  StepLaunch fn[2] = {};
+  size_t smem = 0;
+  int threads_x = 32, threads_y = 1;
   WorkItem* items = nullptr;  // device
   int nitems = 0;
+  bool node_wise() const { return form == StepForm::node || form == StepForm::node_pairs; }
+  int nodes() const { return form == StepForm::node_pairs || form == StepForm::plane ? 2 : 1; }  // per thread
+  int span() const { return threads_x * nodes(); }      // nodes of a node-wise block
+  int tile_x() const { return TILE_X * nodes(); }       // interior columns of a tile
+};
+
+// The launches of one step.
+struct StepPlan {
+  PhasePlan phase[2];  // phi, then U and theta
+  const SimDev* dd = nullptr;
 };
 
 struct lbpf_sim {
@@ -301,37 +314,32 @@ int set_smem_attrs(const KernelTable& t, const lbpf_lattice& l, int device) {
   return LBPF_OK;
 }
 
-// Kernels of the step of lattices `l` for blocks of `by` rows, or node-wise.
-void plan_kernels(StepPlan& p, const KernelTable& t, const lbpf_lattice& l, int by, bool node_wise, bool pairs) {
+// Kernels of a phase (0: phi, 1: U and theta) of lattices `l` in the given form, for blocks of `by` rows.
+void plan_kernels(PhasePlan& p, int phase, const KernelTable& t, const lbpf_lattice& l, int by, StepForm form) {
   const int a = q_index(l.q_phi), b = q_index(l.q_u), c = qt_index(l.q_theta);
-  p.node_wise = node_wise;
-  if (node_wise) {
-    p.n = 4;
-    p.nphi = 2;
-    const int v = pairs ? 1 : 0;
-    p.nodes = pairs ? 2 : 1;
-    p.fn[0] = t.phi_node[a][v];
-    p.fn[1] = t.phi_moment[a][v];
-    p.fn[2] = t.uth_node[b][c][v];
-    p.fn[3] = t.uth_moment[b][c][v];
-    for (size_t& m : p.smem) m = 0;
-    p.threads_x = node_threads(by);
-    p.threads_y = 1;
-    return;
-  }
-  const int v = block_variant(l.q_phi, by);
-  p.n = 2;
-  p.nphi = 1;
-  p.fn[0] = t.phi[a][v];
-  p.fn[1] = t.uth[b][c][v];
-  p.smem[0] = phi_smem_bytes(t, l.q_phi, by);
-  p.smem[1] = uth_smem_bytes(t, l.q_u, l.q_theta, by);
+  p.form = form;
+  p.smem = 0;
   p.threads_x = 32;
-  p.threads_y = by;
+  p.threads_y = 1;
+  p.n = 1;
+  if (p.node_wise()) {
+    const int v = p.nodes() - 1;
+    p.n = 2;
+    p.fn[0] = phase == 0 ? t.phi_node[a][v] : t.uth_node[b][c][v];
+    p.fn[1] = phase == 0 ? t.phi_moment[a][v] : t.uth_moment[b][c][v];
+    p.threads_x = node_threads(by);
+  } else if (form == StepForm::plane) {
+    p.fn[0] = phase == 0 ? t.phi_plane[a] : t.uth_plane[b][c];
+  } else {
+    const int v = block_variant(l.q_phi, by);
+    p.fn[0] = phase == 0 ? t.phi[a][v] : t.uth[b][c][v];
+    p.smem = phase == 0 ? phi_smem_bytes(t, l.q_phi, by) : uth_smem_bytes(t, l.q_u, l.q_theta, by);
+    p.threads_y = by;
+  }
 }
 
-// Copies the work items to the device (replacing the plan's).
-int plan_items(StepPlan& p, const std::vector<WorkItem>& items) {
+// Copies the work items to the device (replacing the phase's).
+int plan_items(PhasePlan& p, const std::vector<WorkItem>& items) {
   if (p.items) cudaFree(p.items);
   p.items = nullptr;
   p.nitems = 0;
@@ -346,26 +354,51 @@ int plan_items(StepPlan& p, const std::vector<WorkItem>& items) {
   return LBPF_OK;
 }
 
-// Whether a node-wise step takes two nodes per thread: rows of even length, so that every pair
-// lies in one row and is aligned.
+void free_plan(StepPlan& p) {
+  for (PhasePlan& f : p.phase)
+    if (f.items) cudaFree(f.items);
+}
+
+// Whether a step can take two nodes per thread: rows of even length, so that every pair lies in one
+// row and is aligned.
 bool takes_pairs(const KernelTable& t, const lbpf_grid& k) { return t.tbytes == 4 && k.nx % 2 == 0; }
 
-// Whether simulations of `sites` nodes in all step node-wise (lbpf_nodewise.cuh; `pairs`: two nodes
-// per thread, lbpf_nodepair.cuh) or tiled.  The tiled step reads the distributions once but
-// spends 1.4 collisions per node, and small grids have too few tiles for the chip; the node-wise
-// step reads them twice.  Measured (microseconds per step, tiled / node-wise):
-//   FP64, bound by its arithmetic, always node-wise: 128^3 D3Q19/D3Q19 2700 / 816, 32^3 965 / 50,
-//   8000^2 26500 / 23400.
-//   3D FP16/BF16, always node-wise: 96^3 D3Q19/D3Q19/D3Q7 292 / 142 alone; 256^3 1860 / 1177 with pairs.
-//   3D FP32 with pairs, always node-wise: 96^3 229 / 94, 256^3 1640 / 1465, 512^3 D3Q19 x 3 14430 /
-//   14140; with odd rows 301^3 D3Q15/D3Q7/D3Q7 2133 / 1779, but D3Q19 x 3 at 512^3 14430 / 15080.
-//   2D FP32 and FP16 are tiled once the second read leaves L2: 500^2 28 / 14, 1000^2 58 / 62,
-//   8000^2 2381 / 2708.
-bool steps_node_wise(const KernelTable& t, const lbpf_lattice& l, long long sites, bool pairs) {
-  if (t.tbytes == 8) return true;
-  if (lattice_is_2d(l.q_phi)) return sites <= 700000;
-  if (t.sbytes == 2) return true;
-  return pairs || l.q_theta + l.q_u <= 26 || sites <= 8000000;
+// The form of a phase (0: phi, 1: U and theta) for simulations of `sites` nodes in all.  Tiles read the
+// distributions once but spend 1.4 collisions per node, and small grids have too few tiles for
+// the chip; the node-wise forms read them twice.  Measured, microseconds per step (or of the phase):
+//   FP64, bound by its arithmetic, always node-wise: 128^3 D3Q19/D3Q19 tiled 2700, node-wise 816;
+//   32^3 965 / 50; 8000^2 26500 / 23400.
+//   3D FP16/BF16 node-wise: 96^3 D3Q19/D3Q19/D3Q7 292 / 142 alone; 256^3 1860 / 1197 with pairs.
+//   3D FP32 node-wise with pairs: 96^3 229 / 91, 256^3 D3Q19/D3Q19/D3Q7 1680 / 1480; but U and theta both
+//   on D3Q19 (38 populations): 256^3 1233 / 1275, 512^3 9200 / 9810 tiled from 8 M nodes on.  With odd
+//   rows 301^3 D3Q15/D3Q7/D3Q7 2133 / 1779, D3Q19 x 3 tiled from 8 M nodes on (512^3 14430 / 15080).
+//   2D FP32, FP16 and BF16: node-wise while the second read stays in L2 (500^2 tiled 29, node-wise 15;
+//   4244 x 186 61 / 42, 1000^2 59 / 54), then planes for U and theta (2000^2 FP32 tiled 93, plane 83,
+//   8000^2 1279 / 1062), and for phi from 12 M nodes on (2000^2 84 / 111, 8000^2 1141 / 1093; whole
+//   step FP32 2409 / 2143, FP16 2490 / 1773), else tiles.
+StepForm choose_form(int phase, const KernelTable& t, const lbpf_lattice& l, long long sites, bool pairs) {
+  const StepForm node = pairs ? StepForm::node_pairs : StepForm::node;
+  if (t.tbytes == 8) return node;
+  if (lattice_is_2d(l.q_phi)) {
+    if (sites <= (pairs ? 1200000 : 700000)) return node;
+    return pairs && (phase == 1 || sites > 12000000) ? StepForm::plane : StepForm::tile;
+  }
+  if (t.sbytes == 2 || sites <= 8000000 || l.q_u + l.q_theta <= 26) return node;
+  return phase == 0 && pairs ? node : StepForm::tile;
+}
+
+// Appends a phase's work items of one simulation; returns the z-chunk used.  `zchunk` 0: the
+// default, for `blocks` node-wise blocks of a plane each in all.
+int phase_items(const PhasePlan& p, int sim, const lbpf_grid& k, int zchunk, int by, long long blocks,
+                std::vector<WorkItem>& items) {
+  if (p.node_wise()) {
+    const int zc = zchunk > 0 ? std::min(zchunk, k.nz) : node_zchunk(blocks, k.nz);
+    build_node_items(sim, k.nx, k.ny, k.nz, p.span(), zc, items);
+    return zc;
+  }
+  const int zc = zchunk > 0 ? zchunk : default_zchunk(k.nx, k.ny, k.nz, by);
+  build_items(sim, k.nx, k.ny, k.nz, by, zc, items, p.tile_x());
+  return zc;
 }
 
 int apply_tiling(lbpf_sim* s, int by, int zchunk) {
@@ -373,28 +406,23 @@ int apply_tiling(lbpf_sim* s, int by, int zchunk) {
   if (lattice_is_2d(s->lat.q_phi)) by = 1;  // 2D: one-row blocks, no y halo
   s->by = by;
   s->zreq = zchunk;
-  const bool pairs = takes_pairs(t, s->kg);
-  plan_kernels(s->plan, t, s->lat, by, steps_node_wise(t, s->lat, s->nsite, pairs), pairs);
   s->plan.dd = s->dd;
   const lbpf_grid& k = s->kg;
   const int tile_zc = zchunk > 0 ? zchunk : default_zchunk(k.nx, k.ny, k.nz, by);
   std::vector<WorkItem> items;
-  if (s->plan.node_wise) {
-    const int span = s->plan.threads_x * s->plan.nodes;
-    const int zc = zchunk > 0 ? zchunk : node_zchunk(node_blocks(k.nx, k.ny, k.nz, span), k.nz);
-    build_node_items(0, k.nx, k.ny, k.nz, span, zc, items);
-    s->zchunk = zc;
-  } else {
+  for (int f = 1; f >= 0; --f) {
+    PhasePlan& p = s->plan.phase[f];
+    plan_kernels(p, f, t, s->lat, by, choose_form(f, t, s->lat, s->nsite, takes_pairs(t, k)));
     int maxsm = 0;
     CK(s, cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, s->device));
-    if ((int)s->plan.smem[0] > maxsm || (int)s->plan.smem[1] > maxsm) return LBPF_EINVAL;
-    build_items(0, k.nx, k.ny, k.nz, by, tile_zc, items);
-    s->zchunk = tile_zc;
-  }
-  const int rc0 = plan_items(s->plan, items);
-  if (rc0 != LBPF_OK) {
-    if (rc0 == LBPF_ECUDA) s->sticky = rc0;
-    return rc0;
+    if ((int)p.smem > maxsm) return LBPF_EINVAL;
+    items.clear();
+    s->zchunk = phase_items(p, 0, k, zchunk, by, node_blocks(k.nx, k.ny, k.nz, p.span()), items);
+    const int rc0 = plan_items(p, items);
+    if (rc0 != LBPF_OK) {
+      if (rc0 == LBPF_ECUDA) s->sticky = rc0;
+      return rc0;
+    }
   }
   if (s->gexec) cudaGraphExecDestroy(s->gexec);
   s->gexec = nullptr;
@@ -414,17 +442,21 @@ int apply_tiling(lbpf_sim* s, int by, int zchunk) {
   return rc;
 }
 
-// Kernels first .. last-1 of a step.
-int launch_kernels(cudaStream_t st, const StepPlan& p, int first, int last, int s6) {
-  for (int k = first; k < last; ++k)
-    if (p.fn[k](dim3(p.nitems), dim3(p.threads_x, p.threads_y), p.smem[k], st, p.dd, p.items, s6) != cudaSuccess)
+// The kernels of a phase.
+int launch_phase(cudaStream_t st, const StepPlan& plan, int phase, int s6) {
+  const PhasePlan& p = plan.phase[phase];
+  for (int k = 0; k < p.n; ++k)
+    if (p.fn[k](dim3(p.nitems), dim3(p.threads_x, p.threads_y), p.smem, st, plan.dd, p.items, s6) != cudaSuccess)
       return LBPF_ECUDA;
   return LBPF_OK;
 }
 
 // One step: the plan's kernels, or the one-launch kernel when `ol` is selected.
 int launch_step(cudaStream_t st, const StepPlan& p, int by, int s6, const OneLaunch& ol) {
-  if (!ol.on) return launch_kernels(st, p, 0, p.n, s6);
+  if (!ol.on) {
+    const int rc = launch_phase(st, p, 0, s6);
+    return rc != LBPF_OK ? rc : launch_phase(st, p, 1, s6);
+  }
   if (cudaMemsetAsync(ol.d_ctl, 0, ol.ctl_bytes, st) != cudaSuccess) return LBPF_ECUDA;
   return ol.fn(dim3(ol.grid), dim3(32, by), ol.smem, st, p.dd, ol.d_items, ol.sc, s6) == cudaSuccess ? LBPF_OK
                                                                                                     : LBPF_ECUDA;
@@ -555,7 +587,7 @@ void free_sim(lbpf_sim* s) {
   for (int l = 0; l < 3; ++l)
     if (s->th[l]) cudaFree(s->th[l]);
   if (s->dd) cudaFree(s->dd);
-  if (s->plan.items) cudaFree(s->plan.items);
+  free_plan(s->plan);
   if (s->d_part) cudaFree(s->d_part);
   if (s->d_small) cudaFree(s->d_small);
   if (s->h_small) cudaFreeHost(s->h_small);
@@ -742,9 +774,9 @@ int lbpf_step_timed(lbpf_sim* s, int64_t n, double ms_kernels[3]) {
     const int s6 = s6_of(s);
     // one launch per step: all of its time is counted as the first phase's
     int rc = s->ol.on ? launch_step(s->stream, s->plan, s->by, s6, s->ol)
-                      : launch_kernels(s->stream, s->plan, 0, s->plan.nphi, s6);
+                      : launch_phase(s->stream, s->plan, 0, s6);
     CK(s, cudaEventRecord(ev[2 * k + 1], s->stream));
-    if (rc == LBPF_OK && !s->ol.on) rc = launch_kernels(s->stream, s->plan, s->plan.nphi, s->plan.n, s6);
+    if (rc == LBPF_OK && !s->ol.on) rc = launch_phase(s->stream, s->plan, 1, s6);
     if (rc != LBPF_OK) {
       s->sticky = LBPF_ECUDA;
       return LBPF_ECUDA;
@@ -1106,8 +1138,9 @@ int lbpf_autotune(lbpf_sim* s, int32_t steps, double* best_ms) {
   for (int by : bys) {
     if (by > s->kg.ny + 2 && by != bys[0]) continue;
     const lbpf_grid& k = s->kg;
-    const bool node = s->plan.node_wise && !s->ol.on;
-    const int zdef = node ? node_zchunk(node_blocks(k.nx, k.ny, k.nz, node_threads(s->by == 1 ? 1 : by) * s->plan.nodes), k.nz)
+    const PhasePlan& p0 = s->plan.phase[0];
+    const bool node = p0.node_wise() && !s->ol.on;
+    const int zdef = node ? node_zchunk(node_blocks(k.nx, k.ny, k.nz, node_threads(s->by == 1 ? 1 : by) * p0.nodes()), k.nz)
                           : default_zchunk(k.nx, k.ny, k.nz, by);
     const int zcs[] = {zdef, std::max(node ? 1 : 8, zdef / 2), std::min(k.nz, zdef * 2),
                        node ? std::min(k.nz, zdef * 4) : k.nz};
@@ -1224,37 +1257,46 @@ int lbpf_load(lbpf_sim* s, const char* path) {
 static int batch_tiling(lbpf_batch* b, int by, int zchunk) {
   const KernelTable& t = *b->sims[0]->kt;
   const lbpf_lattice& l = b->sims[0]->lat;
-  std::vector<WorkItem> items, node_items;
+  std::vector<WorkItem> items, ol_items;
   std::vector<TileGeom> geo;
   long long sites = 0;
-  for (const lbpf_sim* s : b->sims) sites += s->nsite;
   bool pairs = true;
-  for (const lbpf_sim* s : b->sims) pairs = pairs && takes_pairs(t, s->kg);
-  plan_kernels(b->plan, t, l, by, steps_node_wise(t, l, sites, pairs), pairs);
-  b->plan.dd = b->dd;
-  const int span = b->plan.threads_x * b->plan.nodes;
-  long long blocks = 0;  // of one plane each, over all members
-  for (const lbpf_sim* s : b->sims) blocks += node_blocks(s->kg.nx, s->kg.ny, s->kg.nz, span);
-  for (size_t i = 0; i < b->sims.size(); ++i) {
-    const lbpf_grid& k = b->sims[i]->kg;
-    const int zc = zchunk > 0 ? std::min(zchunk, k.nz) : default_zchunk(k.nx, k.ny, k.nz, by);
-    build_items((int)i, k.nx, k.ny, k.nz, by, zc, items);
-    geo.push_back(TileGeom{k.nx, k.ny, k.nz, zc});
-    if (b->plan.node_wise)
-      build_node_items((int)i, k.nx, k.ny, k.nz, span, zchunk > 0 ? zc : node_zchunk(blocks, k.nz), node_items);
+  for (const lbpf_sim* s : b->sims) {
+    sites += s->nsite;
+    pairs = pairs && takes_pairs(t, s->kg);
   }
-  // interleave large and small simulations: sort items by descending z-chunk work
-  for (std::vector<WorkItem>* v : {&items, &node_items})
-    std::stable_sort(v->begin(), v->end(),
-                     [](const WorkItem& a, const WorkItem& c) { return (a.z1 - a.z0) > (c.z1 - c.z0); });
-  if (plan_items(b->plan, b->plan.node_wise ? node_items : items) != LBPF_OK) return LBPF_ENOMEM;
+  // large chunks first, so that large and small simulations interleave
+  auto by_chunk = [](const WorkItem& a, const WorkItem& c) { return (a.z1 - a.z0) > (c.z1 - c.z0); };
+  b->plan.dd = b->dd;
+  for (int f = 0; f < 2; ++f) {
+    PhasePlan& p = b->plan.phase[f];
+    plan_kernels(p, f, t, l, by, choose_form(f, t, l, sites, pairs));
+    long long blocks = 0;  // of one plane each, over all members
+    for (const lbpf_sim* s : b->sims) blocks += node_blocks(s->kg.nx, s->kg.ny, s->kg.nz, p.span());
+    items.clear();
+    for (size_t i = 0; i < b->sims.size(); ++i) {
+      const lbpf_grid& k = b->sims[i]->kg;
+      phase_items(p, (int)i, k, zchunk > 0 ? std::min(zchunk, k.nz) : 0, by, blocks, items);
+    }
+    std::stable_sort(items.begin(), items.end(), by_chunk);
+    if (plan_items(p, items) != LBPF_OK) return LBPF_ENOMEM;
+  }
+  if (b->ol.on) {
+    for (size_t i = 0; i < b->sims.size(); ++i) {
+      const lbpf_grid& k = b->sims[i]->kg;
+      const int zc = zchunk > 0 ? std::min(zchunk, k.nz) : default_zchunk(k.nx, k.ny, k.nz, by);
+      build_items((int)i, k.nx, k.ny, k.nz, by, zc, ol_items);
+      geo.push_back(TileGeom{k.nx, k.ny, k.nz, zc});
+    }
+    std::stable_sort(ol_items.begin(), ol_items.end(), by_chunk);
+  }
   b->by = by;
   b->zchunk = zchunk;
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
   b->gexec = nullptr;
   b->graph_ok = false;
   if (b->ol.on) {
-    const int rc = setup_one_launch(b->ol, items, geo, by, step_smem_bytes(t, l.q_phi, l.q_u, l.q_theta, by),
+    const int rc = setup_one_launch(b->ol, ol_items, geo, by, step_smem_bytes(t, l.q_phi, l.q_u, l.q_theta, by),
                                     t.step_fn[q_index(l.q_phi)][q_index(l.q_u)][qt_index(l.q_theta)],
                                     b->sims[0]->device);
     if (rc != LBPF_OK) return rc;
@@ -1523,7 +1565,7 @@ int lbpf_batch_destroy(lbpf_batch* b) {
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
   if (b->dd) cudaFree(b->dd);
   if (b->h_desc) cudaFreeHost(b->h_desc);
-  if (b->plan.items) cudaFree(b->plan.items);
+  free_plan(b->plan);
   if (b->ev) cudaEventDestroy(b->ev);
   // borrowed members outlive the batch: they keep a failure the batch saw, not its flag
   for (lbpf_sim* s : b->sims)

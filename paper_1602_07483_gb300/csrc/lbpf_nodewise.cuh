@@ -25,6 +25,9 @@ struct NodeAt {
   unsigned plane, NS, p;
   int x, y;
   bool in;
+  __device__ __forceinline__ NodeAt(const SimDev& sd, int x_, int y_)  // by coordinates (p and in unset)
+      : nx(sd.nx), ny(sd.ny), nz(sd.nz), plane((unsigned)sd.nx * (unsigned)sd.ny), NS((unsigned)sd.nsite), p(0), x(x_),
+        y(y_), in(false) {}
   __device__ __forceinline__ NodeAt(const SimDev& sd, unsigned node)
       : nx(sd.nx), ny(sd.ny), nz(sd.nz), plane((unsigned)sd.nx * (unsigned)sd.ny), NS((unsigned)sd.nsite), p(node) {
     in = p < plane;

@@ -23,13 +23,14 @@ struct WorkItem {
   int z0, z1;  // planes [z0, z1) written by this block
 };
 
-// Tiles of one simulation for blocks of `by` rows and z-chunks of `zchunk` planes, z-chunk
-// major, then rows, then columns.
-inline void build_items(int sim_index, int nx, int ny, int nz, int by, int zchunk, std::vector<WorkItem>& out) {
+// Tiles of one simulation for blocks of `by` rows (tiles of `tile_x` columns) and z-chunks of
+// `zchunk` planes, z-chunk major, then rows, then columns.
+inline void build_items(int sim_index, int nx, int ny, int nz, int by, int zchunk, std::vector<WorkItem>& out,
+                        int tile_x = TILE_X) {
   const int ty = by == 1 ? 1 : by - 2;  // interior rows per block: one-row blocks (2D) have no y halo
   for (int z0 = 0; z0 < nz; z0 += zchunk)
     for (int y0 = 0; y0 < ny; y0 += ty)
-      for (int x0 = 0; x0 < nx; x0 += TILE_X) out.push_back(WorkItem{sim_index, x0, y0, z0, std::min(nz, z0 + zchunk)});
+      for (int x0 = 0; x0 < nx; x0 += tile_x) out.push_back(WorkItem{sim_index, x0, y0, z0, std::min(nz, z0 + zchunk)});
 }
 
 // Blocks of one simulation's node-wise step: `span` consecutive nodes of a plane (x0 the first)

@@ -27,6 +27,9 @@ struct KernelTable {
   StepLaunch uth[5][6][2];
   const void* phi_fn[5][2];
   const void* uth_fn[5][6][2];
+  // the 2D step with two nodes per thread (lbpf_plane.cuh; null for FP64 and the 3D lattices)
+  StepLaunch phi_plane[5];
+  StepLaunch uth_plane[5][6];
   // the node-wise step (lbpf_nodewise.cuh): collisions and moments of phi, then of U and theta;
   // last index: one node per thread, or two (lbpf_nodepair.cuh; null for FP64)
   StepLaunch phi_node[5][2], phi_moment[5][2];

@@ -6,6 +6,7 @@
 #include "lbpf_aux.cuh"
 #include "lbpf_nodepair.cuh"
 #include "lbpf_nodewise.cuh"
+#include "lbpf_plane.cuh"
 #include "lbpf_table.h"
 
 namespace lbpf {
@@ -44,6 +45,17 @@ template <int QU, int QT, typename S, int BYC>
 cudaError_t launch_uth(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
                        int s6) {
   return launch_pdl(k_uth<QU, QT, S, BYC>, g, b, smem, st, sims, items, s6);
+}
+
+template <int QP, typename S>
+cudaError_t launch_phi_plane(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
+                             int s6) {
+  return launch_pdl(k_phi_plane<QP, S>, g, b, smem, st, sims, items, s6);
+}
+template <int QU, int QT, typename S>
+cudaError_t launch_uth_plane(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
+                             int s6) {
+  return launch_pdl(k_uth_plane<QU, QT, S>, g, b, smem, st, sims, items, s6);
 }
 
 // V nodes per thread (1 or 2; FP64 has no pairs)
@@ -87,6 +99,14 @@ void fill_node_kernels(KernelTable& t) {
 #undef LBPF_N
 #define LBPF_N(qa, qb) t.uth_node[lattice_slot(qa)][lattice_slot(qb)][V - 1] = launch_uth_node<qa, qb, S, V>;
   LBPF_UTH_PAIRS(LBPF_N)
+#undef LBPF_N
+}
+template <typename S>
+void fill_plane_kernels(KernelTable& t) {
+  t.phi_plane[lattice_slot(5)] = launch_phi_plane<5, S>;
+  t.phi_plane[lattice_slot(9)] = launch_phi_plane<9, S>;
+#define LBPF_N(qa, qb) t.uth_plane[lattice_slot(qa)][lattice_slot(qb)] = launch_uth_plane<qa, qb, S>;
+  LBPF_N(5, 0) LBPF_N(5, 5) LBPF_N(5, 9) LBPF_N(9, 0) LBPF_N(9, 5) LBPF_N(9, 9)
 #undef LBPF_N
 }
 template <typename S, int V>
@@ -207,7 +227,10 @@ KernelTable build_table() {
   t.sbytes = (int)sizeof(S);
   t.tbytes = (int)sizeof(typename Codec<S>::T);
   t.shifted = Codec<S>::shifted;
-  if constexpr (sizeof(S) < 8) fill_tile_kernels_2d<S>(t);
+  if constexpr (sizeof(S) < 8) {
+    fill_tile_kernels_2d<S>(t);
+    fill_plane_kernels<S>(t);
+  }
   t.init_scalar = AuxImpl<S>::init_scalar;
   t.init_pop = AuxImpl<S>::init_pop;
   t.pack = AuxImpl<S>::pack;

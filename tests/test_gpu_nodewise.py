@@ -84,3 +84,26 @@ def test_pairs_equal_single_nodes(storage, shapes, lattices):
         for x, y in zip(a.get_state(), b.get_state()):
             assert x is None or np.array_equal(x, y)
     batch.close()
+
+
+# planes large enough for the warp-per-tile step (rows of even length), whole and ragged last tiles,
+# one chunk and many; in a batch with one odd row length every member runs the tiled form of one
+# node per thread: the same values
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("shape,lattices", [((1020, 1300, 1), (9, 5, 5)), ((1262, 1001, 1), (5, 9, 9)),
+                                            ((32, 40000, 1), (9, 9, 0)), ((3202, 3800, 1), (9, 5, 9)), ((150002, 9, 1), (9, 9, 5)),
+                                            ((1400002, 1, 1), (5, 5, 9))])
+def test_planes_equal_single_nodes(storage, shape, lattices):
+    p = dict(workloads.base_params(kappa=100.0))
+    shapes = [shape, (901, 900, 1)]
+    batch = lbpf.Batch.create(shapes, lattices, [lbpf.make_params(storage, **p) for _ in shapes])
+    alone = lbpf.Sim(shape, lattices, storage=storage, **p)
+    c = np.array([[0.0, 0.0, 0.0], [0.7 * shape[0], 0.6 * shape[1], 0.0]])
+    for s in (batch.sims[0], alone):
+        s.init_seed(c, np.array([9.0, 12.0]), -0.55, -0.3)
+    batch.sims[1].init_seed(c[:1], np.array([9.0]), -0.55, -0.3)
+    batch.step(7)
+    alone.step(7)
+    for x, y in zip(batch.sims[0].read_fields(), alone.read_fields()):
+        assert np.isfinite(x).all() and np.array_equal(x, y)
+    batch.close()

@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_MOM
     k_phi_moment2(const SimDev* __restrict__ sims, const WorkItem* __restrict__ items, int s6) {
   using C = Codec<S>;
   constexpr bool HY = Lat<QP>::has_y;
-  const WorkItem it = items[blockIdx.x];
+  const WorkItem it = items[moment_block()];
   const SimDev& sd = sims[it.sim];
   const PairAt<HY> at(sd, it);
   pdl_trigger();
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_MOM
   using C = Codec<S>;
   constexpr int QTL = QT > 0 ? QT : 7;
   constexpr bool HY = Lat<QU>::has_y;
-  const WorkItem it = items[blockIdx.x];
+  const WorkItem it = items[moment_block()];
   const SimDev& sd = sims[it.sim];
   const PairAt<HY> at(sd, it);
   pdl_trigger();

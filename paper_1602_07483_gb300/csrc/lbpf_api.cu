@@ -573,6 +573,7 @@ void fill_dev(lbpf_sim* s) {
 
 int upload_dev(lbpf_sim* s) {
   fill_dev(s);
+  CK(s, cudaStreamSynchronize(s->stream));  // steps in flight read the descriptor
   CK(s, cudaMemcpy(s->dd, &s->hd, sizeof(SimDev), cudaMemcpyHostToDevice));
   return LBPF_OK;
 }

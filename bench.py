@@ -291,7 +291,7 @@ def run_own(args):
             with open(tr_path) as f:
                 tr = json.load(f)
             ent = tr.get(dom[0])
-            if ent and ent.get("source_hash") == kernel_source_hash():
+            if ent and ent.get("source_hash") == kernel_source_hash() and ent["alg_bytes_per_launch"] == dom[1]:
                 traffic = ent["bytes_per_launch_full"]
         except Exception:
             traffic = None
@@ -359,6 +359,7 @@ def run_own(args):
                          "step_alg_GBps": step_alg, "step_frac": step_alg / hbm},
             "cpu_baseline": cpu,
             "e2e": e2e,
+            # one per phase; a node-wise phase is two kernels (collision, moments), counted here as one
             "gpu_launches": (1 if args.schedule == "one_launch" else 2) * args.steps,
             "clocks": clk,
             "developed": developed,
@@ -429,10 +430,11 @@ def run_variants(args, st):
         out[name] = {"grid": list(w.grid), "storage": storage, "GLUPS": glups, "ms_per_step": ms,
                      "phi_ms": phi_ms, "uth_ms": uth_ms, "alg_GBps": alg, "hbm_frac": alg / hbm}
         if name == "f64":
-            out[name]["fp64_GFLOPs"] = glups * 687  # FP64 operations per site-update counted by ncu (halo included)
+            # 261 FP64 operations per site-update, counted by ncu over a step of this case
+            out[name]["fp64_GFLOPs"] = glups * 261
             peak = fp64_peak_gflops(st)
             out[name]["fp64_peak_GFLOPs"] = peak
-            out[name]["fp64_frac"] = glups * 687 / peak
+            out[name]["fp64_frac"] = glups * 261 / peak
             out[name]["fp64_peak_source"] = "cuBLAS DGEMM 8192^3 through torch.matmul, CUDA events, this run"
         if name.startswith("dense"):
             out[name]["seeds"] = len(w.radii)

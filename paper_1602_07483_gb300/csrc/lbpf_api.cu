@@ -205,6 +205,15 @@ int default_zchunk(int nx, int ny, int nz, int by) {
   return (nz + chunks - 1) / chunks;
 }
 
+// Copies host data to the device after the work already in `st` (steps in flight read what it
+// replaces) and before the work enqueued on it next.  A plain cudaMemcpy orders neither: it runs on
+// the default stream, which a non-blocking stream does not wait for, and from pageable memory it
+// may return before the data has arrived.
+cudaError_t upload(void* dst, const void* src, size_t n, cudaStream_t st) {
+  const cudaError_t e = cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, st);
+  return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+}
+
 // The dynamic shared-memory limit is an attribute of the kernel, shared by every
 // simulation that launches it: raise it once to the device's opt-in maximum so
 // that no handle's tiling can lower it under another handle's launches.
@@ -248,9 +257,9 @@ void free_one_launch(OneLaunch& ol) {
   ol.sc = StepSched{};
 }
 
-// (Re)builds the one-launch schedule of `items` on the device.  Synchronous.
+// (Re)builds the one-launch schedule of `items` on the device, for steps on `st`.  Synchronous.
 int setup_one_launch(OneLaunch& ol, const std::vector<WorkItem>& items, const std::vector<TileGeom>& geo, int by,
-                     size_t smem, const void* fn, int device) {
+                     size_t smem, const void* fn, int device, cudaStream_t st) {
   free_one_launch(ol);
   if (!ol.h_err) {
     if (cudaHostAlloc(&ol.h_err, sizeof(int), cudaHostAllocMapped) != cudaSuccess) {
@@ -288,8 +297,8 @@ int setup_one_launch(OneLaunch& ol, const std::vector<WorkItem>& items, const st
     free_one_launch(ol);
     return LBPF_ENOMEM;
   }
-  if (cudaMemcpy(ol.d_items, items.data(), n * sizeof(WorkItem), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(ol.d_sched, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) {
+  if (upload(ol.d_items, items.data(), n * sizeof(WorkItem), st) != cudaSuccess ||
+      upload(ol.d_sched, all.data(), all.size() * sizeof(int), st) != cudaSuccess) {
     free_one_launch(ol);
     return LBPF_ECUDA;
   }
@@ -338,8 +347,8 @@ void plan_kernels(PhasePlan& p, int phase, const KernelTable& t, const lbpf_latt
   }
 }
 
-// Copies the work items to the device (replacing the phase's).
-int plan_items(PhasePlan& p, const std::vector<WorkItem>& items) {
+// Copies the work items to the device (replacing the phase's), for steps on `st`.
+int plan_items(PhasePlan& p, const std::vector<WorkItem>& items, cudaStream_t st) {
   if (p.items) cudaFree(p.items);
   p.items = nullptr;
   p.nitems = 0;
@@ -348,8 +357,7 @@ int plan_items(PhasePlan& p, const std::vector<WorkItem>& items) {
     p.items = nullptr;
     return LBPF_ENOMEM;
   }
-  if (cudaMemcpy(p.items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice) != cudaSuccess)
-    return LBPF_ECUDA;
+  if (upload(p.items, items.data(), items.size() * sizeof(WorkItem), st) != cudaSuccess) return LBPF_ECUDA;
   p.nitems = (int)items.size();
   return LBPF_OK;
 }
@@ -418,7 +426,7 @@ int apply_tiling(lbpf_sim* s, int by, int zchunk) {
     if ((int)p.smem > maxsm) return LBPF_EINVAL;
     items.clear();
     s->zchunk = phase_items(p, 0, k, zchunk, by, node_blocks(k.nx, k.ny, k.nz, p.span()), items);
-    const int rc0 = plan_items(p, items);
+    const int rc0 = plan_items(p, items, s->stream);
     if (rc0 != LBPF_OK) {
       if (rc0 == LBPF_ECUDA) s->sticky = rc0;
       return rc0;
@@ -434,7 +442,7 @@ int apply_tiling(lbpf_sim* s, int by, int zchunk) {
     const int rc = setup_one_launch(s->ol, items, {TileGeom{k.nx, k.ny, k.nz, tile_zc}}, by,
                                     step_smem_bytes(t, s->lat.q_phi, s->lat.q_u, s->lat.q_theta, by),
                                     t.step_fn[q_index(s->lat.q_phi)][q_index(s->lat.q_u)][qt_index(s->lat.q_theta)],
-                                    s->device);
+                                    s->device, s->stream);
     if (rc != LBPF_OK) return rc;
   }
   const int rc = set_smem_attrs(t, s->lat, s->device);
@@ -573,8 +581,7 @@ void fill_dev(lbpf_sim* s) {
 
 int upload_dev(lbpf_sim* s) {
   fill_dev(s);
-  CK(s, cudaStreamSynchronize(s->stream));  // steps in flight read the descriptor
-  CK(s, cudaMemcpy(s->dd, &s->hd, sizeof(SimDev), cudaMemcpyHostToDevice));
+  CK(s, upload(s->dd, &s->hd, sizeof(SimDev), s->stream));
   return LBPF_OK;
 }
 
@@ -715,7 +722,7 @@ int lbpf_init_seed(lbpf_sim* s, int32_t n, const double* centres, const double* 
   std::vector<double> cen(centres, centres + 3 * n);
   if (lattice_is_2d(s->lat.q_phi))  // kernel coordinates (x, z, y)
     for (int m = 0; m < n; ++m) std::swap(cen[3 * m + 1], cen[3 * m + 2]);
-  CK(s, cudaMemcpy(d_seed, cen.data(), sizeof(double) * 3 * n, cudaMemcpyHostToDevice));
+  CK(s, cudaMemcpyAsync(d_seed, cen.data(), sizeof(double) * 3 * n, cudaMemcpyHostToDevice, s->stream));
   CK(s, cudaMemcpyAsync(d_seed + 3 * n, radii, sizeof(double) * n, cudaMemcpyHostToDevice, s->stream));
   const double c = s->p.dx / (sqrt(2.0) * s->p.W0);
   // phi of the seeds into level 1 (scratch), populations at buffer 0, moments at level 0,
@@ -1280,7 +1287,7 @@ static int batch_tiling(lbpf_batch* b, int by, int zchunk) {
       phase_items(p, (int)i, k, zchunk > 0 ? std::min(zchunk, k.nz) : 0, by, blocks, items);
     }
     std::stable_sort(items.begin(), items.end(), by_chunk);
-    if (plan_items(p, items) != LBPF_OK) return LBPF_ENOMEM;
+    if (plan_items(p, items, b->stream) != LBPF_OK) return LBPF_ENOMEM;
   }
   if (b->ol.on) {
     for (size_t i = 0; i < b->sims.size(); ++i) {
@@ -1299,7 +1306,7 @@ static int batch_tiling(lbpf_batch* b, int by, int zchunk) {
   if (b->ol.on) {
     const int rc = setup_one_launch(b->ol, ol_items, geo, by, step_smem_bytes(t, l.q_phi, l.q_u, l.q_theta, by),
                                     t.step_fn[q_index(l.q_phi)][q_index(l.q_u)][qt_index(l.q_theta)],
-                                    b->sims[0]->device);
+                                    b->sims[0]->device, b->stream);
     if (rc != LBPF_OK) return rc;
     for (lbpf_sim* s : b->sims) s->batch_err = b->ol.h_err;
   }
@@ -1328,7 +1335,7 @@ int batch_init(lbpf_batch* b) {
       memcpy(&b->h_desc[i], &b->sims[i]->hd, sizeof(SimDev));
     }
   }
-  ok = ok && cudaMemcpy(b->dd, b->h_desc, n * sizeof(SimDev), cudaMemcpyHostToDevice) == cudaSuccess;
+  ok = ok && upload(b->dd, b->h_desc, n * sizeof(SimDev), b->stream) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) == cudaSuccess;
   ok = ok && batch_tiling(b, lattice_is_2d(s0->lat.q_phi) ? 1 : MAX_BLOCK_ROWS, 0) == LBPF_OK;
   ok = ok && set_smem_attrs(t, s0->lat, s0->device) == LBPF_OK;

@@ -1,0 +1,80 @@
+"""The host side of the library (work lists, graphs, uploads) without a GPU.
+
+The compiled objects are linked against tests/fake_cudart.cpp in place of the CUDA runtime: every
+launch of a step kernel is checked to read live memory whose upload is ordered before it, and
+recorded, and allocations can be made to fail.
+"""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+from paper_1602_07483_gb300 import build, lbpf
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+class Fake:
+    def __init__(self, lib):
+        self.lib = lib
+        lib.fake_launch.restype = lib.fake_violation.restype = ctypes.c_char_p
+
+    def clear(self):
+        self.lib.fake_clear()
+
+    def fail_malloc(self, after, count=1):
+        self.lib.fake_fail_malloc(after, count)
+
+    def violations(self):
+        return [self.lib.fake_violation(i).decode() for i in range(self.lib.fake_violations())]
+
+    def launches(self):
+        """(kernel, blocks, threads, planes of the first and of the longest work item)"""
+        return [self.lib.fake_launch(i).decode() for i in range(self.lib.fake_launches())]
+
+
+@pytest.fixture(scope="module")
+def fake_path(tmp_path_factory):
+    build.build()
+    out = str(tmp_path_factory.mktemp("fake") / "liblbpf_fake.so")
+    objs = [os.path.join(build.OUT_DIR, "obj", s.replace(".cu", ".o")) for s in build.SOURCES]
+    subprocess.run([build.nvcc(), "-std=c++17", "-shared", "-cudart", "none", "-Xcompiler", "-fPIC,-Wall", "-Xlinker",
+                    "-Bsymbolic", "-o", out, os.path.join(HERE, "fake_cudart.cpp")] + objs, check=True)
+    return out
+
+
+@pytest.fixture
+def fake(fake_path, monkeypatch):
+    monkeypatch.setattr(lbpf, "_LIB", None)
+    f = Fake(lbpf.load(fake_path))
+    f.fail_malloc(-1, 0)
+    f.clear()
+    yield f
+    f.fail_malloc(-1, 0)
+
+
+# 3D and 2D, node-wise and tiled forms
+SIMS = [((32, 32, 32), (15, 19, 0), "f64"), ((33, 20, 18), (19, 19, 7), "f32"), ((202, 202, 202), (19, 19, 19), "f32"),
+        ((64, 48, 1), (9, 5, 5), "f16"), ((1600, 1500, 1), (9, 5, 5), "bf16")]
+
+
+@pytest.mark.parametrize("shape,lattices,storage", SIMS)
+@pytest.mark.parametrize("schedule", ["two_kernels", "one_launch"])
+def test_uploads_are_ordered_before_the_steps(fake, shape, lattices, storage, schedule):
+    s = lbpf.Sim(shape, lattices, storage=storage)
+    if schedule == "one_launch":
+        try:
+            s.set_schedule(schedule)
+        except lbpf.LbpfError:
+            pytest.skip("no one-launch step for these lattices and storage")
+    s.step(7)
+    s.set_tiling(4, 5)
+    s.step(7)
+    b = lbpf.Batch([s])
+    b.step(7)
+    b.set_tiling(6, 4)
+    b.step(7)
+    assert len(fake.launches()) >= 28
+    assert fake.violations() == []
+    b.close()

@@ -175,7 +175,7 @@ int lbpf_load(lbpf_sim* sim, const char* path);
  * and small 2D grids where that is faster) use blocks of 16 x by threads over
  * consecutive nodes of a plane.  Results do not depend on the tiling.  0 keeps
  * the current value.  Takes effect at the next lbpf_step (the step graph is
- * re-captured). */
+ * re-captured).  LBPF_ENOMEM, tiling unchanged, when its work lists do not fit. */
 int lbpf_set_tiling(lbpf_sim* sim, int32_t by, int32_t zchunk);
 int lbpf_get_tiling(const lbpf_sim* sim, int32_t* by, int32_t* zchunk);
 

@@ -257,18 +257,32 @@ void free_one_launch(OneLaunch& ol) {
   ol.sc = StepSched{};
 }
 
-// (Re)builds the one-launch schedule of `items` on the device, for steps on `st`.  Synchronous.
+// A one-launch schedule like `ol` (kernel, selection, wait flag and bound) that holds no buffers yet.
+OneLaunch without_buffers(const OneLaunch& ol) {
+  OneLaunch o = ol;
+  o.d_items = nullptr;
+  o.d_sched = nullptr;
+  o.d_ctl = nullptr;
+  o.sc = StepSched{};
+  return o;
+}
+
+// The host-visible flag of failed waits; lives as long as its handle or batch.
+int ensure_wait_flag(OneLaunch& ol) {
+  if (ol.h_err) return LBPF_OK;
+  if (cudaHostAlloc(&ol.h_err, sizeof(int), cudaHostAllocMapped) != cudaSuccess) {
+    cudaGetLastError();
+    ol.h_err = nullptr;
+    return LBPF_ENOMEM;
+  }
+  *ol.h_err = 0;
+  return LBPF_OK;
+}
+
+// Builds the one-launch schedule of `items` on the device, for steps on `st`, in `ol` (which holds no
+// buffers; on failure it is left so).  Synchronous.
 int setup_one_launch(OneLaunch& ol, const std::vector<WorkItem>& items, const std::vector<TileGeom>& geo, int by,
                      size_t smem, const void* fn, int device, cudaStream_t st) {
-  free_one_launch(ol);
-  if (!ol.h_err) {
-    if (cudaHostAlloc(&ol.h_err, sizeof(int), cudaHostAllocMapped) != cudaSuccess) {
-      cudaGetLastError();
-      ol.h_err = nullptr;
-      return LBPF_ENOMEM;
-    }
-    *ol.h_err = 0;
-  }
   int* d_err = nullptr;
   if (cudaHostGetDevicePointer((void**)&d_err, ol.h_err, 0) != cudaSuccess) return LBPF_ECUDA;
   int nb = 0, sms = 0;
@@ -347,11 +361,8 @@ void plan_kernels(PhasePlan& p, int phase, const KernelTable& t, const lbpf_latt
   }
 }
 
-// Copies the work items to the device (replacing the phase's), for steps on `st`.
+// Copies the work items of a new plan to the device, for steps on `st`.
 int plan_items(PhasePlan& p, const std::vector<WorkItem>& items, cudaStream_t st) {
-  if (p.items) cudaFree(p.items);
-  p.items = nullptr;
-  p.nitems = 0;
   if (cudaMalloc(&p.items, items.size() * sizeof(WorkItem)) != cudaSuccess) {
     cudaGetLastError();
     p.items = nullptr;
@@ -365,6 +376,20 @@ int plan_items(PhasePlan& p, const std::vector<WorkItem>& items, cudaStream_t st
 void free_plan(StepPlan& p) {
   for (PhasePlan& f : p.phase)
     if (f.items) cudaFree(f.items);
+}
+
+// Makes a complete new plan the one in use.  The step graph goes first: its kernels read the lists
+// that are freed here.  Until this call a handle or batch keeps stepping by its old plan, which
+// stays whole when the new one cannot be built.
+void adopt_plan(StepPlan& cur, OneLaunch& cur_ol, cudaGraphExec_t& gexec, bool& graph_ok, const StepPlan& plan,
+                const OneLaunch& ol) {
+  if (gexec) cudaGraphExecDestroy(gexec);
+  gexec = nullptr;
+  graph_ok = false;
+  free_plan(cur);
+  cur = plan;
+  free_one_launch(cur_ol);
+  cur_ol = ol;
 }
 
 // Whether a step can take two nodes per thread: rows of even length, so that every pair lies in one
@@ -409,45 +434,56 @@ int phase_items(const PhasePlan& p, int sim, const lbpf_grid& k, int zchunk, int
   return zc;
 }
 
-int apply_tiling(lbpf_sim* s, int by, int zchunk) {
+// The plan of `s` for blocks of `by` rows and z-chunks of `zchunk` planes (0: the defaults), in `plan`
+// and, for the one-launch schedule, `ol`; `zc` becomes the z-chunk to report.
+int build_tiling(lbpf_sim* s, int by, int zchunk, StepPlan& plan, OneLaunch& ol, int& zc) {
   const KernelTable& t = *s->kt;
-  if (lattice_is_2d(s->lat.q_phi)) by = 1;  // 2D: one-row blocks, no y halo
-  s->by = by;
-  s->zreq = zchunk;
-  s->plan.dd = s->dd;
   const lbpf_grid& k = s->kg;
-  const int tile_zc = zchunk > 0 ? zchunk : default_zchunk(k.nx, k.ny, k.nz, by);
+  int maxsm = 0;
+  if (cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, s->device) != cudaSuccess ||
+      set_smem_attrs(t, s->lat, s->device) != LBPF_OK)
+    return LBPF_ECUDA;
+  plan.dd = s->dd;
   std::vector<WorkItem> items;
   for (int f = 1; f >= 0; --f) {
-    PhasePlan& p = s->plan.phase[f];
+    PhasePlan& p = plan.phase[f];
     plan_kernels(p, f, t, s->lat, by, choose_form(f, t, s->lat, s->nsite, takes_pairs(t, k)));
-    int maxsm = 0;
-    CK(s, cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, s->device));
     if ((int)p.smem > maxsm) return LBPF_EINVAL;
     items.clear();
-    s->zchunk = phase_items(p, 0, k, zchunk, by, node_blocks(k.nx, k.ny, k.nz, p.span()), items);
-    const int rc0 = plan_items(p, items, s->stream);
-    if (rc0 != LBPF_OK) {
-      if (rc0 == LBPF_ECUDA) s->sticky = rc0;
-      return rc0;
-    }
-  }
-  if (s->gexec) cudaGraphExecDestroy(s->gexec);
-  s->gexec = nullptr;
-  s->graph_ok = false;
-  if (s->ol.on) {
-    s->zchunk = tile_zc;
-    items.clear();
-    build_items(0, k.nx, k.ny, k.nz, by, tile_zc, items);
-    const int rc = setup_one_launch(s->ol, items, {TileGeom{k.nx, k.ny, k.nz, tile_zc}}, by,
-                                    step_smem_bytes(t, s->lat.q_phi, s->lat.q_u, s->lat.q_theta, by),
-                                    t.step_fn[q_index(s->lat.q_phi)][q_index(s->lat.q_u)][qt_index(s->lat.q_theta)],
-                                    s->device, s->stream);
+    zc = phase_items(p, 0, k, zchunk, by, node_blocks(k.nx, k.ny, k.nz, p.span()), items);
+    const int rc = plan_items(p, items, s->stream);
     if (rc != LBPF_OK) return rc;
   }
-  const int rc = set_smem_attrs(t, s->lat, s->device);
-  if (rc != LBPF_OK) s->sticky = rc;
-  return rc;
+  if (!ol.on) return LBPF_OK;
+  zc = zchunk > 0 ? zchunk : default_zchunk(k.nx, k.ny, k.nz, by);
+  items.clear();
+  build_items(0, k.nx, k.ny, k.nz, by, zc, items);
+  return setup_one_launch(ol, items, {TileGeom{k.nx, k.ny, k.nz, zc}}, by,
+                          step_smem_bytes(t, s->lat.q_phi, s->lat.q_u, s->lat.q_theta, by),
+                          t.step_fn[q_index(s->lat.q_phi)][q_index(s->lat.q_u)][qt_index(s->lat.q_theta)], s->device,
+                          s->stream);
+}
+
+// Steps `s` by a new tiling under the schedule `one_launch`; on failure everything stays as it was.
+int apply_tiling(lbpf_sim* s, int by, int zchunk, bool one_launch) {
+  if (lattice_is_2d(s->lat.q_phi)) by = 1;  // 2D: one-row blocks, no y halo
+  if (one_launch && ensure_wait_flag(s->ol) != LBPF_OK) return LBPF_ENOMEM;
+  StepPlan plan;
+  OneLaunch ol = without_buffers(s->ol);
+  ol.on = one_launch;
+  int zc = 0;
+  const int rc = build_tiling(s, by, zchunk, plan, ol, zc);
+  if (rc != LBPF_OK) {
+    free_plan(plan);
+    free_one_launch(ol);
+    if (rc == LBPF_ECUDA) s->sticky = rc;
+    return rc;
+  }
+  adopt_plan(s->plan, s->ol, s->gexec, s->graph_ok, plan, ol);
+  s->by = by;
+  s->zreq = zchunk;
+  s->zchunk = zc;
+  return LBPF_OK;
 }
 
 // The kernels of a phase.
@@ -687,7 +723,7 @@ int lbpf_create(const lbpf_grid* grid, const lbpf_lattice* lattice, const lbpf_p
   s->ol.fn = s->kt->step[q_index(lattice->q_phi)][q_index(lattice->q_u)][qt_index(lattice->q_theta)];
   // 32 x 8 blocks: two resident blocks per SM at 128 registers per thread
   const int by = lattice_is_2d(lattice->q_phi) ? 1 : std::min(8, std::max(4, grid->ny + 2));
-  if ((rc = upload_dev(s)) != LBPF_OK || (rc = apply_tiling(s, by, 0)) != LBPF_OK) {
+  if ((rc = upload_dev(s)) != LBPF_OK || (rc = apply_tiling(s, by, 0, false)) != LBPF_OK) {
     free_sim(s);
     return rc;
   }
@@ -1002,7 +1038,7 @@ int lbpf_set_tiling(lbpf_sim* s, int32_t by, int32_t zchunk) {
   if (!s || by < 0 || zchunk < 0 || (by && (by < 4 || by > MAX_BLOCK_ROWS))) return LBPF_EINVAL;
   if (status(s)) return s->sticky;
   CK(s, cudaStreamSynchronize(s->stream));
-  return apply_tiling(s, by ? by : s->by, zchunk ? zchunk : (by ? 0 : s->zreq));
+  return apply_tiling(s, by ? by : s->by, zchunk ? zchunk : (by ? 0 : s->zreq), s->ol.on);
 }
 
 int lbpf_get_tiling(const lbpf_sim* s, int32_t* by, int32_t* zchunk) {
@@ -1017,17 +1053,7 @@ int lbpf_set_schedule(lbpf_sim* s, int32_t schedule) {
   if (status(s)) return s->sticky;
   if (schedule == LBPF_SCHED_ONE_LAUNCH && !s->ol.fn) return LBPF_EINVAL;
   CK(s, cudaStreamSynchronize(s->stream));
-  const bool was = s->ol.on;
-  s->ol.on = schedule == LBPF_SCHED_ONE_LAUNCH;
-  const int zreq = s->zreq;
-  const int rc = apply_tiling(s, s->by, zreq);
-  if (rc != LBPF_OK) {
-    s->ol.on = was;
-    free_one_launch(s->ol);
-    apply_tiling(s, s->by, zreq);
-  }
-  if (!s->ol.on) free_one_launch(s->ol);
-  return rc;
+  return apply_tiling(s, s->by, s->zreq, schedule == LBPF_SCHED_ONE_LAUNCH);
 }
 
 int lbpf_set_wait_polls(lbpf_sim* s, int32_t polls) {
@@ -1153,7 +1179,7 @@ int lbpf_autotune(lbpf_sim* s, int32_t steps, double* best_ms) {
     const int zcs[] = {zdef, std::max(node ? 1 : 8, zdef / 2), std::min(k.nz, zdef * 2),
                        node ? std::min(k.nz, zdef * 4) : k.nz};
     for (int zc : zcs) {
-      if (apply_tiling(s, by, zc) != LBPF_OK) { s->sticky = LBPF_OK; continue; }
+      if (apply_tiling(s, by, zc, s->ol.on) != LBPF_OK) { s->sticky = LBPF_OK; continue; }
       int rc = lbpf_step(s, 1);  // warm-up
       CK(s, cudaEventRecord(e0, s->stream));
       if (rc == LBPF_OK) rc = lbpf_step(s, steps);
@@ -1178,7 +1204,7 @@ int lbpf_autotune(lbpf_sim* s, int32_t steps, double* best_ms) {
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   free_all(snap);
-  int rc = apply_tiling(s, bbest, zbest);
+  int rc = apply_tiling(s, bbest, zbest, s->ol.on);
   if (best_ms) *best_ms = best;
   return rc;
 }
@@ -1260,13 +1286,12 @@ int lbpf_load(lbpf_sim* s, const char* path) {
 
 // ---------------------------------------------------------------- batch
 
-// Work items of all member simulations for blocks of `by` rows and z-chunks of
-// `zchunk` planes (0: each simulation's default), large chunks first.
-static int batch_tiling(lbpf_batch* b, int by, int zchunk) {
+// The plan of all member simulations for blocks of `by` rows and z-chunks of `zchunk` planes (0: each
+// simulation's default), large chunks first, in `plan` and, for the one-launch schedule, `ol`.
+static int build_batch_tiling(lbpf_batch* b, int by, int zchunk, StepPlan& plan, OneLaunch& ol) {
   const KernelTable& t = *b->sims[0]->kt;
   const lbpf_lattice& l = b->sims[0]->lat;
-  std::vector<WorkItem> items, ol_items;
-  std::vector<TileGeom> geo;
+  std::vector<WorkItem> items;
   long long sites = 0;
   bool pairs = true;
   for (const lbpf_sim* s : b->sims) {
@@ -1275,9 +1300,9 @@ static int batch_tiling(lbpf_batch* b, int by, int zchunk) {
   }
   // large chunks first, so that large and small simulations interleave
   auto by_chunk = [](const WorkItem& a, const WorkItem& c) { return (a.z1 - a.z0) > (c.z1 - c.z0); };
-  b->plan.dd = b->dd;
+  plan.dd = b->dd;
   for (int f = 0; f < 2; ++f) {
-    PhasePlan& p = b->plan.phase[f];
+    PhasePlan& p = plan.phase[f];
     plan_kernels(p, f, t, l, by, choose_form(f, t, l, sites, pairs));
     long long blocks = 0;  // of one plane each, over all members
     for (const lbpf_sim* s : b->sims) blocks += node_blocks(s->kg.nx, s->kg.ny, s->kg.nz, p.span());
@@ -1289,27 +1314,38 @@ static int batch_tiling(lbpf_batch* b, int by, int zchunk) {
     std::stable_sort(items.begin(), items.end(), by_chunk);
     if (plan_items(p, items, b->stream) != LBPF_OK) return LBPF_ENOMEM;
   }
-  if (b->ol.on) {
-    for (size_t i = 0; i < b->sims.size(); ++i) {
-      const lbpf_grid& k = b->sims[i]->kg;
-      const int zc = zchunk > 0 ? std::min(zchunk, k.nz) : default_zchunk(k.nx, k.ny, k.nz, by);
-      build_items((int)i, k.nx, k.ny, k.nz, by, zc, ol_items);
-      geo.push_back(TileGeom{k.nx, k.ny, k.nz, zc});
-    }
-    std::stable_sort(ol_items.begin(), ol_items.end(), by_chunk);
+  if (!ol.on) return LBPF_OK;
+  std::vector<TileGeom> geo;
+  items.clear();
+  for (size_t i = 0; i < b->sims.size(); ++i) {
+    const lbpf_grid& k = b->sims[i]->kg;
+    const int zc = zchunk > 0 ? std::min(zchunk, k.nz) : default_zchunk(k.nx, k.ny, k.nz, by);
+    build_items((int)i, k.nx, k.ny, k.nz, by, zc, items);
+    geo.push_back(TileGeom{k.nx, k.ny, k.nz, zc});
   }
+  std::stable_sort(items.begin(), items.end(), by_chunk);
+  return setup_one_launch(ol, items, geo, by, step_smem_bytes(t, l.q_phi, l.q_u, l.q_theta, by),
+                          t.step_fn[q_index(l.q_phi)][q_index(l.q_u)][qt_index(l.q_theta)], b->sims[0]->device,
+                          b->stream);
+}
+
+// Steps the batch by a new tiling under the schedule `one_launch`; on failure everything stays as it was.
+static int batch_tiling(lbpf_batch* b, int by, int zchunk, bool one_launch) {
+  if (one_launch && ensure_wait_flag(b->ol) != LBPF_OK) return LBPF_ENOMEM;
+  StepPlan plan;
+  OneLaunch ol = without_buffers(b->ol);
+  ol.on = one_launch;
+  const int rc = build_batch_tiling(b, by, zchunk, plan, ol);
+  if (rc != LBPF_OK) {
+    free_plan(plan);
+    free_one_launch(ol);
+    return rc;
+  }
+  adopt_plan(b->plan, b->ol, b->gexec, b->graph_ok, plan, ol);
   b->by = by;
   b->zchunk = zchunk;
-  if (b->gexec) cudaGraphExecDestroy(b->gexec);
-  b->gexec = nullptr;
-  b->graph_ok = false;
-  if (b->ol.on) {
-    const int rc = setup_one_launch(b->ol, ol_items, geo, by, step_smem_bytes(t, l.q_phi, l.q_u, l.q_theta, by),
-                                    t.step_fn[q_index(l.q_phi)][q_index(l.q_u)][qt_index(l.q_theta)],
-                                    b->sims[0]->device, b->stream);
-    if (rc != LBPF_OK) return rc;
+  if (one_launch)
     for (lbpf_sim* s : b->sims) s->batch_err = b->ol.h_err;
-  }
   return LBPF_OK;
 }
 
@@ -1337,7 +1373,7 @@ int batch_init(lbpf_batch* b) {
   }
   ok = ok && upload(b->dd, b->h_desc, n * sizeof(SimDev), b->stream) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) == cudaSuccess;
-  ok = ok && batch_tiling(b, lattice_is_2d(s0->lat.q_phi) ? 1 : MAX_BLOCK_ROWS, 0) == LBPF_OK;
+  ok = ok && batch_tiling(b, lattice_is_2d(s0->lat.q_phi) ? 1 : MAX_BLOCK_ROWS, 0, false) == LBPF_OK;
   ok = ok && set_smem_attrs(t, s0->lat, s0->device) == LBPF_OK;
   if (!ok) {
     cudaGetLastError();
@@ -1469,7 +1505,7 @@ int lbpf_batch_set_tiling(lbpf_batch* b, int32_t by, int32_t zchunk) {
     if (status(s)) return s->sticky;
   if (cudaStreamSynchronize(b->stream) != cudaSuccess) return LBPF_ECUDA;
   if (lattice_is_2d(b->sims[0]->lat.q_phi)) by = 1;  // 2D: one-row blocks
-  return batch_tiling(b, by ? by : b->by, zchunk);
+  return batch_tiling(b, by ? by : b->by, zchunk, b->ol.on);
 }
 
 int lbpf_batch_set_schedule(lbpf_batch* b, int32_t schedule) {
@@ -1478,16 +1514,7 @@ int lbpf_batch_set_schedule(lbpf_batch* b, int32_t schedule) {
     if (status(s)) return s->sticky;
   if (schedule == LBPF_SCHED_ONE_LAUNCH && !b->ol.fn) return LBPF_EINVAL;
   if (cudaStreamSynchronize(b->stream) != cudaSuccess) return LBPF_ECUDA;
-  const bool was = b->ol.on;
-  b->ol.on = schedule == LBPF_SCHED_ONE_LAUNCH;
-  const int rc = batch_tiling(b, b->by, b->zchunk);
-  if (rc != LBPF_OK) {
-    b->ol.on = was;
-    free_one_launch(b->ol);
-    batch_tiling(b, b->by, b->zchunk);
-  }
-  if (!b->ol.on) free_one_launch(b->ol);
-  return rc;
+  return batch_tiling(b, b->by, b->zchunk, schedule == LBPF_SCHED_ONE_LAUNCH);
 }
 
 int lbpf_batch_get_schedule(const lbpf_batch* b, int32_t* schedule) {
@@ -1539,7 +1566,7 @@ int lbpf_batch_autotune(lbpf_batch* b, int32_t steps, double* best_ms) {
   double best = 1e300;
   int bbest = by0, zbest = zc0;
   for (size_t c = 0; c < cand.size() && ok; ++c) {
-    if (batch_tiling(b, cand[c].first, cand[c].second) != LBPF_OK) continue;
+    if (batch_tiling(b, cand[c].first, cand[c].second, b->ol.on) != LBPF_OK) continue;
     rc = lbpf_batch_step(b, align + kGraphSteps);
     ok = cudaEventRecord(e0, b->stream) == cudaSuccess;
     if (rc == LBPF_OK && ok) rc = lbpf_batch_step(b, timed);
@@ -1562,7 +1589,7 @@ int lbpf_batch_autotune(lbpf_batch* b, int32_t steps, double* best_ms) {
     for (lbpf_sim* s : b->sims) s->sticky = LBPF_ECUDA;
     return LBPF_ECUDA;
   }
-  rc = batch_tiling(b, bbest, zbest);
+  rc = batch_tiling(b, bbest, zbest, b->ol.on);
   if (best_ms) *best_ms = best;
   return rc;
 }

@@ -216,7 +216,8 @@ cudaError_t cudaMemcpyAsync(void* dst, const void* src, size_t n, cudaMemcpyKind
   return cudaSuccess;
 }
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) {
-  if (n < kCopied) memset(p, v, n);
+  if (live_bytes(p) < n) g_bad.push_back("a memset of what is not allocated");
+  else if (n < kCopied) memset(p, v, n);
   return cudaSuccess;
 }
 cudaError_t cudaGetSymbolAddress(void** p, const void*) {

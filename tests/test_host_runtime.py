@@ -78,3 +78,53 @@ def test_uploads_are_ordered_before_the_steps(fake, shape, lattices, storage, sc
     assert len(fake.launches()) >= 28
     assert fake.violations() == []
     b.close()
+
+
+@pytest.mark.parametrize("shape,lattices,storage", SIMS)
+@pytest.mark.parametrize("batched", [False, True])
+@pytest.mark.parametrize("schedule", ["two_kernels", "one_launch"])
+def test_a_failed_tiling_keeps_the_old_one(fake, shape, lattices, storage, batched, schedule):
+    """Whichever allocation fails, the call reports it and the steps run on as planned before."""
+    s = lbpf.Sim(shape, lattices, storage=storage)
+    s = lbpf.Batch([s]) if batched else s
+    if schedule == "one_launch":
+        try:
+            s.set_schedule(schedule)
+        except lbpf.LbpfError:
+            pytest.skip("no one-launch step for these lattices and storage")
+
+    def steps():
+        fake.clear()
+        s.step(6)  # a graph
+        s.step(5)
+        s.step(1)
+        assert fake.violations() == []
+        return fake.launches()
+
+    def fails(call):
+        """Runs the call with its first, second, ... allocation failing until it succeeds."""
+        for after in range(20):
+            fake.fail_malloc(after)
+            try:
+                call()
+            except lbpf.LbpfError as e:
+                if e.code == lbpf.LBPF_EINVAL:  # no one-launch step for these lattices and storage
+                    return 2
+                assert e.code == lbpf.LBPF_ENOMEM
+            else:
+                fake.fail_malloc(-1, 0)
+                return after
+            fake.fail_malloc(-1, 0)
+            assert steps() == before
+            assert s.schedule == schedule
+            if not batched:
+                assert s.get_tiling() == tiling
+        raise AssertionError("never succeeded")
+
+    before, tiling = steps(), s.get_tiling()
+    assert fails(lambda: s.set_tiling(4, 5)) >= 2
+    before, tiling = steps(), s.get_tiling()
+    assert fails(lambda: s.set_schedule("one_launch" if schedule == "two_kernels" else "two_kernels")) >= 2
+    fake.fail_malloc(-1, 0)
+    steps()
+    s.close()

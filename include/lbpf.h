@@ -173,14 +173,15 @@ int lbpf_load(lbpf_sim* sim, const char* path);
  * (>= 1; the z range is split into chunks processed by separate thread
  * blocks).  Steps that run node-wise (FP64, FP16 and BF16 on 3D lattices, FP32
  * and small 2D grids where that is faster) use blocks of 16 x by threads over
- * consecutive nodes of a plane.  Results do not depend on the tiling.  0 keeps
+ * consecutive nodes of a plane; where only one phase of a step does, `zchunk` is
+ * the other's (the tiles').  Results do not depend on the tiling.  0 keeps
  * the current value.  Takes effect at the next lbpf_step (the step graph is
  * re-captured).  LBPF_ENOMEM, tiling unchanged, when its work lists do not fit. */
 int lbpf_set_tiling(lbpf_sim* sim, int32_t by, int32_t zchunk);
 int lbpf_get_tiling(const lbpf_sim* sim, int32_t* by, int32_t* zchunk);
 
-/* Autotuner: times `steps` steps for each candidate tiling on a snapshot of
- * the current state, keeps the fastest, and restores the state.  best_ms
+/* Autotuner: times `steps` steps for each candidate tiling (the current one among
+ * them) on a snapshot of the current state, keeps the fastest, and restores the state.  best_ms
  * (may be NULL) receives the best time per step.  Synchronous. */
 int lbpf_autotune(lbpf_sim* sim, int32_t steps, double* best_ms);
 

@@ -123,6 +123,12 @@ struct PhasePlan {
 struct StepPlan {
   PhasePlan phase[2];  // phi, then U and theta
   const SimDev* dd = nullptr;
+  // One phase tiled, the other node-wise.  A z-chunk asked for is then the tiles', whose halo planes
+  // it decides; the node-wise phase keeps its default (16 planes of phi against 32 of U and theta at
+  // 512^3 FP32, and no common chunk is as fast).
+  bool mixed() const { return phase[0].node_wise() != phase[1].node_wise(); }
+  bool takes_request(int f) const { return !mixed() || !phase[f].node_wise(); }
+  int reporting() const { return takes_request(0) ? 0 : 1; }  // the phase whose z-chunk is reported
 };
 
 struct lbpf_sim {
@@ -143,7 +149,7 @@ struct lbpf_sim {
   SimDev* dd = nullptr;
   StepPlan plan;
   int by = MAX_BLOCK_ROWS, zchunk = 0;  // tiling in effect
-  int zreq = 0;                         // z-chunk asked for (0: the default)
+  int zreq = 0;                         // z-chunk asked for (0: the defaults)
   double* d_part = nullptr;  // reduction partials + 4 results
   int npart = 0;
   double* d_small = nullptr; // tip output
@@ -445,12 +451,16 @@ int build_tiling(lbpf_sim* s, int by, int zchunk, StepPlan& plan, OneLaunch& ol,
     return LBPF_ECUDA;
   plan.dd = s->dd;
   std::vector<WorkItem> items;
-  for (int f = 1; f >= 0; --f) {
+  for (int f = 0; f < 2; ++f) {
+    plan_kernels(plan.phase[f], f, t, s->lat, by, choose_form(f, t, s->lat, s->nsite, takes_pairs(t, k)));
+    if ((int)plan.phase[f].smem > maxsm) return LBPF_EINVAL;
+  }
+  for (int f = 0; f < 2; ++f) {
     PhasePlan& p = plan.phase[f];
-    plan_kernels(p, f, t, s->lat, by, choose_form(f, t, s->lat, s->nsite, takes_pairs(t, k)));
-    if ((int)p.smem > maxsm) return LBPF_EINVAL;
     items.clear();
-    zc = phase_items(p, 0, k, zchunk, by, node_blocks(k.nx, k.ny, k.nz, p.span()), items);
+    const int used = phase_items(p, 0, k, plan.takes_request(f) ? zchunk : 0, by,
+                                 node_blocks(k.nx, k.ny, k.nz, p.span()), items);
+    if (f == plan.reporting()) zc = zchunk > 0 ? zchunk : used;
     const int rc = plan_items(p, items, s->stream);
     if (rc != LBPF_OK) return rc;
   }
@@ -1162,43 +1172,46 @@ int lbpf_autotune(lbpf_sim* s, int32_t steps, double* best_ms) {
     return src;
   }
   const int64_t steps0 = s->steps;
-  const int by0 = s->by, zc0 = s->zchunk;
+  const int by0 = s->by, zc0 = s->zreq;
+  // the tiling in use first (the default has no equal among the others where the phases' chunks
+  // differ), then chunks around the default of the phase that takes the request
+  std::vector<std::pair<int, int>> cand{{by0, zc0}};
+  const lbpf_grid& k = s->kg;
+  const PhasePlan& p0 = s->plan.phase[s->plan.reporting()];
+  const bool node = p0.node_wise() && !s->ol.on;
+  for (int by : {4, 6, 8}) {
+    if (by > k.ny + 2 && by != 4) continue;
+    const int span = node_threads(by0 == 1 ? 1 : by) * p0.nodes();
+    const int zdef = node ? node_zchunk(node_blocks(k.nx, k.ny, k.nz, span), k.nz)
+                          : default_zchunk(k.nx, k.ny, k.nz, by);
+    const int longest = node ? std::min(k.nz, zdef * 4) : k.nz;
+    for (int zc : {zdef, std::max(node ? 1 : 8, zdef / 2), std::min(k.nz, zdef * 2), longest}) cand.push_back({by, zc});
+  }
   cudaEvent_t e0, e1;
   CK(s, cudaEventCreate(&e0));
   CK(s, cudaEventCreate(&e1));
   double best = 1e300;
   int bbest = by0, zbest = zc0;
-  const int bys[] = {4, 6, 8};
-  for (int by : bys) {
-    if (by > s->kg.ny + 2 && by != bys[0]) continue;
-    const lbpf_grid& k = s->kg;
-    const PhasePlan& p0 = s->plan.phase[0];
-    const bool node = p0.node_wise() && !s->ol.on;
-    const int zdef = node ? node_zchunk(node_blocks(k.nx, k.ny, k.nz, node_threads(s->by == 1 ? 1 : by) * p0.nodes()), k.nz)
-                          : default_zchunk(k.nx, k.ny, k.nz, by);
-    const int zcs[] = {zdef, std::max(node ? 1 : 8, zdef / 2), std::min(k.nz, zdef * 2),
-                       node ? std::min(k.nz, zdef * 4) : k.nz};
-    for (int zc : zcs) {
-      if (apply_tiling(s, by, zc, s->ol.on) != LBPF_OK) { s->sticky = LBPF_OK; continue; }
-      int rc = lbpf_step(s, 1);  // warm-up
-      CK(s, cudaEventRecord(e0, s->stream));
-      if (rc == LBPF_OK) rc = lbpf_step(s, steps);
-      CK(s, cudaEventRecord(e1, s->stream));
-      CK(s, cudaEventSynchronize(e1));
-      float ms = 0;
-      CK(s, cudaEventElapsedTime(&ms, e0, e1));
-      if (rc == LBPF_OK && ms / steps < best) {
-        best = ms / steps;
-        bbest = by;
-        zbest = zc;
-      }
-      // back to the snapshot and the step counter (the parity the snapshot was taken at)
-      s->steps = steps0;
-      if (restore_state(live, snap, s->stream) != LBPF_OK || cudaStreamSynchronize(s->stream) != cudaSuccess) {
-        s->sticky = LBPF_ECUDA;
-        free_all(snap);
-        return LBPF_ECUDA;
-      }
+  for (const auto& c : cand) {
+    if (apply_tiling(s, c.first, c.second, s->ol.on) != LBPF_OK) { s->sticky = LBPF_OK; continue; }
+    int rc = lbpf_step(s, 1);  // warm-up
+    CK(s, cudaEventRecord(e0, s->stream));
+    if (rc == LBPF_OK) rc = lbpf_step(s, steps);
+    CK(s, cudaEventRecord(e1, s->stream));
+    CK(s, cudaEventSynchronize(e1));
+    float ms = 0;
+    CK(s, cudaEventElapsedTime(&ms, e0, e1));
+    if (rc == LBPF_OK && ms / steps < best) {
+      best = ms / steps;
+      bbest = c.first;
+      zbest = c.second;
+    }
+    // back to the snapshot and the step counter (the parity the snapshot was taken at)
+    s->steps = steps0;
+    if (restore_state(live, snap, s->stream) != LBPF_OK || cudaStreamSynchronize(s->stream) != cudaSuccess) {
+      s->sticky = LBPF_ECUDA;
+      free_all(snap);
+      return LBPF_ECUDA;
     }
   }
   cudaEventDestroy(e0);
@@ -1301,15 +1314,16 @@ static int build_batch_tiling(lbpf_batch* b, int by, int zchunk, StepPlan& plan,
   // large chunks first, so that large and small simulations interleave
   auto by_chunk = [](const WorkItem& a, const WorkItem& c) { return (a.z1 - a.z0) > (c.z1 - c.z0); };
   plan.dd = b->dd;
+  for (int f = 0; f < 2; ++f) plan_kernels(plan.phase[f], f, t, l, by, choose_form(f, t, l, sites, pairs));
   for (int f = 0; f < 2; ++f) {
     PhasePlan& p = plan.phase[f];
-    plan_kernels(p, f, t, l, by, choose_form(f, t, l, sites, pairs));
+    const int zreq = plan.takes_request(f) ? zchunk : 0;
     long long blocks = 0;  // of one plane each, over all members
     for (const lbpf_sim* s : b->sims) blocks += node_blocks(s->kg.nx, s->kg.ny, s->kg.nz, p.span());
     items.clear();
     for (size_t i = 0; i < b->sims.size(); ++i) {
       const lbpf_grid& k = b->sims[i]->kg;
-      phase_items(p, (int)i, k, zchunk > 0 ? std::min(zchunk, k.nz) : 0, by, blocks, items);
+      phase_items(p, (int)i, k, zreq > 0 ? std::min(zreq, k.nz) : 0, by, blocks, items);
     }
     std::stable_sort(items.begin(), items.end(), by_chunk);
     if (plan_items(p, items, b->stream) != LBPF_OK) return LBPF_ENOMEM;

@@ -128,3 +128,28 @@ def test_a_failed_tiling_keeps_the_old_one(fake, shape, lattices, storage, batch
     fake.fail_malloc(-1, 0)
     steps()
     s.close()
+
+
+@pytest.mark.parametrize("shape,lattices,storage", SIMS)
+def test_tuning_starts_from_the_tiling_in_use(fake, shape, lattices, storage):
+    """Setting the reported tiling changes nothing, and tuning never ends slower than it began:
+    phi of the 202^3 box runs node-wise and U and theta tiled, with chunks of their own."""
+    s = lbpf.Sim(shape, lattices, storage=storage)
+
+    def step():
+        fake.clear()
+        ms = s.step_timed(6)[2]
+        return fake.launches(), ms
+
+    launches, ms = step()
+    s.set_tiling(*((0, s.get_tiling()[1]) if shape[2] == 1 else s.get_tiling()))
+    assert step() == (launches, ms)
+    s.set_tiling(8, 0)
+    before, ms = step()
+    assert before == launches
+    s.autotune(6)
+    assert step()[1] <= ms
+    s.set_tiling(8, 1000)
+    assert s.get_tiling()[1] == 1000
+    s.set_schedule("two_kernels")
+    assert s.get_tiling()[1] == 1000

@@ -46,6 +46,11 @@ __host__ __device__ constexpr int class_rep(int c) {
   return c == 0 ? 0 : (c == 1 ? 1 : Lat<Q>::diag0);
 }
 
+// Which links a collision computes: all of them, or (the tiles' halo rows) those wanted(e_y).
+struct AllLinks {
+  __device__ __forceinline__ constexpr bool operator()(int) const { return true; }
+};
+
 // Coefficients of a node's collisions (FP32 and FP64 arithmetic have their own).
 template <typename T>
 struct PhiCoef;
@@ -178,8 +183,9 @@ __device__ __forceinline__ T eq_of(int i, T K, T ax, T ay, T az) {
 
 // Post-collision populations of the links wanted(e_y) in place of the pulled ones (in the
 // stored units, before the conversion to the storage type).
-template <int QP, typename W>
-__device__ __forceinline__ void phi_collide(const PhiCoef<float>& c, float (&gp)[QP], const float (&gn)[QP], W wanted) {
+template <int QP, typename W = AllLinks>
+__device__ __forceinline__ void phi_collide(const PhiCoef<float>& c, float (&gp)[QP], const float (&gn)[QP],
+                                            W wanted = W()) {
   using L = Lat<QP>;
   if (c.flat) {
 #pragma unroll
@@ -307,8 +313,8 @@ __device__ __forceinline__ void uth_coef(const Consts<float>& P, bool at_on, flo
   }
 }
 
-template <int QU, typename W>
-__device__ __forceinline__ void u_collide(const UthCoef<float>& c, float (&h)[QU], W wanted) {
+template <int QU, typename W = AllLinks>
+__device__ __forceinline__ void u_collide(const UthCoef<float>& c, float (&h)[QU], W wanted = W()) {
   using L = Lat<QU>;
 #pragma unroll
   for (int i = 0; i < QU; ++i) {
@@ -350,15 +356,15 @@ __device__ __forceinline__ bool has_gradient(const Consts<double>& P, double dx,
   return rmul(rfma(dx, dx, rfma(dy, dy, rmul(dz, dz))), P.inv2dx2) >= P.grad2_min;
 }
 
-template <int QP, typename S, bool BRANCH>
+template <int QP, typename S, bool BRANCH>  // FP64 steps node-wise only, and always branches
 __device__ __forceinline__ void phi_coef(const Consts<double>& P, double ph, double U, double th, double dx, double dy,
                                          double dz, bool wall, double, PhiCoef<double>& c) {
   using T = double;
   using L = Lat<QP>;
   const T omp2 = rfma(-ph, ph, T(1));
   const T Q = rmul(rmul(rfma(-rfma(P.lamM, U, rmul(P.lam, th)), omp2, ph), omp2), P.dt_tau0);
-  const bool flat = !has_gradient(P, dx, dy, dz);
-  c.flat = BRANCH && flat;
+  static_assert(BRANCH, "FP64 has no form without the branch");
+  c.flat = !has_gradient(P, dx, dy, dz);
   if (c.flat) {
     const T kk = rfma(P.inv_eta1, ph, Q);
     c.A = radd(T(1), -P.inv_eta1);
@@ -366,38 +372,33 @@ __device__ __forceinline__ void phi_coef(const Consts<double>& P, double ph, dou
     for (int k = 0; k < 3; ++k) c.K[k] = rmul((T)L::w(class_rep<QP>(k)), kk);
     return;
   }
-  T as = T(1), Nx = T(0), Ny = T(0), Nz = T(0);
-  if (BRANCH || !flat) {
-    // a_s(n) = a0 + a4 sum n^4 + a6 nx^2 ny^2 nz^2 covers Eq. (Anisotropic-Function_As) and
-    // Eq. (As_K41-K61); N = |grad phi|^2 a_s d a_s / d(grad phi) (Eq. TermesAnisotropes)
-    const T s2 = rfma(dx, dx, rfma(dy, dy, rmul(dz, dz)));
-    const T iG = rsq(s2);
-    const T nx = rmul(dx, iG), ny = rmul(dy, iG), nz = rmul(dz, iG);
-    const T x2 = rmul(nx, nx), y2 = rmul(ny, ny), z2 = rmul(nz, nz);
-    const T s4 = rfma(x2, x2, rfma(y2, y2, rmul(z2, z2)));
-    const T c4 = rmul(T(4), P.a4);
-    as = rfma(P.a4, s4, P.a0);
-    T px = rmul(c4, radd(x2, -s4)), py = rmul(c4, radd(y2, -s4)), pz = rmul(c4, radd(z2, -s4));
-    if (P.a6 != T(0)) {
-      const T yz = rmul(y2, z2), xz = rmul(x2, z2), xy = rmul(x2, y2);
-      const T c6 = rmul(T(2), P.a6);
-      as = rfma(P.a6, rmul(x2, yz), as);
-      px = rfma(rmul(c6, yz), rfma(T(-3), x2, T(1)), px);
-      py = rfma(rmul(c6, xz), rfma(T(-3), y2, T(1)), py);
-      pz = rfma(rmul(c6, xy), rfma(T(-3), z2, T(1)), pz);
-    }
-    const T f = rmul(rmul(rmul(s2, iG), P.inv2dx), as);  // |grad phi| a_s
-    Nx = rmul(f, rmul(nx, px));
-    Ny = rmul(f, rmul(ny, py));
-    Nz = rmul(f, rmul(nz, pz));
+  // a_s(n) = a0 + a4 sum n^4 + a6 nx^2 ny^2 nz^2 covers Eq. (Anisotropic-Function_As) and
+  // Eq. (As_K41-K61); N = |grad phi|^2 a_s d a_s / d(grad phi) (Eq. TermesAnisotropes)
+  const T s2 = rfma(dx, dx, rfma(dy, dy, rmul(dz, dz)));
+  const T iG = rsq(s2);
+  const T nx = rmul(dx, iG), ny = rmul(dy, iG), nz = rmul(dz, iG);
+  const T x2 = rmul(nx, nx), y2 = rmul(ny, ny), z2 = rmul(nz, nz);
+  const T s4 = rfma(x2, x2, rfma(y2, y2, rmul(z2, z2)));
+  const T c4 = rmul(T(4), P.a4);
+  T as = rfma(P.a4, s4, P.a0);
+  T px = rmul(c4, radd(x2, -s4)), py = rmul(c4, radd(y2, -s4)), pz = rmul(c4, radd(z2, -s4));
+  if (P.a6 != T(0)) {
+    const T yz = rmul(y2, z2), xz = rmul(x2, z2), xy = rmul(x2, y2);
+    const T c6 = rmul(T(2), P.a6);
+    as = rfma(P.a6, rmul(x2, yz), as);
+    px = rfma(rmul(c6, yz), rfma(T(-3), x2, T(1)), px);
+    py = rfma(rmul(c6, xz), rfma(T(-3), y2, T(1)), py);
+    pz = rfma(rmul(c6, xy), rfma(T(-3), z2, T(1)), pz);
   }
+  const T f = rmul(rmul(rmul(s2, iG), P.inv2dx), as);  // |grad phi| a_s
+  T Nx = rmul(f, rmul(nx, px));
+  T Ny = rmul(f, rmul(ny, py));
+  T Nz = rmul(f, rmul(nz, pz));
   const T as2 = rmul(as, as);
   const T eta = rfma(P.c_eta, as2, T(0.5));
   const T a2 = wall ? T(1) : as2;
   const T r = rcp(rmul(eta, as2));  // one division for both
-  T inv_eta = rmul(r, as2), inv_a2 = rmul(r, eta);
-  if (wall || flat) inv_a2 = T(1);
-  if (flat) inv_eta = P.inv_eta1;
+  const T inv_eta = rmul(r, as2), inv_a2 = wall ? T(1) : rmul(r, eta);
   const T oma2 = radd(T(1), -a2);
   const T kk = rmul(rfma(inv_eta, ph, Q), inv_a2);
   const T nn = -rmul(rmul(inv_eta, P.c_N), inv_a2);
@@ -416,25 +417,24 @@ __device__ __forceinline__ void phi_coef(const Consts<double>& P, double ph, dou
   }
 }
 
-template <int QP, typename W>
-__device__ __forceinline__ void phi_collide(const PhiCoef<double>& c, double (&gp)[QP], const double (&gn)[QP], W wanted) {
+template <int QP>
+__device__ __forceinline__ void phi_collide(const PhiCoef<double>& c, double (&gp)[QP], const double (&gn)[QP]) {
   using T = double;
   using L = Lat<QP>;
   if (c.flat) {
 #pragma unroll
-    for (int i = 0; i < QP; ++i)
-      if (wanted(L::ey(i))) gp[i] = rfma(c.A, gp[i], c.K[L::cls(i)]);
+    for (int i = 0; i < QP; ++i) gp[i] = rfma(c.A, gp[i], c.K[L::cls(i)]);
     return;
   }
-  if (wanted(0)) gp[0] = rfma(c.A, gp[0], rfma(c.B, gn[0], c.K[0]));
+  gp[0] = rfma(c.A, gp[0], rfma(c.B, gn[0], c.K[0]));
 #pragma unroll
   for (int i = 1; i < QP; ++i) {
     const int j = L::opp(i);
     if (j < i) continue;
     const int k = L::cls(i);
     const T d = along<L>(i, c.nx[k], c.ny[k], c.nz[k]);
-    if (wanted(L::ey(i))) gp[i] = rfma(c.A, gp[i], rfma(c.B, gn[i], radd(c.K[k], d)));
-    if (wanted(L::ey(j))) gp[j] = rfma(c.A, gp[j], rfma(c.B, gn[j], radd(c.K[k], -d)));
+    gp[i] = rfma(c.A, gp[i], rfma(c.B, gn[i], radd(c.K[k], d)));
+    gp[j] = rfma(c.A, gp[j], rfma(c.B, gn[j], radd(c.K[k], -d)));
   }
 }
 
@@ -560,25 +560,24 @@ __device__ __forceinline__ void uth_coef(const Consts<double>& P, bool at_on, do
   }
 }
 
-template <int QU, typename W>
-__device__ __forceinline__ void u_collide(const UthCoef<double>& c, double (&h)[QU], W wanted) {
+template <int QU>
+__device__ __forceinline__ void u_collide(const UthCoef<double>& c, double (&h)[QU]) {
   using T = double;
   using L = Lat<QU>;
   if (c.flat) {
 #pragma unroll
-    for (int i = 0; i < QU; ++i)
-      if (wanted(L::ey(i))) h[i] = rfma(c.A, h[i], c.K[L::cls(i)]);
+    for (int i = 0; i < QU; ++i) h[i] = rfma(c.A, h[i], c.K[L::cls(i)]);
     return;
   }
-  if (wanted(0)) h[0] = rfma(c.A, h[0], c.K[0]);
+  h[0] = rfma(c.A, h[0], c.K[0]);
 #pragma unroll
   for (int i = 1; i < QU; ++i) {
     const int j = L::opp(i);
     if (j < i) continue;
     const int k = L::cls(i);
     const T d = along<L>(i, c.jx[k], c.jy[k], c.jz[k]);
-    if (wanted(L::ey(i))) h[i] = rfma(c.A, h[i], radd(c.K[k], d));
-    if (wanted(L::ey(j))) h[j] = rfma(c.A, h[j], radd(c.K[k], -d));
+    h[i] = rfma(c.A, h[i], radd(c.K[k], d));
+    h[j] = rfma(c.A, h[j], radd(c.K[k], -d));
   }
 }
 

@@ -66,25 +66,18 @@ __device__ __forceinline__ F2 shifted(float ws, F2 ref, F2 raw) {
   return radd(raw, F2{rmul(ws, ref.x), rmul(ws, ref.y)});
 }
 
-struct AllLinks {
-  __device__ __forceinline__ constexpr bool operator()(int) const { return true; }
-};
-__device__ constexpr AllLinks all_links{};
-
 // Pulled populations of a pair; with REF, the raw stored number G plus the shift S w ref(source)
 // (FP16/BF16; ref: phi or theta of the step that stored it).  Off the y and z walls a link from
 // beyond an x wall is chosen by selects (NodeAt::core).
-// Only the links wanted(e_y) are read.
-template <int Q, typename S, bool HY, bool REF, bool FUSED, typename W>
+template <int Q, typename S, bool HY, bool REF, bool FUSED>
 __device__ __forceinline__ void pull2(const PairAt<HY>& at, int z, unsigned site, const S* __restrict__ pop,
-                                      const float* __restrict__ ref, float scale, F2 (&v)[Q], W wanted) {
+                                      const float* __restrict__ ref, float scale, F2 (&v)[Q]) {
   using L = Lat<Q>;
   using C = Codec<S>;
   if (at.core(z)) {
     const bool wl = at.a.x == 0, wr = at.b.x == at.b.nx - 1;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      if (!wanted(L::ey(i))) continue;
       const unsigned in = (unsigned)i * at.a.NS - (unsigned)(L::ez(i) * (int)at.a.plane + L::ey(i) * at.a.nx);
       const unsigned out = (unsigned)L::opp(i) * at.a.NS;
       if (L::ex(i) == 0) v[i] = ld2(pop + (site + in));
@@ -126,7 +119,6 @@ __device__ __forceinline__ void pull2(const PairAt<HY>& at, int z, unsigned site
       const NodeAt<HY>& at1 = n == 0 ? at.a : at.b;
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
-        if (!wanted(L::ey(i))) continue;
         const bool inside = at1.has(z, L::ex(i), L::ey(i), L::ez(i));
         const unsigned s = inside ? site + n - at1.template back<L>(i) : site + n;
         float g = C::raw(ldro(pop + ((unsigned)(inside ? i : L::opp(i)) * at1.NS + s)));
@@ -234,7 +226,7 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_PHI
     const F2 dz = rsub(cp, cm);
     const F2 U = ld2(Un + site), th = has_th ? ld2(thn + site) : theta0;
     F2 g[QP];
-    pull2<QP, S, HY, C::shifted, true>(at, z, site, gin, phim, scale, g, all_links);
+    pull2<QP, S, HY, C::shifted, true>(at, z, site, gin, phim, scale, g);
     const bool fa = !has_gradient(P, dx.x, dy.x, dz.x), fb = !has_gradient(P, dx.y, dy.y, dz.y);
     if (fa && fb) {  // bulk: no non-local term
       PhiCoef<float> ca, cb;
@@ -286,7 +278,7 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_MOM
   unsigned site = (unsigned)it.z0 * at.a.plane + at.a.p;
   for (int z = it.z0; z < it.z1; ++z, site += at.a.plane) {
     F2 v[QP];
-    pull2<QP, S, HY, C::shifted, false>(at, z, site, g, phin, scale, v, all_links);
+    pull2<QP, S, HY, C::shifted, false>(at, z, site, g, phin, scale, v);
     const F2 m = moment_sum2<QP>(at, z, v);
     st2(phinew + site, C::shifted ? rmul(m, both(iscale)) : m);
   }
@@ -330,8 +322,8 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_UTH
     const F2 yu = HY ? ld2(phi1 + (site + yp)) : cc, yd = HY ? ld2(phi1 + (site - ym)) : cc;
     const F2 U = ld2(Un + site), pn = ld2(phin + site), th = QT > 0 ? ld2(thn + site) : both(0.0f);
     F2 h[QU], f[QTL];
-    pull2<QU, S, HY, false, true>(at, z, site, hin, nullptr, 0.0f, h, all_links);
-    if (QT > 0) pull2<QTL, S, HY, C::shifted, true>(at, z, site, fin, thm, P.scale[2], f, all_links);
+    pull2<QU, S, HY, false, true>(at, z, site, hin, nullptr, 0.0f, h);
+    if (QT > 0) pull2<QTL, S, HY, C::shifted, true>(at, z, site, fin, thm, P.scale[2], f);
     UthCoef<float> ca, cb;
     uth_coef<QU, QT, S>(P, at_on, U.x, th.x, pn.x, cc.x, cc.y, l, yu.x, yd.x, cp.x, cm.x, ca);
     uth_coef<QU, QT, S>(P, at_on, U.y, th.y, pn.y, cc.y, r, cc.x, yu.y, yd.y, cp.y, cm.y, cb);
@@ -378,13 +370,13 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_MOM
   for (int z = it.z0; z < it.z1; ++z, site += at.a.plane) {
     {
       F2 v[QU];
-      pull2<QU, S, HY, false, false>(at, z, site, h, nullptr, 0.0f, v, all_links);
+      pull2<QU, S, HY, false, false>(at, z, site, h, nullptr, 0.0f, v);
       const F2 m = moment_sum2<QU>(at, z, v);
       st2(Unew + site, C::shifted ? rfma(m, both(P.inv_scale[1]), both(P.shift_h)) : m);
     }
     if (QT > 0) {
       F2 v[QTL];
-      pull2<QTL, S, HY, C::shifted, false>(at, z, site, f, thn, P.scale[2], v, all_links);
+      pull2<QTL, S, HY, C::shifted, false>(at, z, site, f, thn, P.scale[2], v);
       const F2 m = moment_sum2<QTL>(at, z, v);
       st2(thnew + site, C::shifted ? rmul(m, both(P.inv_scale[2])) : m);
     }

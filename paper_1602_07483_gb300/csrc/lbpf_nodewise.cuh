@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 8 ? LBPF_NODE64_BLO
     }
     PhiCoef<T> co;
     phi_coef<QP, S, true>(P, cc, U, th, dx, dy, radd(cp, -cm), wall, C::shifted ? ref[0] : T(0), co);
-    phi_collide<QP>(co, gp, gn, [](int) { return true; });
+    phi_collide<QP>(co, gp, gn);
 #pragma unroll
     for (int i = 0; i < QP; ++i) gout[(unsigned)i * at.NS + site] = C::pack(gp[i]);
     cm = cc;
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 8 ? LBPF_NODE64_BLO
     }
     UthCoef<T> co;
     uth_coef<QU, QT, S>(P, at_on, U, th, phn, cc, pxp, pxm, pyp, pym, cp, cm, co);
-    u_collide<QU>(co, h, [](int) { return true; });
+    u_collide<QU>(co, h);
 #pragma unroll
     for (int i = 0; i < QU; ++i) hout[(unsigned)i * at.NS + site] = C::pack(h[i]);
     if (QT > 0) {

@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(32, LBPF_PLANE_BLOCKS)
     if (in) {
       const F2 dx = rsub(F2{c.y, n.y}, F2{n.x, c.x}), dz = rsub(cp, cm);
       const F2 U = ld2(Un + site), th = has_th ? ld2(thn + site) : both(P.theta0);
-      pull2<QP, S, false, C::shifted, true>(at, z, site, gin, phim, P.scale[0], g, all_links);
+      pull2<QP, S, false, C::shifted, true>(at, z, site, gin, phim, P.scale[0], g);
       const bool fa = !has_gradient(P, dx.x, 0.0f, dz.x), fb = !has_gradient(P, dx.y, 0.0f, dz.y);
       PhiCoef<float> ca, cb;
       if (fa && fb) {  // bulk: no non-local term
@@ -203,8 +203,8 @@ __global__ void __launch_bounds__(32, LBPF_PLANE_BLOCKS)
     for (int i = 0; i < QTL; ++i) f[i] = both(0.0f);
     if (in) {
       const F2 U = ld2(Un + site), pn = ld2(phin + site), th = QT > 0 ? ld2(thn + site) : both(0.0f);
-      pull2<QU, S, false, false, true>(at, z, site, hin, nullptr, 0.0f, h, all_links);
-      if (QT > 0) pull2<QTL, S, false, C::shifted, true>(at, z, site, fin, thm, P.scale[2], f, all_links);
+      pull2<QU, S, false, false, true>(at, z, site, hin, nullptr, 0.0f, h);
+      if (QT > 0) pull2<QTL, S, false, C::shifted, true>(at, z, site, fin, thm, P.scale[2], f);
       UthCoef<float> ca, cb;
       uth_coef<QU, QT, S>(P, at_on, U.x, th.x, pn.x, c.x, c.y, n.x, c.x, c.x, cp.x, cm.x, ca);
       uth_coef<QU, QT, S>(P, at_on, U.y, th.y, pn.y, c.y, n.y, c.x, c.y, c.y, cp.y, cm.y, cb);

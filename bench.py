@@ -373,11 +373,18 @@ def run_own(args):
     return 0
 
 
+def kernel_sources():
+    """Every file that decides what the kernels of a step do and which of them run: all headers, the
+    translation units and the dispatch, and the build's flags."""
+    from paper_1602_07483_gb300 import build
+    return [os.path.join(build.CSRC, f) for f in sorted(build.HEADERS + build.SOURCES)] + [build.__file__]
+
+
 def kernel_source_hash():
     import hashlib
     h = hashlib.sha256()
-    for f in ("lbpf_dev.cuh",):
-        with open(os.path.join(ROOT, "paper_1602_07483_gb300", "csrc", f), "rb") as fh:
+    for f in kernel_sources():
+        with open(f, "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 

@@ -50,3 +50,19 @@ def test_own_arm_line_small():
     assert d["config"]["workload"].startswith("kh64")
     dev = d["developed"]
     assert dev["GLUPS"] > 0 and dev["after_steps"] >= 2000
+
+
+def test_recorded_traffic_is_tied_to_every_kernel_source():
+    """The recorded DRAM traffic counts as the present kernels' only while no file they are compiled
+    from has changed: every file that a translation unit includes is part of the hash."""
+    sys.path.insert(0, ROOT)
+    import re
+
+    import bench
+    hashed = {os.path.basename(f) for f in bench.kernel_sources()}
+    csrc = os.path.join(ROOT, "paper_1602_07483_gb300", "csrc")
+    for f in os.listdir(csrc):
+        assert f in hashed
+        with open(os.path.join(csrc, f)) as fh:
+            for inc in re.findall(r'#include "([^"]+)"', fh.read()):
+                assert os.path.basename(inc) in hashed or inc.endswith("include/lbpf.h")

@@ -237,6 +237,7 @@ def run_own(args):
     if args.autotune:
         sim.autotune(steps=2)
     by, zchunk = sim.get_tiling()
+    kernels_per_step = sim.step_launches
     sim.step(args.warmup)
     barrier_sync()
     clocks = ClockSampler(dev)
@@ -360,6 +361,8 @@ def run_own(args):
             "cpu_baseline": cpu,
             "e2e": e2e,
             # one per phase; a node-wise phase is two kernels (collision, moments), counted here as one
+            # and in full in kernels_per_step
+            "kernels_per_step": kernels_per_step,
             "gpu_launches": (1 if args.schedule == "one_launch" else 2) * args.steps,
             "clocks": clk,
             "developed": developed,

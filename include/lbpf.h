@@ -159,6 +159,10 @@ int lbpf_tip(lbpf_sim* sim, int32_t axis, const double centre_lu[3], double* x_t
 /* Number of steps taken since the last init / set_state / load. */
 int64_t lbpf_steps_done(const lbpf_sim* sim);
 
+/* Kernels that one step launches under the current tiling and schedule (one or two per
+ * phase, or one for the one-launch schedule). */
+int32_t lbpf_step_launches(const lbpf_sim* sim);
+
 /* Checkpoint: write / read a self-describing binary file (header with grid,
  * lattices, parameters, step count; then the post-streaming populations and the
  * moment fields phi^n, phi^{n-1}, U^n, theta^n, theta^{n-1}, all in FP64), so that a

@@ -751,6 +751,11 @@ int lbpf_destroy(lbpf_sim* s) {
 
 int64_t lbpf_steps_done(const lbpf_sim* s) { return s ? s->step_base + s->steps : -1; }
 
+int32_t lbpf_step_launches(const lbpf_sim* s) {
+  if (!s) return LBPF_EINVAL;
+  return s->ol.on ? 1 : s->plan.phase[0].n + s->plan.phase[1].n;
+}
+
 int lbpf_init_seed(lbpf_sim* s, int32_t n, const double* centres, const double* radii, double U0, double theta0) {
   if (!s || n < 1 || !centres || !radii) return LBPF_EINVAL;
   if (status(s)) return s->sticky;

@@ -80,6 +80,7 @@ def load(path: str = LIB_PATH):
             "lbpf_sums": ([_VP, _D], ctypes.c_int),
             "lbpf_tip": ([_VP, i32, _D, _D, _D], ctypes.c_int),
             "lbpf_steps_done": ([_VP], i64),
+            "lbpf_step_launches": ([_VP], i32),
             "lbpf_save": ([_VP, ctypes.c_char_p], ctypes.c_int),
             "lbpf_load": ([_VP, ctypes.c_char_p], ctypes.c_int),
             "lbpf_set_tiling": ([_VP, i32, i32], ctypes.c_int),
@@ -217,6 +218,11 @@ class Sim:
     @property
     def steps_done(self):
         return int(self._L.lbpf_steps_done(self._h))
+
+    @property
+    def step_launches(self):
+        """Kernels launched per step under the current tiling and schedule."""
+        return int(self._L.lbpf_step_launches(self._h))
 
     def save(self, path):
         _check(self._L.lbpf_save(self._h, os.fsencode(path)), "lbpf_save")

@@ -153,3 +153,16 @@ def test_tuning_starts_from_the_tiling_in_use(fake, shape, lattices, storage):
     assert s.get_tiling()[1] == 1000
     s.set_schedule("two_kernels")
     assert s.get_tiling()[1] == 1000
+
+
+@pytest.mark.parametrize("shape,lattices,storage", SIMS)
+def test_step_launches_counts_the_kernels(fake, shape, lattices, storage):
+    s = lbpf.Sim(shape, lattices, storage=storage)
+    for schedule in ("two_kernels", "one_launch"):
+        try:
+            s.set_schedule(schedule)
+        except lbpf.LbpfError:
+            continue
+        fake.clear()
+        s.step(8)
+        assert len(fake.launches()) == 8 * s.step_launches

@@ -347,8 +347,6 @@ template <int QP, typename S, int BYC>
 __global__ void __launch_bounds__(32 * MAX_BLOCK_ROWS, Lat<QP>::has_y ? LBPF_PHI_MIN_BLOCKS : LBPF_PHI2D_MIN_BLOCKS)
     k_phi(const SimDev* __restrict__ sims, const WorkItem* __restrict__ items, int s6) {
   const WorkItem it = items[blockIdx.x];
-  pdl_trigger();
-  pdl_wait();
   phi_tile<QP, S, BYC>(sims, it, s6);
 }
 
@@ -689,8 +687,6 @@ template <int QU, int QT, typename S, int BYC>
 __global__ void __launch_bounds__(32 * MAX_BLOCK_ROWS, Lat<QU>::has_y ? LBPF_UTH_MIN_BLOCKS : LBPF_UTH2D_MIN_BLOCKS)
     k_uth(const SimDev* __restrict__ sims, const WorkItem* __restrict__ items, int s6) {
   const WorkItem it = items[blockIdx.x];
-  pdl_trigger();
-  pdl_wait();
   uth_tile<QU, QT, S, false, BYC>(sims, it, s6);
 }
 

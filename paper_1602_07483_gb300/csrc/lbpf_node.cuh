@@ -28,17 +28,33 @@ __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
 __device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
 
-// Read-only (non-coherent) load: what a step kernel reads this way is never written by the
+// Read-only (non-coherent) load, for kernels that start after the kernels before them have ended
+// (the tiles, the planes and the one-launch step): what they read this way is never written by the
 // same launch.
 template <typename S>
 __device__ __forceinline__ S ldro(const S* p) { return __ldg(p); }
 
-// Programmatic dependent launch: the kernels of a step are launched so that the next one may
+// Programmatic dependent launch: the node-wise kernels are launched so that the next one may
 // start while the last blocks of this one still run.  pdl_trigger() allows that; pdl_wait()
 // returns once the kernels before have finished and their writes are visible, and comes
 // before the first access to what they write (or read, where this kernel writes it).
+//
+// Such a kernel reads what is still being written when it starts.  A non-coherent load is for data
+// that nobody writes during the whole kernel, and the compiler may move it up across the wait, so
+// these kernels use plain loads, which stay behind it.  They cost next to nothing: over 170 grids
+// of all storage types a step takes 0.95 to 1.02 of the time with non-coherent loads (geometric mean
+// 0.997).  The tiles and planes keep non-coherent loads (FP16 planes of 4000^2: 508 us per step, 536
+// with plain ones) and start after the kernel ahead has ended; starting early did not pay there
+// either: waiting blocks fill the SMs unevenly (841^2 FP16 tiles 64.6 us per step, 49.9 without).
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// RO: by ldro, otherwise a plain load.
+template <bool RO, typename S>
+__device__ __forceinline__ S ld(const S* p) {
+  if constexpr (RO) return ldro(p);
+  else return *p;
+}
 
 // Index of the first population of weight class c (0 rest, 1 axis, 2 diagonal).
 template <int Q>

@@ -27,12 +27,17 @@ __device__ __forceinline__ F2 rfma(F2 a, F2 b, F2 c) { return as_f2(__ffma2_rn(a
 __device__ __forceinline__ F2 rsub(F2 a, F2 b) { return rfma(b, both(-1.0f), a); }
 
 // Two consecutive stored numbers (the first at an even index), as raw FP32 values and back.
-__device__ __forceinline__ F2 ld2(const float* p) { return as_f2(__ldg(reinterpret_cast<const float2*>(p))); }
-__device__ __forceinline__ F2 ld2(const __half* p) {
-  return as_f2(__half22float2(__ldg(reinterpret_cast<const __half2*>(p))));
+template <bool RO>
+__device__ __forceinline__ F2 ld2(const float* p) {
+  return as_f2(ld<RO>(reinterpret_cast<const float2*>(p)));
 }
+template <bool RO>
+__device__ __forceinline__ F2 ld2(const __half* p) {
+  return as_f2(__half22float2(ld<RO>(reinterpret_cast<const __half2*>(p))));
+}
+template <bool RO>
 __device__ __forceinline__ F2 ld2(const __nv_bfloat16* p) {
-  return as_f2(__bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162*>(p))));
+  return as_f2(__bfloat1622float2(ld<RO>(reinterpret_cast<const __nv_bfloat162*>(p))));
 }
 __device__ __forceinline__ void st2(float* p, F2 v) { *reinterpret_cast<float2*>(p) = make_float2(v.x, v.y); }
 __device__ __forceinline__ void st2(__half* p, F2 v) { *reinterpret_cast<__half2*>(p) = __floats2half2_rn(v.x, v.y); }
@@ -69,7 +74,7 @@ __device__ __forceinline__ F2 shifted(float ws, F2 ref, F2 raw) {
 // Pulled populations of a pair; with REF, the raw stored number G plus the shift S w ref(source)
 // (FP16/BF16; ref: phi or theta of the step that stored it).  Off the y and z walls a link from
 // beyond an x wall is chosen by selects (NodeAt::core).
-template <int Q, typename S, bool HY, bool REF, bool FUSED>
+template <int Q, typename S, bool HY, bool REF, bool FUSED, bool RO>
 __device__ __forceinline__ void pull2(const PairAt<HY>& at, int z, unsigned site, const S* __restrict__ pop,
                                       const float* __restrict__ ref, float scale, F2 (&v)[Q]) {
   using L = Lat<Q>;
@@ -80,14 +85,14 @@ __device__ __forceinline__ void pull2(const PairAt<HY>& at, int z, unsigned site
     for (int i = 0; i < Q; ++i) {
       const unsigned in = (unsigned)i * at.a.NS - (unsigned)(L::ez(i) * (int)at.a.plane + L::ey(i) * at.a.nx);
       const unsigned out = (unsigned)L::opp(i) * at.a.NS;
-      if (L::ex(i) == 0) v[i] = ld2(pop + (site + in));
+      if (L::ex(i) == 0) v[i] = ld2<RO>(pop + (site + in));
       else if (L::ex(i) > 0)
-        v[i] = F2{C::raw(ldro(pop + (site + (wl ? out : in - 1)))), C::raw(ldro(pop + (site + in)))};
+        v[i] = F2{C::raw(ld<RO>(pop + (site + (wl ? out : in - 1)))), C::raw(ld<RO>(pop + (site + in)))};
       else
-        v[i] = F2{C::raw(ldro(pop + (site + (in + 1)))), C::raw(ldro(pop + (site + (wr ? out + 1 : in + 2))))};
+        v[i] = F2{C::raw(ld<RO>(pop + (site + (in + 1)))), C::raw(ld<RO>(pop + (site + (wr ? out + 1 : in + 2))))};
     }
     if (REF) {
-      const F2 own = ld2(ref + site);
+      const F2 own = ld2<RO>(ref + site);
       // the rows (e_y, e_z) that the lattice pulls from, each read once
 #pragma unroll
       for (int ez = -1; ez <= 1; ++ez)
@@ -103,9 +108,9 @@ __device__ __forceinline__ void pull2(const PairAt<HY>& at, int z, unsigned site
             }
           if (!any) continue;
           const unsigned row = site - (unsigned)(ez * (int)at.a.plane + ey * at.a.nx);
-          const F2 m = ey == 0 && ez == 0 ? own : ld2(ref + row);
-          const float l = left ? ldro(ref + (wl ? site : row - 1)) : 0.0f;
-          const float r = right ? ldro(ref + (wr ? site + 1 : row + 2)) : 0.0f;
+          const F2 m = ey == 0 && ez == 0 ? own : ld2<RO>(ref + row);
+          const float l = left ? ld<RO>(ref + (wl ? site : row - 1)) : 0.0f;
+          const float r = right ? ld<RO>(ref + (wr ? site + 1 : row + 2)) : 0.0f;
 #pragma unroll
           for (int i = 0; i < Q; ++i)
             if (L::ey(i) == ey && L::ez(i) == ez)
@@ -121,8 +126,8 @@ __device__ __forceinline__ void pull2(const PairAt<HY>& at, int z, unsigned site
       for (int i = 0; i < Q; ++i) {
         const bool inside = at1.has(z, L::ex(i), L::ey(i), L::ez(i));
         const unsigned s = inside ? site + n - at1.template back<L>(i) : site + n;
-        float g = C::raw(ldro(pop + ((unsigned)(inside ? i : L::opp(i)) * at1.NS + s)));
-        if (REF) g = shifted<FUSED>(rmul(scale, (float)L::w(i)), ldro(ref + s), g);
+        float g = C::raw(ld<RO>(pop + ((unsigned)(inside ? i : L::opp(i)) * at1.NS + s)));
+        if (REF) g = shifted<FUSED>(rmul(scale, (float)L::w(i)), ld<RO>(ref + s), g);
         (n == 0 ? v[i].x : v[i].y) = g;
       }
     }
@@ -217,16 +222,16 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_PHI
   const int xr = a.x < a.nx - 2 ? 2 : 1, xl = a.x > 0 ? 1 : 0;  // mirror ghosts
   const int yp = HY && a.y < a.ny - 1 ? a.nx : 0, ym = HY && a.y > 0 ? a.nx : 0;
   unsigned site = (unsigned)it.z0 * a.plane + a.p;
-  F2 cm = ld2(phin + (it.z0 > 0 ? site - a.plane : site)), cc = ld2(phin + site);
+  F2 cm = ld2<false>(phin + (it.z0 > 0 ? site - a.plane : site)), cc = ld2<false>(phin + site);
   for (int z = it.z0; z < it.z1; ++z, site += a.plane) {
-    const F2 cp = z < a.nz - 1 ? ld2(phin + (site + a.plane)) : cc;
-    const float l = ldro(phin + (site - xl)), r = ldro(phin + (site + xr));
+    const F2 cp = z < a.nz - 1 ? ld2<false>(phin + (site + a.plane)) : cc;
+    const float l = ld<false>(phin + (site - xl)), r = ld<false>(phin + (site + xr));
     const F2 dx = rsub(F2{cc.y, r}, F2{l, cc.x});
-    const F2 dy = HY ? rsub(ld2(phin + (site + yp)), ld2(phin + (site - ym))) : both(0.0f);
+    const F2 dy = HY ? rsub(ld2<false>(phin + (site + yp)), ld2<false>(phin + (site - ym))) : both(0.0f);
     const F2 dz = rsub(cp, cm);
-    const F2 U = ld2(Un + site), th = has_th ? ld2(thn + site) : theta0;
+    const F2 U = ld2<false>(Un + site), th = has_th ? ld2<false>(thn + site) : theta0;
     F2 g[QP];
-    pull2<QP, S, HY, C::shifted, true>(at, z, site, gin, phim, scale, g);
+    pull2<QP, S, HY, C::shifted, true, false>(at, z, site, gin, phim, scale, g);
     const bool fa = !has_gradient(P, dx.x, dy.x, dz.x), fb = !has_gradient(P, dx.y, dy.y, dz.y);
     if (fa && fb) {  // bulk: no non-local term
       PhiCoef<float> ca, cb;
@@ -239,9 +244,9 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_PHI
       F2 gn[QP];
       const bool wa = !a.inner(z), wb = !at.b.inner(z);
 #pragma unroll
-      for (int i = 0; i < QP; ++i) gn[i] = ld2(gin + ((unsigned)i * a.NS + site));  // B = 0 at walls
+      for (int i = 0; i < QP; ++i) gn[i] = ld2<false>(gin + ((unsigned)i * a.NS + site));  // B = 0 at walls
       F2 ref = both(0.0f);
-      if (C::shifted) ref = ld2(phim + site);
+      if (C::shifted) ref = ld2<false>(phim + site);
       PhiCoef<float> ca, cb;
       phi_coef<QP, S, false>(P, cc.x, U.x, th.x, dx.x, dy.x, dz.x, wa, ref.x, ca);
       phi_coef<QP, S, false>(P, cc.y, U.y, th.y, dx.y, dy.y, dz.y, wb, ref.y, cb);
@@ -278,7 +283,7 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_MOM
   unsigned site = (unsigned)it.z0 * at.a.plane + at.a.p;
   for (int z = it.z0; z < it.z1; ++z, site += at.a.plane) {
     F2 v[QP];
-    pull2<QP, S, HY, C::shifted, false>(at, z, site, g, phin, scale, v);
+    pull2<QP, S, HY, C::shifted, false, false>(at, z, site, g, phin, scale, v);
     const F2 m = moment_sum2<QP>(at, z, v);
     st2(phinew + site, C::shifted ? rmul(m, both(iscale)) : m);
   }
@@ -315,15 +320,15 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_UTH
   const int xr = a.x < a.nx - 2 ? 2 : 1, xl = a.x > 0 ? 1 : 0;  // mirror ghosts
   const int yp = HY && a.y < a.ny - 1 ? a.nx : 0, ym = HY && a.y > 0 ? a.nx : 0;
   unsigned site = (unsigned)it.z0 * a.plane + a.p;
-  F2 cm = ld2(phi1 + (it.z0 > 0 ? site - a.plane : site)), cc = ld2(phi1 + site);
+  F2 cm = ld2<false>(phi1 + (it.z0 > 0 ? site - a.plane : site)), cc = ld2<false>(phi1 + site);
   for (int z = it.z0; z < it.z1; ++z, site += a.plane) {
-    const F2 cp = z < a.nz - 1 ? ld2(phi1 + (site + a.plane)) : cc;
-    const float l = ldro(phi1 + (site - xl)), r = ldro(phi1 + (site + xr));
-    const F2 yu = HY ? ld2(phi1 + (site + yp)) : cc, yd = HY ? ld2(phi1 + (site - ym)) : cc;
-    const F2 U = ld2(Un + site), pn = ld2(phin + site), th = QT > 0 ? ld2(thn + site) : both(0.0f);
+    const F2 cp = z < a.nz - 1 ? ld2<false>(phi1 + (site + a.plane)) : cc;
+    const float l = ld<false>(phi1 + (site - xl)), r = ld<false>(phi1 + (site + xr));
+    const F2 yu = HY ? ld2<false>(phi1 + (site + yp)) : cc, yd = HY ? ld2<false>(phi1 + (site - ym)) : cc;
+    const F2 U = ld2<false>(Un + site), pn = ld2<false>(phin + site), th = QT > 0 ? ld2<false>(thn + site) : both(0.0f);
     F2 h[QU], f[QTL];
-    pull2<QU, S, HY, false, true>(at, z, site, hin, nullptr, 0.0f, h);
-    if (QT > 0) pull2<QTL, S, HY, C::shifted, true>(at, z, site, fin, thm, P.scale[2], f);
+    pull2<QU, S, HY, false, true, false>(at, z, site, hin, nullptr, 0.0f, h);
+    if (QT > 0) pull2<QTL, S, HY, C::shifted, true, false>(at, z, site, fin, thm, P.scale[2], f);
     UthCoef<float> ca, cb;
     uth_coef<QU, QT, S>(P, at_on, U.x, th.x, pn.x, cc.x, cc.y, l, yu.x, yd.x, cp.x, cm.x, ca);
     uth_coef<QU, QT, S>(P, at_on, U.y, th.y, pn.y, cc.y, r, cc.x, yu.y, yd.y, cp.y, cm.y, cb);
@@ -370,13 +375,13 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_MOM
   for (int z = it.z0; z < it.z1; ++z, site += at.a.plane) {
     {
       F2 v[QU];
-      pull2<QU, S, HY, false, false>(at, z, site, h, nullptr, 0.0f, v);
+      pull2<QU, S, HY, false, false, false>(at, z, site, h, nullptr, 0.0f, v);
       const F2 m = moment_sum2<QU>(at, z, v);
       st2(Unew + site, C::shifted ? rfma(m, both(P.inv_scale[1]), both(P.shift_h)) : m);
     }
     if (QT > 0) {
       F2 v[QTL];
-      pull2<QTL, S, HY, C::shifted, false>(at, z, site, f, thn, P.scale[2], v);
+      pull2<QTL, S, HY, C::shifted, false, false>(at, z, site, f, thn, P.scale[2], v);
       const F2 m = moment_sum2<QTL>(at, z, v);
       st2(thnew + site, C::shifted ? rmul(m, both(P.inv_scale[2])) : m);
     }

@@ -65,7 +65,7 @@ __device__ __forceinline__ void pull(const NodeAt<HY>& at, int z, unsigned site,
     for (int i = 0; i < Q; ++i) {
       const bool out = at.beyond(L::ex(i));
       const unsigned back = out ? 0u : at.template back<L>(i);
-      v[i] = C::raw(ldro(pop + (site + ((unsigned)(out ? L::opp(i) : i) * at.NS - back))));
+      v[i] = C::raw(ld<false>(pop + (site + ((unsigned)(out ? L::opp(i) : i) * at.NS - back))));
       src(i, site - back);
     }
   } else {
@@ -73,7 +73,7 @@ __device__ __forceinline__ void pull(const NodeAt<HY>& at, int z, unsigned site,
     for (int i = 0; i < Q; ++i) {
       const bool inside = at.has(z, L::ex(i), L::ey(i), L::ez(i));
       const unsigned s = inside ? site - at.template back<L>(i) : site;
-      v[i] = C::raw(ldro(pop + ((unsigned)(inside ? i : L::opp(i)) * at.NS + s)));
+      v[i] = C::raw(ld<false>(pop + ((unsigned)(inside ? i : L::opp(i)) * at.NS + s)));
       src(i, s);
     }
   }
@@ -163,22 +163,22 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 8 ? LBPF_NODE64_BLO
   const int xp = at.x < at.nx - 1 ? 1 : 0, xm = at.x > 0 ? 1 : 0;  // mirror ghosts
   const int yp = HY && at.y < at.ny - 1 ? at.nx : 0, ym = HY && at.y > 0 ? at.nx : 0;
   unsigned site = (unsigned)it.z0 * at.plane + at.p;
-  T cm = ldro(phin + (it.z0 > 0 ? site - at.plane : site)), cc = ldro(phin + site);
+  T cm = ld<false>(phin + (it.z0 > 0 ? site - at.plane : site)), cc = ld<false>(phin + site);
   for (int z = it.z0; z < it.z1; ++z, site += at.plane) {
-    const T cp = z < at.nz - 1 ? ldro(phin + (site + at.plane)) : cc;
-    const T dx = radd(ldro(phin + (site + xp)), -ldro(phin + (site - xm)));
-    const T dy = HY ? radd(ldro(phin + (site + yp)), -ldro(phin + (site - ym))) : T(0);
-    const T U = ldro(Un + site), th = has_th ? ldro(thn + site) : theta0;
+    const T cp = z < at.nz - 1 ? ld<false>(phin + (site + at.plane)) : cc;
+    const T dx = radd(ld<false>(phin + (site + xp)), -ld<false>(phin + (site - xm)));
+    const T dy = HY ? radd(ld<false>(phin + (site + yp)), -ld<false>(phin + (site - ym))) : T(0);
+    const T U = ld<false>(Un + site), th = has_th ? ld<false>(thn + site) : theta0;
     const bool wall = !at.inner(z);
     T gp[QP], gn[QP];
     T ref[C::shifted ? QP : 1];
     pull<QP, S>(at, z, site, gin, gp, [&](int i, unsigned s) {
-      if (C::shifted) ref[i] = ldro(phim + s);
+      if (C::shifted) ref[i] = ld<false>(phim + s);
     });
     const bool flat = !has_gradient(P, dx, dy, radd(cp, -cm));
     if (!flat) {  // no non-local term in the bulk
 #pragma unroll
-      for (int i = 0; i < QP; ++i) gn[i] = C::raw(ldro(gin + ((unsigned)i * at.NS + site)));  // B = 0 at walls
+      for (int i = 0; i < QP; ++i) gn[i] = C::raw(ld<false>(gin + ((unsigned)i * at.NS + site)));  // B = 0 at walls
     }
     if (C::shifted) {
 #pragma unroll
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(NODE_THREADS)
     T v[QP];
     T ref[C::shifted ? QP : 1];
     pull<QP, S>(at, z, site, g, v, [&](int i, unsigned s) {
-      if (C::shifted) ref[i] = ldro(phin + s);
+      if (C::shifted) ref[i] = ld<false>(phin + s);
     });
     if (C::shifted) {
 #pragma unroll
@@ -259,19 +259,19 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 8 ? LBPF_NODE64_BLO
   const int xp = at.x < at.nx - 1 ? 1 : 0, xm = at.x > 0 ? 1 : 0;  // mirror ghosts
   const int yp = HY && at.y < at.ny - 1 ? at.nx : 0, ym = HY && at.y > 0 ? at.nx : 0;
   unsigned site = (unsigned)it.z0 * at.plane + at.p;
-  T cm = ldro(phi1 + (it.z0 > 0 ? site - at.plane : site)), cc = ldro(phi1 + site);
+  T cm = ld<false>(phi1 + (it.z0 > 0 ? site - at.plane : site)), cc = ld<false>(phi1 + site);
   for (int z = it.z0; z < it.z1; ++z, site += at.plane) {
-    const T cp = z < at.nz - 1 ? ldro(phi1 + (site + at.plane)) : cc;
-    const T pxp = ldro(phi1 + (site + xp)), pxm = ldro(phi1 + (site - xm));
-    const T pyp = HY ? ldro(phi1 + (site + yp)) : cc, pym = HY ? ldro(phi1 + (site - ym)) : cc;
-    const T U = ldro(Un + site), phn = ldro(phin + site), th = QT > 0 ? ldro(thn + site) : T(0);
+    const T cp = z < at.nz - 1 ? ld<false>(phi1 + (site + at.plane)) : cc;
+    const T pxp = ld<false>(phi1 + (site + xp)), pxm = ld<false>(phi1 + (site - xm));
+    const T pyp = HY ? ld<false>(phi1 + (site + yp)) : cc, pym = HY ? ld<false>(phi1 + (site - ym)) : cc;
+    const T U = ld<false>(Un + site), phn = ld<false>(phin + site), th = QT > 0 ? ld<false>(thn + site) : T(0);
     T h[QU];
     T f[QTL];
     T ref[C::shifted && QT > 0 ? QTL : 1];
     pull<QU, S>(at, z, site, hin, h, [](int, unsigned) {});
     if (QT > 0) {
       pull<QTL, S>(at, z, site, fin, f, [&](int i, unsigned s) {
-        if (C::shifted) ref[i] = ldro(thm + s);
+        if (C::shifted) ref[i] = ld<false>(thm + s);
       });
       if (C::shifted) {
 #pragma unroll
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(NODE_THREADS)
       T v[QTL];
       T ref[C::shifted ? QTL : 1];
       pull<QTL, S>(at, z, site, f, v, [&](int i, unsigned s) {
-        if (C::shifted) ref[i] = ldro(thn + s);
+        if (C::shifted) ref[i] = ld<false>(thn + s);
       });
       if (C::shifted) {
 #pragma unroll

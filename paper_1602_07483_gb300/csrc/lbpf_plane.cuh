@@ -93,22 +93,20 @@ __global__ void __launch_bounds__(32, LBPF_PLANE_BLOCKS)
   const float* __restrict__ Un = (const float*)sd.U[par];
   const float* __restrict__ thn = (const float*)sd.th[s6 % 3];
   const bool has_th = sd.q_theta != 0;
-  pdl_trigger();
-  pdl_wait();
   const int zlo = max(it.z0 - 1, 0), zhi = min(it.z1, nz - 1);
   unsigned site = (unsigned)zlo * (unsigned)nx + (unsigned)(in ? at.a.x : 0);
-  F2 cm = ld2(phin + (zlo > 0 ? site - nx : site)), c = ld2(phin + site);
+  F2 cm = ld2<true>(phin + (zlo > 0 ? site - nx : site)), c = ld2<true>(phin + site);
   F2 a0 = both(0.0f), a1 = a0, a2 = a0;
   for (int z = zlo; z <= zhi; ++z, site += nx) {
-    const F2 cp = z < nz - 1 ? ld2(phin + (site + nx)) : c;
+    const F2 cp = z < nz - 1 ? ld2<true>(phin + (site + nx)) : c;
     const F2 n = beside(c, wl, wr);
     F2 g[QP];
 #pragma unroll
     for (int i = 0; i < QP; ++i) g[i] = both(0.0f);
     if (in) {
       const F2 dx = rsub(F2{c.y, n.y}, F2{n.x, c.x}), dz = rsub(cp, cm);
-      const F2 U = ld2(Un + site), th = has_th ? ld2(thn + site) : both(P.theta0);
-      pull2<QP, S, false, C::shifted, true>(at, z, site, gin, phim, P.scale[0], g);
+      const F2 U = ld2<true>(Un + site), th = has_th ? ld2<true>(thn + site) : both(P.theta0);
+      pull2<QP, S, false, C::shifted, true, true>(at, z, site, gin, phim, P.scale[0], g);
       const bool fa = !has_gradient(P, dx.x, 0.0f, dz.x), fb = !has_gradient(P, dx.y, 0.0f, dz.y);
       PhiCoef<float> ca, cb;
       if (fa && fb) {  // bulk: no non-local term
@@ -119,9 +117,9 @@ __global__ void __launch_bounds__(32, LBPF_PLANE_BLOCKS)
       } else {
         F2 gn[QP];
 #pragma unroll
-        for (int i = 0; i < QP; ++i) gn[i] = ld2(gin + ((unsigned)i * NS + site));  // factor 0 at walls
+        for (int i = 0; i < QP; ++i) gn[i] = ld2<true>(gin + ((unsigned)i * NS + site));  // factor 0 at walls
         F2 ref = both(0.0f);
-        if (C::shifted) ref = ld2(phim + site);
+        if (C::shifted) ref = ld2<true>(phim + site);
         phi_coef<QP, S, false>(P, c.x, U.x, th.x, dx.x, 0.0f, dz.x, !at.a.inner(z), ref.x, ca);
         phi_coef<QP, S, false>(P, c.y, U.y, th.y, dx.y, 0.0f, dz.y, !at.b.inner(z), ref.y, cb);
         const F2 omw{ca.omw, cb.omw}, noma2{-ca.oma2, -cb.oma2}, inv_a2{ca.inv_a2, cb.inv_a2};
@@ -187,14 +185,12 @@ __global__ void __launch_bounds__(32, LBPF_PLANE_BLOCKS)
   const float* __restrict__ thm = (const float*)sd.th[(s6 + 2) % 3];
   float* __restrict__ thnew = (float*)sd.th[(s6 + 1) % 3];
   const bool at_on = sd.antitrapping != 0;
-  pdl_trigger();
-  pdl_wait();
   const int zlo = max(it.z0 - 1, 0), zhi = min(it.z1, nz - 1);
   unsigned site = (unsigned)zlo * (unsigned)nx + (unsigned)(in ? at.a.x : 0);
-  F2 cm = ld2(phi1 + (zlo > 0 ? site - nx : site)), c = ld2(phi1 + site);
+  F2 cm = ld2<true>(phi1 + (zlo > 0 ? site - nx : site)), c = ld2<true>(phi1 + site);
   F2 u0 = both(0.0f), u1 = u0, u2 = u0, t0 = u0, t1 = u0, t2 = u0;
   for (int z = zlo; z <= zhi; ++z, site += nx) {
-    const F2 cp = z < nz - 1 ? ld2(phi1 + (site + nx)) : c;
+    const F2 cp = z < nz - 1 ? ld2<true>(phi1 + (site + nx)) : c;
     const F2 n = beside(c, wl, wr);
     F2 h[QU], f[QTL];
 #pragma unroll
@@ -202,9 +198,9 @@ __global__ void __launch_bounds__(32, LBPF_PLANE_BLOCKS)
 #pragma unroll
     for (int i = 0; i < QTL; ++i) f[i] = both(0.0f);
     if (in) {
-      const F2 U = ld2(Un + site), pn = ld2(phin + site), th = QT > 0 ? ld2(thn + site) : both(0.0f);
-      pull2<QU, S, false, false, true>(at, z, site, hin, nullptr, 0.0f, h);
-      if (QT > 0) pull2<QTL, S, false, C::shifted, true>(at, z, site, fin, thm, P.scale[2], f);
+      const F2 U = ld2<true>(Un + site), pn = ld2<true>(phin + site), th = QT > 0 ? ld2<true>(thn + site) : both(0.0f);
+      pull2<QU, S, false, false, true, true>(at, z, site, hin, nullptr, 0.0f, h);
+      if (QT > 0) pull2<QTL, S, false, C::shifted, true, true>(at, z, site, fin, thm, P.scale[2], f);
       UthCoef<float> ca, cb;
       uth_coef<QU, QT, S>(P, at_on, U.x, th.x, pn.x, c.x, c.y, n.x, c.x, c.x, cp.x, cm.x, ca);
       uth_coef<QU, QT, S>(P, at_on, U.y, th.y, pn.y, c.y, n.y, c.x, c.y, c.y, cp.y, cm.y, cb);

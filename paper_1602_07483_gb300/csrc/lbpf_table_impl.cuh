@@ -19,7 +19,7 @@ inline int aux_blocks(long long n) {
   return (int)(b < 1 ? 1 : b);
 }
 
-// Launch that may overlap the end of the kernel before it in the stream (pdl_wait).
+// Launch that may overlap the end of the kernel before it in the stream (pdl_wait): node-wise kernels.
 inline cudaError_t launch_pdl(void (*fn)(const SimDev*, const WorkItem*, int), dim3 g, dim3 b, size_t smem,
                               cudaStream_t st, const SimDev* sims, const WorkItem* items, int s6) {
   cudaLaunchAttribute at{};
@@ -38,24 +38,28 @@ inline cudaError_t launch_pdl(void (*fn)(const SimDev*, const WorkItem*, int), d
 template <int QP, typename S, int BYC>
 cudaError_t launch_phi(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
                        int s6) {
-  return launch_pdl(k_phi<QP, S, BYC>, g, b, smem, st, sims, items, s6);
+  k_phi<QP, S, BYC><<<g, b, smem, st>>>(sims, items, s6);
+  return cudaGetLastError();
 }
 
 template <int QU, int QT, typename S, int BYC>
 cudaError_t launch_uth(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
                        int s6) {
-  return launch_pdl(k_uth<QU, QT, S, BYC>, g, b, smem, st, sims, items, s6);
+  k_uth<QU, QT, S, BYC><<<g, b, smem, st>>>(sims, items, s6);
+  return cudaGetLastError();
 }
 
 template <int QP, typename S>
 cudaError_t launch_phi_plane(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
                              int s6) {
-  return launch_pdl(k_phi_plane<QP, S>, g, b, smem, st, sims, items, s6);
+  k_phi_plane<QP, S><<<g, b, smem, st>>>(sims, items, s6);
+  return cudaGetLastError();
 }
 template <int QU, int QT, typename S>
 cudaError_t launch_uth_plane(dim3 g, dim3 b, size_t smem, cudaStream_t st, const SimDev* sims, const WorkItem* items,
                              int s6) {
-  return launch_pdl(k_uth_plane<QU, QT, S>, g, b, smem, st, sims, items, s6);
+  k_uth_plane<QU, QT, S><<<g, b, smem, st>>>(sims, items, s6);
+  return cudaGetLastError();
 }
 
 // V nodes per thread (1 or 2; FP64 has no pairs)

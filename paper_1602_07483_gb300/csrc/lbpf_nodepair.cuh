@@ -243,13 +243,16 @@ __global__ void __launch_bounds__(NODE_THREADS, sizeof(S) == 2 ? LBPF_PAIR16_PHI
     } else {
       F2 gn[QP];
       const bool wa = !a.inner(z), wb = !at.b.inner(z);
-#pragma unroll
-      for (int i = 0; i < QP; ++i) gn[i] = ld2<false>(gin + ((unsigned)i * a.NS + site));  // B = 0 at walls
       F2 ref = both(0.0f);
       if (C::shifted) ref = ld2<false>(phim + site);
       PhiCoef<float> ca, cb;
       phi_coef<QP, S, false>(P, cc.x, U.x, th.x, dx.x, dy.x, dz.x, wa, ref.x, ca);
       phi_coef<QP, S, false>(P, cc.y, U.y, th.y, dx.y, dy.y, dz.y, wb, ref.y, cb);
+      // the non-local values after the coefficients, whose arithmetic then has the registers: before
+      // them they spilled (56 bytes), and FP32 512^3 with a gradient at most nodes took 15.03 ms per
+      // step, 14.71 so (14.77 as tiles)
+#pragma unroll
+      for (int i = 0; i < QP; ++i) gn[i] = ld2<false>(gin + ((unsigned)i * a.NS + site));  // B = 0 at walls
       const F2 omw{ca.omw, cb.omw}, noma2{-ca.oma2, -cb.oma2}, inv_a2{ca.inv_a2, cb.inv_a2};
 #pragma unroll
       for (int i = 0; i < QP; ++i) {

@@ -123,9 +123,9 @@ struct PhasePlan {
 struct StepPlan {
   PhasePlan phase[2];  // phi, then U and theta
   const SimDev* dd = nullptr;
-  // One phase tiled, the other node-wise.  A z-chunk asked for is then the tiles', whose halo planes
-  // it decides; the node-wise phase keeps its default (16 planes of phi against 32 of U and theta at
-  // 512^3 FP32, and no common chunk is as fast).
+  // One phase tiled, the other node-wise or as planes.  A z-chunk asked for is then the tiles', whose
+  // halo planes it decides; the other phase keeps its default (16 planes of phi against 32 of U and
+  // theta at 512^3 FP32, and no common chunk is as fast).
   bool mixed() const { return phase[0].node_wise() != phase[1].node_wise(); }
   bool takes_request(int f) const { return !mixed() || !phase[f].node_wise(); }
   int reporting() const { return takes_request(0) ? 0 : 1; }  // the phase whose z-chunk is reported
@@ -343,8 +343,10 @@ int set_smem_attrs(const KernelTable& t, const lbpf_lattice& l, int device) {
   return LBPF_OK;
 }
 
-// Kernels of a phase (0: phi, 1: U and theta) of lattices `l` in the given form, for blocks of `by` rows.
-void plan_kernels(PhasePlan& p, int phase, const KernelTable& t, const lbpf_lattice& l, int by, StepForm form) {
+// Kernels of a phase (0: phi, 1: U and theta) of lattices `l` in the given form, for blocks of `by` rows
+// and planes of up to `plane` nodes.
+void plan_kernels(PhasePlan& p, int phase, const KernelTable& t, const lbpf_lattice& l, int by, StepForm form,
+                  long long plane) {
   const int a = q_index(l.q_phi), b = q_index(l.q_u), c = qt_index(l.q_theta);
   p.form = form;
   p.smem = 0;
@@ -356,7 +358,7 @@ void plan_kernels(PhasePlan& p, int phase, const KernelTable& t, const lbpf_latt
     p.n = 2;
     p.fn[0] = phase == 0 ? t.phi_node[a][v] : t.uth_node[b][c][v];
     p.fn[1] = phase == 0 ? t.phi_moment[a][v] : t.uth_moment[b][c][v];
-    p.threads_x = node_threads(by);
+    p.threads_x = node_threads(by, plane, p.nodes());
   } else if (form == StepForm::plane) {
     p.fn[0] = phase == 0 ? t.phi_plane[a] : t.uth_plane[b][c];
   } else {
@@ -402,7 +404,24 @@ void adopt_plan(StepPlan& cur, OneLaunch& cur_ol, cudaGraphExec_t& gexec, bool& 
 // row and is aligned.
 bool takes_pairs(const KernelTable& t, const lbpf_grid& k) { return t.tbytes == 4 && k.nx % 2 == 0; }
 
-// The form of a phase (0: phi, 1: U and theta) for simulations of `sites` nodes in all.  Tiles read the
+// What the forms of a step go by, over all simulations stepped together.
+struct StepSize {
+  long long sites = 0;
+  long long plane = 0;  // nodes of the largest xy plane (2D: row)
+  bool pairs = true;
+};
+template <typename Sims>
+StepSize step_size(const KernelTable& t, const Sims& sims) {
+  StepSize z;
+  for (const lbpf_sim* s : sims) {
+    z.sites += s->nsite;
+    z.plane = std::max(z.plane, (long long)s->kg.nx * s->kg.ny);
+    z.pairs = z.pairs && takes_pairs(t, s->kg);
+  }
+  return z;
+}
+
+// The form of a phase (0: phi, 1: U and theta) of simulations stepped together.  Tiles read the
 // distributions once but spend 1.4 collisions per node, and small grids have too few tiles for
 // the chip; the node-wise forms read them twice.  Measured, microseconds per step (or of the phase):
 //   FP64, bound by its arithmetic, always node-wise: 128^3 D3Q19/D3Q19 tiled 2700, node-wise 816;
@@ -415,28 +434,40 @@ bool takes_pairs(const KernelTable& t, const lbpf_grid& k) { return t.tbytes == 
 //   4244 x 186 61 / 42, 1000^2 59 / 54), then planes for U and theta (2000^2 FP32 tiled 93, plane 83,
 //   8000^2 1279 / 1062), and for phi from 12 M nodes on (2000^2 84 / 111, 8000^2 1141 / 1093; whole
 //   step FP32 2409 / 2143, FP16 2490 / 1773), else tiles.
-StepForm choose_form(int phase, const KernelTable& t, const lbpf_lattice& l, long long sites, bool pairs) {
-  const StepForm node = pairs ? StepForm::node_pairs : StepForm::node;
+StepForm choose_form(int phase, const KernelTable& t, const lbpf_lattice& l, const StepSize& z) {
+  const StepForm node = z.pairs ? StepForm::node_pairs : StepForm::node;
   if (t.tbytes == 8) return node;
   if (lattice_is_2d(l.q_phi)) {
-    if (sites <= (pairs ? 1200000 : 700000)) return node;
-    return pairs && (phase == 1 || sites > 12000000) ? StepForm::plane : StepForm::tile;
+    if (z.sites <= (z.pairs ? 1200000 : 700000)) return node;
+    return z.pairs && (phase == 1 || z.sites > 12000000) ? StepForm::plane : StepForm::tile;
   }
-  if (t.sbytes == 2 || sites <= 8000000 || l.q_u + l.q_theta <= 26) return node;
-  return phase == 0 && pairs ? node : StepForm::tile;
+  if (t.sbytes == 2 || z.sites <= 8000000 || l.q_u + l.q_theta <= 26) return node;
+  return phase == 0 && z.pairs ? node : StepForm::tile;
 }
 
-// Appends a phase's work items of one simulation; returns the z-chunk used.  `zchunk` 0: the
-// default, for `blocks` node-wise blocks of a plane each in all.
+// Blocks per plane (2D: row) of a phase's form over all `sims`, counted at one plane each for the
+// node-wise forms.
+template <typename Sims>
+long long phase_blocks(const PhasePlan& p, const Sims& sims) {
+  long long n = 0;
+  for (const lbpf_sim* s : sims)
+    n += p.node_wise() ? node_blocks(s->kg.nx, s->kg.ny, s->kg.nz, p.span()) : (s->kg.nx + p.tile_x() - 1) / p.tile_x();
+  return n;
+}
+
+// The default z-chunk of a phase for one of the simulations stepped together, with `blocks` blocks in
+// all (phase_blocks).
+int phase_zchunk(const PhasePlan& p, const lbpf_grid& k, int by, long long blocks) {
+  if (p.node_wise()) return node_zchunk(blocks, k.nz);
+  return default_zchunk(k.nx, k.ny, k.nz, by);
+}
+
+// Appends a phase's work items of one simulation; returns the z-chunk used.  `zchunk` 0: the default.
 int phase_items(const PhasePlan& p, int sim, const lbpf_grid& k, int zchunk, int by, long long blocks,
                 std::vector<WorkItem>& items) {
-  if (p.node_wise()) {
-    const int zc = zchunk > 0 ? std::min(zchunk, k.nz) : node_zchunk(blocks, k.nz);
-    build_node_items(sim, k.nx, k.ny, k.nz, p.span(), zc, items);
-    return zc;
-  }
-  const int zc = zchunk > 0 ? zchunk : default_zchunk(k.nx, k.ny, k.nz, by);
-  build_items(sim, k.nx, k.ny, k.nz, by, zc, items, p.tile_x());
+  const int zc = zchunk > 0 ? zchunk : phase_zchunk(p, k, by, blocks);
+  if (p.node_wise()) build_node_items(sim, k.nx, k.ny, k.nz, p.span(), std::min(zc, k.nz), items);
+  else build_items(sim, k.nx, k.ny, k.nz, by, zc, items, p.tile_x());
   return zc;
 }
 
@@ -451,15 +482,16 @@ int build_tiling(lbpf_sim* s, int by, int zchunk, StepPlan& plan, OneLaunch& ol,
     return LBPF_ECUDA;
   plan.dd = s->dd;
   std::vector<WorkItem> items;
+  const lbpf_sim* sims[] = {s};
+  const StepSize size = step_size(t, sims);
   for (int f = 0; f < 2; ++f) {
-    plan_kernels(plan.phase[f], f, t, s->lat, by, choose_form(f, t, s->lat, s->nsite, takes_pairs(t, k)));
+    plan_kernels(plan.phase[f], f, t, s->lat, by, choose_form(f, t, s->lat, size), size.plane);
     if ((int)plan.phase[f].smem > maxsm) return LBPF_EINVAL;
   }
   for (int f = 0; f < 2; ++f) {
     PhasePlan& p = plan.phase[f];
     items.clear();
-    const int used = phase_items(p, 0, k, plan.takes_request(f) ? zchunk : 0, by,
-                                 node_blocks(k.nx, k.ny, k.nz, p.span()), items);
+    const int used = phase_items(p, 0, k, plan.takes_request(f) ? zchunk : 0, by, phase_blocks(p, sims), items);
     if (f == plan.reporting()) zc = zchunk > 0 ? zchunk : used;
     const int rc = plan_items(p, items, s->stream);
     if (rc != LBPF_OK) return rc;
@@ -1186,9 +1218,10 @@ int lbpf_autotune(lbpf_sim* s, int32_t steps, double* best_ms) {
   const bool node = p0.node_wise() && !s->ol.on;
   for (int by : {4, 6, 8}) {
     if (by > k.ny + 2 && by != 4) continue;
-    const int span = node_threads(by0 == 1 ? 1 : by) * p0.nodes();
-    const int zdef = node ? node_zchunk(node_blocks(k.nx, k.ny, k.nz, span), k.nz)
-                          : default_zchunk(k.nx, k.ny, k.nz, by);
+    PhasePlan q = p0;
+    if (node) q.threads_x = node_threads(by0 == 1 ? 1 : by, (long long)k.nx * k.ny, q.nodes());
+    const lbpf_sim* sims[] = {s};
+    const int zdef = s->ol.on ? default_zchunk(k.nx, k.ny, k.nz, by) : phase_zchunk(q, k, by0 == 1 ? 1 : by, phase_blocks(q, sims));
     const int longest = node ? std::min(k.nz, zdef * 4) : k.nz;
     for (int zc : {zdef, std::max(node ? 1 : 8, zdef / 2), std::min(k.nz, zdef * 2), longest}) cand.push_back({by, zc});
   }
@@ -1310,21 +1343,15 @@ static int build_batch_tiling(lbpf_batch* b, int by, int zchunk, StepPlan& plan,
   const KernelTable& t = *b->sims[0]->kt;
   const lbpf_lattice& l = b->sims[0]->lat;
   std::vector<WorkItem> items;
-  long long sites = 0;
-  bool pairs = true;
-  for (const lbpf_sim* s : b->sims) {
-    sites += s->nsite;
-    pairs = pairs && takes_pairs(t, s->kg);
-  }
+  const StepSize size = step_size(t, b->sims);
   // large chunks first, so that large and small simulations interleave
   auto by_chunk = [](const WorkItem& a, const WorkItem& c) { return (a.z1 - a.z0) > (c.z1 - c.z0); };
   plan.dd = b->dd;
-  for (int f = 0; f < 2; ++f) plan_kernels(plan.phase[f], f, t, l, by, choose_form(f, t, l, sites, pairs));
+  for (int f = 0; f < 2; ++f) plan_kernels(plan.phase[f], f, t, l, by, choose_form(f, t, l, size), size.plane);
   for (int f = 0; f < 2; ++f) {
     PhasePlan& p = plan.phase[f];
     const int zreq = plan.takes_request(f) ? zchunk : 0;
-    long long blocks = 0;  // of one plane each, over all members
-    for (const lbpf_sim* s : b->sims) blocks += node_blocks(s->kg.nx, s->kg.ny, s->kg.nz, p.span());
+    const long long blocks = phase_blocks(p, b->sims);
     items.clear();
     for (size_t i = 0; i < b->sims.size(); ++i) {
       const lbpf_grid& k = b->sims[i]->kg;

@@ -42,10 +42,15 @@ inline void build_node_items(int sim_index, int nx, int ny, int nz, int span, in
       out.push_back(WorkItem{sim_index, p0, 0, z0, std::min(nz, z0 + zchunk)});
 }
 
-// Threads of a node-wise block for a tiling of `by` rows (1: the 2D lattices, which have no rows
-// to choose).  128 (the default, by = 8) against 256 on GB300: 32^3 FP64 64 against 69 us per
-// step, 301^3 D3Q15/D3Q7/D3Q7 FP32 1835 against 1909 us, 256^3 FP16 the same.
-inline int node_threads(int by) { return by == 1 ? NODE_THREADS : 16 * by; }
+// Threads of a node-wise block, `nodes` nodes each, for a tiling of `by` rows (1: the 2D lattices, which
+// have no rows to choose).  128 (the default, by = 8) against 256 on GB300: 32^3 FP64 64 against
+// 69 us per step, 301^3 D3Q15/D3Q7/D3Q7 FP32 1835 against 1909 us, 256^3 FP16 the same.  Planes (in
+// 2D rows) of fewer nodes take whole warps only: 2D 40 x 4000 FP32 25.0 us per step with 128 threads,
+// 18.8 with 32; 16 x 8000 29.9, 22.9; 90 x 2000 18.1 with 128, 14.8 with 64.
+inline int node_threads(int by, long long plane, int nodes) {
+  const long long lanes = (plane + nodes - 1) / nodes;
+  return (int)std::min<long long>(by == 1 ? NODE_THREADS : 16 * by, (lanes + 31) / 32 * 32);
+}
 
 // Blocks of `span` nodes of a node-wise kernel at one plane each.
 inline long long node_blocks(int nx, int ny, int nz, int span) {

@@ -54,9 +54,9 @@ def fake(fake_path, monkeypatch):
     f.fail_malloc(-1, 0)
 
 
-# 3D and 2D, node-wise and tiled forms
+# 3D and 2D, node-wise, tiled and plane forms, and mixed ones
 SIMS = [((32, 32, 32), (15, 19, 0), "f64"), ((33, 20, 18), (19, 19, 7), "f32"), ((202, 202, 202), (19, 19, 19), "f32"),
-        ((64, 48, 1), (9, 5, 5), "f16"), ((1600, 1500, 1), (9, 5, 5), "bf16")]
+        ((64, 48, 1), (9, 5, 5), "f16"), ((1200, 1000, 1), (9, 5, 5), "f32"), ((1600, 1500, 1), (9, 5, 5), "bf16")]
 
 
 @pytest.mark.parametrize("shape,lattices,storage", SIMS)
@@ -166,3 +166,11 @@ def test_step_launches_counts_the_kernels(fake, shape, lattices, storage):
         fake.clear()
         s.step(8)
         assert len(fake.launches()) == 8 * s.step_launches
+
+
+def test_narrow_rows_take_whole_warps(fake):
+    for shape, threads in (((40, 400, 1), 32), ((90, 200, 1), 64), ((256, 20, 1), 128), ((300, 20, 1), 128)):
+        s = lbpf.Sim(shape, (9, 5, 5), storage="f32")
+        fake.clear()
+        s.step(1)
+        assert {int(l.split()[2]) for l in fake.launches()} == {threads}

@@ -126,8 +126,8 @@ struct StepPlan {
   // One phase tiled, the other node-wise or as planes.  A z-chunk asked for is then the tiles', whose
   // halo planes it decides; the other phase keeps its default (16 planes of phi against 32 of U and
   // theta at 512^3 FP32, and no common chunk is as fast).
-  bool mixed() const { return phase[0].node_wise() != phase[1].node_wise(); }
-  bool takes_request(int f) const { return !mixed() || !phase[f].node_wise(); }
+  bool mixed() const { return phase[0].form != phase[1].form; }
+  bool takes_request(int f) const { return !mixed() || phase[f].form == StepForm::tile; }
   int reporting() const { return takes_request(0) ? 0 : 1; }  // the phase whose z-chunk is reported
 };
 
@@ -459,7 +459,7 @@ long long phase_blocks(const PhasePlan& p, const Sims& sims) {
 // all (phase_blocks).
 int phase_zchunk(const PhasePlan& p, const lbpf_grid& k, int by, long long blocks) {
   if (p.node_wise()) return node_zchunk(blocks, k.nz);
-  return default_zchunk(k.nx, k.ny, k.nz, by);
+  return p.form == StepForm::plane ? plane_zchunk(blocks, k.nz) : default_zchunk(k.nx, k.ny, k.nz, by);
 }
 
 // Appends a phase's work items of one simulation; returns the z-chunk used.  `zchunk` 0: the default.

@@ -66,6 +66,16 @@ inline int node_zchunk(long long blocks, int nz) {
   return (int)std::max<long long>(1, std::min<long long>({zc, 16, (long long)nz}));
 }
 
+// Rows per block of the plane kernels: blocks are one warp each, 24 of which an SM holds, and run in
+// waves, so a simulation of `tiles` blocks per row takes one wave where chunks of 8 to 48 rows make
+// one, else chunks of 32 rows (two of which are recomputed).  2D FP16, us per step with chunks that
+// count 30-column tiles / these: 2000^2 D2Q9/D2Q5/D2Q5 183 / 134 (half a wave / one), 3000^2 330 / 279
+// (1.29 waves / one), D2Q9 x 3 466 / 384; 3400^2 in one wave of 54 rows FP32 D2Q9 x 3 666, in 32 rows 608.
+inline int plane_zchunk(long long tiles, int nz) {
+  const long long wave = 152 * 24, rows = (nz + std::max(1ll, wave / tiles) - 1) / std::max(1ll, wave / tiles);
+  return (int)std::min<long long>(nz, rows <= 48 ? std::max<long long>(rows, 8) : 32);
+}
+
 struct TileGeom {
   int nx, ny, nz, zchunk;
 };

@@ -174,3 +174,21 @@ def test_narrow_rows_take_whole_warps(fake):
         fake.clear()
         s.step(1)
         assert {int(l.split()[2]) for l in fake.launches()} == {threads}
+
+
+def test_plane_chunks_fill_whole_waves(fake):
+    """One-warp blocks, 24 to an SM: one wave where chunks of 8 to 48 rows make one, else 32 rows."""
+    for shape in ((2000, 2000, 1), (2100, 2100, 1), (3000, 3000, 1), (1030, 1100, 1)):
+        s = lbpf.Sim(shape, (9, 5, 5), storage="f16")
+        fake.clear()
+        s.step(1)
+        for l in fake.launches():
+            name, blocks, _, _, rows = l.split()
+            if "plane" not in name:
+                continue
+            assert 8 <= int(rows) <= 48 and int(blocks) <= 152 * 24
+            assert int(blocks) > 0.9 * 152 * 24 or int(rows) == 8
+    s = lbpf.Sim((5000, 5000, 1), (9, 5, 5), storage="f16")
+    fake.clear()
+    s.step(1)
+    assert {l.split()[-1] for l in fake.launches() if "plane" in l} == {"32"}

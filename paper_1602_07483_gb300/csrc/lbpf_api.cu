@@ -407,41 +407,55 @@ bool takes_pairs(const KernelTable& t, const lbpf_grid& k) { return t.tbytes == 
 // What the forms of a step go by, over all simulations stepped together.
 struct StepSize {
   long long sites = 0;
+  long long slots = 0;  // nodes of the node-wise blocks, the idle lanes at the end of a plane (2D: a row) too
   long long plane = 0;  // nodes of the largest xy plane (2D: row)
   bool pairs = true;
 };
 template <typename Sims>
-StepSize step_size(const KernelTable& t, const Sims& sims) {
+StepSize step_size(const KernelTable& t, const Sims& sims, int by) {
   StepSize z;
   for (const lbpf_sim* s : sims) {
     z.sites += s->nsite;
     z.plane = std::max(z.plane, (long long)s->kg.nx * s->kg.ny);
     z.pairs = z.pairs && takes_pairs(t, s->kg);
   }
+  const int nodes = z.pairs ? 2 : 1, span = node_threads(by, z.plane, nodes) * nodes;
+  for (const lbpf_sim* s : sims) z.slots += node_blocks(s->kg.nx, s->kg.ny, s->kg.nz, span) * span;
   return z;
 }
 
-// The form of a phase (0: phi, 1: U and theta) of simulations stepped together.  Tiles read the
-// distributions once but spend 1.4 collisions per node, and small grids have too few tiles for
-// the chip; the node-wise forms read them twice.  Measured, microseconds per step (or of the phase):
+// The form of a phase (0: phi, 1: U and theta).  Tiles read the distributions once but spend 1.4
+// collisions per node, and small grids have too few tiles for the chip; the node-wise forms read
+// them twice.  Measured, microseconds per step (or of the phase):
 //   FP64, bound by its arithmetic, always node-wise: 128^3 D3Q19/D3Q19 tiled 2700, node-wise 816;
 //   32^3 965 / 50; 8000^2 26500 / 23400.
 //   3D FP16/BF16 node-wise: 96^3 D3Q19/D3Q19/D3Q7 292 / 142 alone; 256^3 1860 / 1197 with pairs.
-//   3D FP32 node-wise with pairs: 96^3 229 / 91, 256^3 D3Q19/D3Q19/D3Q7 1680 / 1480; but U and theta both
-//   on D3Q19 (38 populations): 256^3 1233 / 1275, 512^3 9200 / 9810 tiled from 8 M nodes on.  With odd
-//   rows 301^3 D3Q15/D3Q7/D3Q7 2133 / 1779, D3Q19 x 3 tiled from 8 M nodes on (512^3 14430 / 15080).
-//   2D FP32, FP16 and BF16: node-wise while the second read stays in L2 (500^2 tiled 29, node-wise 15;
-//   4244 x 186 61 / 42, 1000^2 59 / 54), then planes for U and theta (2000^2 FP32 tiled 93, plane 83,
-//   8000^2 1279 / 1062), and for phi from 12 M nodes on (2000^2 84 / 111, 8000^2 1141 / 1093; whole
-//   step FP32 2409 / 2143, FP16 2490 / 1773), else tiles.
+//   3D FP32 node-wise below 8 M nodes: 96^3 with pairs 229 / 91, 193^3 D3Q19 x 3 938 / 929.
+//   From 8 M nodes on by the populations of U and theta.  Up to 26 node-wise: 256^3 D3Q19/D3Q19/D3Q7
+//   1679 / 1487, 301^3 (odd rows) 2768 / 2636, D3Q15/D3Q7/D3Q7 2191 / 1797.  30 and more as tiles, phi
+//   as pairs where rows are even (all tiled / all node-wise / phi as pairs, U and theta tiled): D3Q19/D3Q15/D3Q15
+//   256^3 1763 / 1630 / 1691, 301^3 2907 / 2885 / -; D3Q19 x 3 256^3 1938 / 1896 / 1865, 300^3 3026 / 3129 / 2984,
+//   301^3 3217 / 3409 / -, 512^3 14500 / 14737 / 14030 (with a gradient at most nodes 14580 / 15580 / 14710).
+//   2D FP32, FP16 and BF16 node-wise while a step is a matter of launches and of what stays in L2.
+//   Pairs FP32 to 0.7 M nodes and 0.85 M slots (D2Q9/D2Q5/D2Q5 as tiles, U and theta as planes / node-wise: 500^2
+//   24.6 / 14.1, 800^2 36.2 / 36.0, 900^2 42.6 / 46.2, 100000 x 8 36.7 / 42.2, 16 x 60000 in 3.8 M slots 88.7 / 112),
+//   16-bit to 1.05 M slots (all planes / node-wise: 900^2 D2Q9 x 3 64.9 / 56.3, 1100^2 81 / 92); odd rows FP32 to
+//   0.6 M slots (tiles / node-wise: 701^2 31.6 / 31.3, 841^2 39.3 / 47.8), 16-bit to 1.1 M (FP16 841^2 49.9 / 45.6,
+//   1301^2 94 / 101).
+//   Beyond, odd rows as tiles; even rows of 16 bits as planes (FP16 2000^2 tiles 192, planes 134).  FP32 even rows:
+//   planes from 4.5 M nodes on (2200^2 D2Q9/D2Q5/D2Q5 267 / 187, D2Q9 x 3 333 / 268; 3000^2 359 / 337, 485 / 505), below
+//   for U and theta of up to 14 populations (2000^2 D2Q9/D2Q5/D2Q5 169 / 155, D2Q9/D2Q9/D2Q5 187 / 178; D2Q9 x 3 214 / 220).
 StepForm choose_form(int phase, const KernelTable& t, const lbpf_lattice& l, const StepSize& z) {
   const StepForm node = z.pairs ? StepForm::node_pairs : StepForm::node;
+  const int q = l.q_u + l.q_theta;
   if (t.tbytes == 8) return node;
   if (lattice_is_2d(l.q_phi)) {
-    if (z.sites <= (z.pairs ? 1200000 : 700000)) return node;
-    return z.pairs && (phase == 1 || z.sites > 12000000) ? StepForm::plane : StepForm::tile;
+    if (!z.pairs) return z.slots <= (t.sbytes == 2 ? 1100000 : 600000) ? node : StepForm::tile;
+    if (t.sbytes == 2) return z.slots <= 1050000 ? node : StepForm::plane;
+    if (z.sites <= 700000 && z.slots <= 850000) return node;
+    return z.sites > 4500000 || (phase == 1 && q <= 14) ? StepForm::plane : StepForm::tile;
   }
-  if (t.sbytes == 2 || z.sites <= 8000000 || l.q_u + l.q_theta <= 26) return node;
+  if (t.sbytes == 2 || z.sites <= 8000000 || q <= 26) return node;
   return phase == 0 && z.pairs ? node : StepForm::tile;
 }
 
@@ -483,7 +497,7 @@ int build_tiling(lbpf_sim* s, int by, int zchunk, StepPlan& plan, OneLaunch& ol,
   plan.dd = s->dd;
   std::vector<WorkItem> items;
   const lbpf_sim* sims[] = {s};
-  const StepSize size = step_size(t, sims);
+  const StepSize size = step_size(t, sims, by);
   for (int f = 0; f < 2; ++f) {
     plan_kernels(plan.phase[f], f, t, s->lat, by, choose_form(f, t, s->lat, size), size.plane);
     if ((int)plan.phase[f].smem > maxsm) return LBPF_EINVAL;
@@ -1343,7 +1357,7 @@ static int build_batch_tiling(lbpf_batch* b, int by, int zchunk, StepPlan& plan,
   const KernelTable& t = *b->sims[0]->kt;
   const lbpf_lattice& l = b->sims[0]->lat;
   std::vector<WorkItem> items;
-  const StepSize size = step_size(t, b->sims);
+  const StepSize size = step_size(t, b->sims, by);
   // large chunks first, so that large and small simulations interleave
   auto by_chunk = [](const WorkItem& a, const WorkItem& c) { return (a.z1 - a.z0) > (c.z1 - c.z0); };
   plan.dd = b->dd;

@@ -168,6 +168,31 @@ def test_step_launches_counts_the_kernels(fake, shape, lattices, storage):
         assert len(fake.launches()) == 8 * s.step_launches
 
 
+# the form of each phase on both sides of the lines that choose it: narrow rows count with their idle
+# lanes, 16 bits and FP32 and odd rows have lines of their own, U and theta theirs
+NODE, PAIR, TILE, PLANE = ("node", "moment"), ("pair", "moment2"), ("",), ("plane",)
+FORMS = [((500, 500, 1), (9, 5, 5), "f32", PAIR, PAIR), ((900, 900, 1), (9, 5, 5), "f32", TILE, PLANE),
+         ((900, 900, 1), (9, 9, 9), "f32", TILE, TILE), ((100000, 8, 1), (9, 5, 5), "f32", TILE, PLANE),
+         ((16, 60000, 1), (9, 5, 5), "f32", TILE, PLANE), ((16, 8000, 1), (9, 5, 5), "f32", PAIR, PAIR),
+         ((2200, 2200, 1), (9, 9, 9), "f32", PLANE, PLANE), ((841, 841, 1), (9, 5, 5), "f32", TILE, TILE),
+         ((701, 701, 1), (9, 5, 5), "f32", NODE, NODE), ((1000, 1000, 1), (9, 9, 9), "f16", PAIR, PAIR),
+         ((1100, 1100, 1), (9, 9, 9), "bf16", PLANE, PLANE), ((1001, 1001, 1), (9, 5, 5), "f16", NODE, NODE),
+         ((1301, 1301, 1), (9, 5, 5), "f16", TILE, TILE), ((3000, 3000, 1), (9, 5, 5), "f64", NODE, NODE),
+         ((202, 202, 202), (19, 15, 15), "f32", PAIR, TILE), ((203, 203, 203), (19, 15, 15), "f32", TILE, TILE),
+         ((203, 203, 203), (19, 19, 7), "f32", NODE, NODE), ((203, 203, 203), (19, 19, 19), "bf16", NODE, NODE)]
+
+
+@pytest.mark.parametrize("shape,lattices,storage,phi,uth", FORMS)
+def test_forms(fake, shape, lattices, storage, phi, uth):
+    s = lbpf.Sim(shape, lattices, storage=storage)
+    s.step(1)
+    names = [l.split()[0] for l in fake.launches()]
+    want = [("k_phi_" if k else "k_phi") + k for k in phi] + [("k_uth_" if k else "k_uth") + k for k in uth]
+    assert len(names) == len(want)
+    for n, w in zip(names, want):
+        assert "%d%sI" % (len(w), w) in n
+
+
 def test_narrow_rows_take_whole_warps(fake):
     for shape, threads in (((40, 400, 1), 32), ((90, 200, 1), 64), ((256, 20, 1), 128), ((300, 20, 1), 128)):
         s = lbpf.Sim(shape, (9, 5, 5), storage="f32")
@@ -184,11 +209,9 @@ def test_plane_chunks_fill_whole_waves(fake):
         s.step(1)
         for l in fake.launches():
             name, blocks, _, _, rows = l.split()
-            if "plane" not in name:
-                continue
-            assert 8 <= int(rows) <= 48 and int(blocks) <= 152 * 24
+            assert "plane" in name and 8 <= int(rows) <= 48 and int(blocks) <= 152 * 24
             assert int(blocks) > 0.9 * 152 * 24 or int(rows) == 8
     s = lbpf.Sim((5000, 5000, 1), (9, 5, 5), storage="f16")
     fake.clear()
     s.step(1)
-    assert {l.split()[-1] for l in fake.launches() if "plane" in l} == {"32"}
+    assert [l.split()[-1] for l in fake.launches()] == ["32", "32"]

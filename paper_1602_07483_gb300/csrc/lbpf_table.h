@@ -18,9 +18,9 @@ struct KernelTable {
   int sbytes;            // bytes per stored population
   int tbytes;            // bytes of the compute type
   bool shifted;          // FP16/BF16 codec
-  // the tiled step (3D: FP32; 2D: all but FP64; null elsewhere), indexed by
-  // lattice_slot(q): 7, 15, 19, 5, 9; theta additionally 0 (frozen) in the last slot.
-  // Only pairings of one dimension are instantiated (the others are null).  Last index: the
+  // the tiled step (3D: FP32, U and theta of 30 populations and more; 2D: all but FP64; null
+  // elsewhere), indexed by lattice_slot(q): 7, 15, 19, 5, 9; theta additionally 0 (frozen) in the
+  // last slot.  Only pairings of one dimension are instantiated (the others are null).  Last index: the
   // block-height variant (block_variant): 1 for blocks of the height compiled in (8 rows in
   // 3D, one row in 2D), 0 for any height (the 2D entries are the one-row kernel in both).
   StepLaunch phi[5][2];

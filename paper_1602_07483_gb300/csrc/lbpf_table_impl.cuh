@@ -207,7 +207,8 @@ void fill_tile_kernels_2d(KernelTable& t) {
 #undef LBPF_UTH2
 }
 
-// The tiled step's 3D kernels (FP32), block height compiled in (BYC rows) or any (BYC = 0).
+// The tiled step's 3D kernels (FP32), block height compiled in (BYC rows) or any (BYC = 0): U and theta of
+// 30 populations and more (with fewer the step is node-wise at every size).
 template <typename S, int BYC>
 void fill_tile_kernels_3d(KernelTable& t) {
   constexpr int v = BYC > 0 ? 1 : 0;
@@ -219,9 +220,7 @@ void fill_tile_kernels_3d(KernelTable& t) {
 #define LBPF_UTH3(qa, qb)                                                              \
   t.uth[lattice_slot(qa)][lattice_slot(qb)][v] = launch_uth<qa, qb, S, BYC>;            \
   t.uth_fn[lattice_slot(qa)][lattice_slot(qb)][v] = (const void*)k_uth<qa, qb, S, BYC>;
-  LBPF_UTH3(7, 0) LBPF_UTH3(7, 7) LBPF_UTH3(7, 15) LBPF_UTH3(7, 19)
-  LBPF_UTH3(15, 0) LBPF_UTH3(15, 7) LBPF_UTH3(15, 15) LBPF_UTH3(15, 19)
-  LBPF_UTH3(19, 0) LBPF_UTH3(19, 7) LBPF_UTH3(19, 15) LBPF_UTH3(19, 19)
+  LBPF_UTH3(15, 15) LBPF_UTH3(15, 19) LBPF_UTH3(19, 15) LBPF_UTH3(19, 19)
 #undef LBPF_UTH3
 }
 

@@ -215,3 +215,18 @@ def test_plane_chunks_fill_whole_waves(fake):
     fake.clear()
     s.step(1)
     assert [l.split()[-1] for l in fake.launches()] == ["32", "32"]
+
+
+@pytest.mark.parametrize("storage", ["f64", "f32", "f16", "bf16"])
+def test_every_pairing_has_its_kernels(fake, storage):
+    """Tiled kernels exist only where some size takes them: every pairing steps, on both sides of the lines."""
+    for shape, qs in (((203, 203, 203), (7, 15, 19)), ((24, 20, 16), (7, 15, 19)), ((1301, 1301, 1), (5, 9)),
+                      ((2200, 2200, 1), (5, 9)), ((900, 900, 1), (5, 9)), ((40, 30, 1), (5, 9))):
+        for qu in qs:
+            for qt in qs + (0,):
+                s = lbpf.Sim(shape, (qs[0], qu, qt), storage=storage)
+                s.step(1)
+                s.set_tiling(5, 0)
+                s.step(1)
+                s.close()
+    assert fake.violations() == []

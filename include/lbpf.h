@@ -176,9 +176,9 @@ int lbpf_load(lbpf_sim* sim, const char* path);
  * 32 x by threads, one node per thread and plane) and z-chunk length
  * (>= 1; the z range is split into chunks processed by separate thread
  * blocks).  Steps that run node-wise (FP64, FP16 and BF16 on 3D lattices, FP32
- * and small 2D grids where that is faster) use blocks of 16 x by threads over
- * consecutive nodes of a plane; where only one phase of a step does, `zchunk` is
- * the other's (the tiles').  Results do not depend on the tiling.  0 keeps
+ * and small 2D grids where that is faster) use blocks of up to 16 x by threads over
+ * consecutive nodes of a plane; where the phases of a step take different forms,
+ * `zchunk` is the tiles'.  Results do not depend on the tiling.  0 keeps
  * the current value.  Takes effect at the next lbpf_step (the step graph is
  * re-captured).  LBPF_ENOMEM, tiling unchanged, when its work lists do not fit. */
 int lbpf_set_tiling(lbpf_sim* sim, int32_t by, int32_t zchunk);
@@ -191,8 +191,10 @@ int lbpf_autotune(lbpf_sim* sim, int32_t steps, double* best_ms);
 
 /* How a step is launched (the order of the work within a step follows Sec. 3.4:
  * phi first, then U and theta with phi^{n+1}; both schedules give bit-identical results).
- *   LBPF_SCHED_TWO_KERNELS (default): the phase-field kernel over all tiles, then the
- *     U/theta kernel over all tiles.
+ *   LBPF_SCHED_TWO_KERNELS (default): the phase-field phase over the whole grid, then the
+ *     U/theta phase.  A phase is one kernel over tiles, or a collision and a moment kernel
+ *     over the nodes (lbpf_step_launches), whichever is faster for the grid, lattices and
+ *     storage.
  *   LBPF_SCHED_ONE_LAUNCH: one persistent kernel per step in which the U/theta tile of a
  *     region starts as soon as the phase-field tiles that write phi^{n+1} around it are done,
  *     so that both phases run side by side on the SMs.  Its blocks wait on flags set by

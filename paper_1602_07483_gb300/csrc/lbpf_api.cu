@@ -1,7 +1,8 @@
 // lbpf_api.cu -- host runtime behind the C ABI of include/lbpf.h.
 //
-// Owns the device state of a simulation, validates parameters, builds the
-// tile work lists of the step kernels, captures the time loop in CUDA graphs
+// Owns the device state of a simulation, validates parameters, chooses the form of
+// each phase of a step and builds its work list (tiles, planes or node-wise
+// blocks), captures the time loop in CUDA graphs
 // (six steps per graph: populations alternate with period 2 and the phi levels
 // with period 3), and moves state between the host convention
 // (post-streaming populations, FP64) and the device pull layout.

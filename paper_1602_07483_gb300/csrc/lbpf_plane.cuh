@@ -12,7 +12,7 @@
 
 namespace lbpf {
 
-constexpr int PLANE_TILE_X = 60;
+static_assert(2 * TILE_X == 60, "lanes 1 to 30 of a warp, two nodes each");
 
 // The stored numbers that a pair of values becomes.
 template <typename S>
@@ -30,9 +30,9 @@ __device__ __forceinline__ F2 beside(F2 v, bool wl, bool wr) {
 
 // Adds a pair's arriving populations to the moments of rows z-1 (a0), z (a1) and z+1 (a2), the
 // links in index order; g: the pair's own post-collision populations (all lanes take part; only
-// those with `add` add).  The wall choices are selects on every lane: a separate path without them
-// for lanes off the walls came out of the compiler with links of the second node missing in FP32
-// (the bitwise tests of planes catch it).
+// those with `add` add).  The wall choices are selects on every lane.  A form with a separate path
+// without them, a branch around part of this loop of full-mask shuffles, gave wrong moments in FP32
+// and was dropped; its cause was not found.
 template <int Q>
 __device__ __forceinline__ void gather_row(const PairAt<false>& at, int z, bool add, const F2 (&g)[Q], F2& a0, F2& a1,
                                            F2& a2) {

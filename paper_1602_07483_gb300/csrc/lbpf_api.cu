@@ -344,10 +344,38 @@ int set_smem_attrs(const KernelTable& t, const lbpf_lattice& l, int device) {
   return LBPF_OK;
 }
 
+// Whether a step can take two nodes per thread: rows of even length, so that every pair lies in one
+// row and is aligned.
+bool takes_pairs(const KernelTable& t, const lbpf_grid& k) { return t.tbytes == 4 && k.nx % 2 == 0; }
+
+// What the forms of a step go by, over all simulations stepped together.
+struct StepSize {
+  long long sites = 0;
+  long long slots = 0;  // nodes of the node-wise blocks, the idle lanes at the end of a plane (2D: a row) too
+  long long plane = 0;  // nodes of the largest xy plane (2D: row)
+  bool pairs = true;
+  bool few = false;     // blocks of small planes take fewer warps
+};
+template <typename Sims>
+StepSize step_size(const KernelTable& t, const Sims& sims, int by) {
+  StepSize z;
+  long long planes = 0;
+  for (const lbpf_sim* s : sims) {
+    z.sites += s->nsite;
+    planes += s->kg.nz;
+    z.few = few_warps(lattice_is_2d(s->lat.q_phi), t.tbytes, t.sbytes, planes);
+    z.plane = std::max(z.plane, (long long)s->kg.nx * s->kg.ny);
+    z.pairs = z.pairs && takes_pairs(t, s->kg);
+  }
+  const int nodes = z.pairs ? 2 : 1, span = node_threads(by, z.plane, nodes, z.few) * nodes;
+  for (const lbpf_sim* s : sims) z.slots += node_blocks(s->kg.nx, s->kg.ny, s->kg.nz, span) * span;
+  return z;
+}
+
 // Kernels of a phase (0: phi, 1: U and theta) of lattices `l` in the given form, for blocks of `by` rows
-// and planes of up to `plane` nodes.
+// and simulations of size `z`.
 void plan_kernels(PhasePlan& p, int phase, const KernelTable& t, const lbpf_lattice& l, int by, StepForm form,
-                  long long plane) {
+                  const StepSize& z) {
   const int a = q_index(l.q_phi), b = q_index(l.q_u), c = qt_index(l.q_theta);
   p.form = form;
   p.smem = 0;
@@ -359,7 +387,7 @@ void plan_kernels(PhasePlan& p, int phase, const KernelTable& t, const lbpf_latt
     p.n = 2;
     p.fn[0] = phase == 0 ? t.phi_node[a][v] : t.uth_node[b][c][v];
     p.fn[1] = phase == 0 ? t.phi_moment[a][v] : t.uth_moment[b][c][v];
-    p.threads_x = node_threads(by, plane, p.nodes());
+    p.threads_x = node_threads(by, z.plane, p.nodes(), z.few);
   } else if (form == StepForm::plane) {
     p.fn[0] = phase == 0 ? t.phi_plane[a] : t.uth_plane[b][c];
   } else {
@@ -399,30 +427,6 @@ void adopt_plan(StepPlan& cur, OneLaunch& cur_ol, cudaGraphExec_t& gexec, bool& 
   cur = plan;
   free_one_launch(cur_ol);
   cur_ol = ol;
-}
-
-// Whether a step can take two nodes per thread: rows of even length, so that every pair lies in one
-// row and is aligned.
-bool takes_pairs(const KernelTable& t, const lbpf_grid& k) { return t.tbytes == 4 && k.nx % 2 == 0; }
-
-// What the forms of a step go by, over all simulations stepped together.
-struct StepSize {
-  long long sites = 0;
-  long long slots = 0;  // nodes of the node-wise blocks, the idle lanes at the end of a plane (2D: a row) too
-  long long plane = 0;  // nodes of the largest xy plane (2D: row)
-  bool pairs = true;
-};
-template <typename Sims>
-StepSize step_size(const KernelTable& t, const Sims& sims, int by) {
-  StepSize z;
-  for (const lbpf_sim* s : sims) {
-    z.sites += s->nsite;
-    z.plane = std::max(z.plane, (long long)s->kg.nx * s->kg.ny);
-    z.pairs = z.pairs && takes_pairs(t, s->kg);
-  }
-  const int nodes = z.pairs ? 2 : 1, span = node_threads(by, z.plane, nodes) * nodes;
-  for (const lbpf_sim* s : sims) z.slots += node_blocks(s->kg.nx, s->kg.ny, s->kg.nz, span) * span;
-  return z;
 }
 
 // The form of a phase (0: phi, 1: U and theta).  Tiles read the distributions once but spend 1.4
@@ -500,7 +504,7 @@ int build_tiling(lbpf_sim* s, int by, int zchunk, StepPlan& plan, OneLaunch& ol,
   const lbpf_sim* sims[] = {s};
   const StepSize size = step_size(t, sims, by);
   for (int f = 0; f < 2; ++f) {
-    plan_kernels(plan.phase[f], f, t, s->lat, by, choose_form(f, t, s->lat, size), size.plane);
+    plan_kernels(plan.phase[f], f, t, s->lat, by, choose_form(f, t, s->lat, size), size);
     if ((int)plan.phase[f].smem > maxsm) return LBPF_EINVAL;
   }
   for (int f = 0; f < 2; ++f) {
@@ -1230,12 +1234,13 @@ int lbpf_autotune(lbpf_sim* s, int32_t steps, double* best_ms) {
   std::vector<std::pair<int, int>> cand{{by0, zc0}};
   const lbpf_grid& k = s->kg;
   const PhasePlan& p0 = s->plan.phase[s->plan.reporting()];
+  const lbpf_sim* sims[] = {s};
+  const StepSize size = step_size(*s->kt, sims, by0);
   const bool node = p0.node_wise() && !s->ol.on;
   for (int by : {4, 6, 8}) {
     if (by > k.ny + 2 && by != 4) continue;
     PhasePlan q = p0;
-    if (node) q.threads_x = node_threads(by0 == 1 ? 1 : by, (long long)k.nx * k.ny, q.nodes());
-    const lbpf_sim* sims[] = {s};
+    if (node) q.threads_x = node_threads(by0 == 1 ? 1 : by, (long long)k.nx * k.ny, q.nodes(), size.few);
     const int zdef = s->ol.on ? default_zchunk(k.nx, k.ny, k.nz, by) : phase_zchunk(q, k, by0 == 1 ? 1 : by, phase_blocks(q, sims));
     const int longest = node ? std::min(k.nz, zdef * 4) : k.nz;
     for (int zc : {zdef, std::max(node ? 1 : 8, zdef / 2), std::min(k.nz, zdef * 2), longest}) cand.push_back({by, zc});
@@ -1362,7 +1367,7 @@ static int build_batch_tiling(lbpf_batch* b, int by, int zchunk, StepPlan& plan,
   // large chunks first, so that large and small simulations interleave
   auto by_chunk = [](const WorkItem& a, const WorkItem& c) { return (a.z1 - a.z0) > (c.z1 - c.z0); };
   plan.dd = b->dd;
-  for (int f = 0; f < 2; ++f) plan_kernels(plan.phase[f], f, t, l, by, choose_form(f, t, l, size), size.plane);
+  for (int f = 0; f < 2; ++f) plan_kernels(plan.phase[f], f, t, l, by, choose_form(f, t, l, size), size);
   for (int f = 0; f < 2; ++f) {
     PhasePlan& p = plan.phase[f];
     const int zreq = plan.takes_request(f) ? zchunk : 0;

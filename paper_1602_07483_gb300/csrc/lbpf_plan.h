@@ -44,12 +44,26 @@ inline void build_node_items(int sim_index, int nx, int ny, int nz, int span, in
 
 // Threads of a node-wise block, `nodes` nodes each, for a tiling of `by` rows (1: the 2D lattices, which
 // have no rows to choose).  128 (the default, by = 8) against 256 on GB300: 32^3 FP64 64 against
-// 69 us per step, 301^3 D3Q15/D3Q7/D3Q7 FP32 1835 against 1909 us, 256^3 FP16 the same.  Planes (in
-// 2D rows) of fewer nodes take whole warps only: 2D 40 x 4000 FP32 25.0 us per step with 128 threads,
-// 18.8 with 32; 16 x 8000 29.9, 22.9; 90 x 2000 18.1 with 128, 14.8 with 64.
-inline int node_threads(int by, long long plane, int nodes) {
+// 69 us per step, 301^3 D3Q15/D3Q7/D3Q7 FP32 1835 against 1909 us, 256^3 FP16 the same.  `few`: planes (in
+// 2D rows) of fewer nodes take whole warps only (few_warps).
+inline int node_threads(int by, long long plane, int nodes, bool few) {
+  const int most = by == 1 ? NODE_THREADS : 16 * by;
   const long long lanes = (plane + nodes - 1) / nodes;
-  return (int)std::min<long long>(by == 1 ? NODE_THREADS : 16 * by, (lanes + 31) / 32 * 32);
+  return few ? (int)std::min<long long>(most, (lanes + 31) / 32 * 32) : most;
+}
+
+// Whether the blocks of `planes` planes in all (in 2D rows) that are too small for a whole block take
+// fewer warps.  In 2D with FP32 arithmetic always: 40 x 4000 FP32 25.0 us per step with 128 threads, 18.8 with 32;
+// 16 x 8000 29.9, 22.9; 90 x 2000 18.1 with 128, 14.8 with 64.  In 3D and FP64, whose registers leave an SM
+// few warps, only where there are more blocks than the chip holds at once.  Fewer than that are placed
+// while the kernel ahead still runs, where it leaves room, and the more of them an SM takes the more
+// uneven that is: D3Q19/D3Q19/D3Q7 FP64, 800 planes of 4 x 4, 31.8 us with 128 threads, 56.1 with 32, and 29.8 with
+// 32 that were placed after the kernel ahead.  With 128 threads / whole warps: 8 x 8 FP64 3000 planes 122 / 111; 6 x 16
+// FP32 600 15.1 / 20.5, 2000 34.2 / 29.0; 12 x 12 FP16 300 17.7 / 20.9, 1200 34.3 / 28.4; 2D D2Q9/D2Q5/D2Q5 FP64 64 x 500
+// 24.2 / 32.6, 24 x 4000 42.2 / 39.5.
+inline bool few_warps(bool two_d, int tbytes, int sbytes, long long planes) {
+  if (two_d && tbytes == 4) return true;
+  return planes >= (tbytes == 8 ? 3000 : sbytes == 4 ? 2000 : 1200);
 }
 
 // Blocks of `span` nodes of a node-wise kernel at one plane each.

@@ -230,3 +230,17 @@ def test_every_pairing_has_its_kernels(fake, storage):
                 s.step(1)
                 s.close()
     assert fake.violations() == []
+
+
+def test_blocks_of_small_planes_stay_whole_where_few_of_them_run(fake):
+    """FP64 and 3D: whole blocks until there are more of them than the chip holds; in a batch all members count."""
+    for shapes, lattices, storage, threads in (
+            ([(64, 500, 1)], (9, 5, 5), "f64", 128), ([(64, 2999, 1)], (9, 5, 5), "f64", 128), ([(24, 3000, 1)], (9, 5, 5), "f64", 32),
+            ([(4, 4, 800)], (19, 19, 7), "f64", 128), ([(6, 16, 1999)], (19, 19, 7), "f32", 128),
+            ([(6, 16, 2000)], (19, 19, 7), "f32", 64), ([(6, 16, 1000)] * 2, (19, 19, 7), "f32", 64),
+            ([(12, 12, 300)], (19, 19, 7), "f16", 128), ([(12, 12, 1200)], (19, 19, 7), "bf16", 96)):
+        b = lbpf.Batch([lbpf.Sim(s, lattices, storage=storage) for s in shapes])
+        fake.clear()
+        b.step(1)
+        assert {int(l.split()[2]) for l in fake.launches()} == {threads}, (shapes, storage)
+        b.close()

@@ -352,6 +352,7 @@ bool takes_pairs(const KernelTable& t, const lbpf_grid& k) { return t.tbytes == 
 struct StepSize {
   long long sites = 0;
   long long slots = 0;  // nodes of the node-wise blocks, the idle lanes at the end of a plane (2D: a row) too
+  long long tile_slots = 0, plane_slots = 0;  // 2D: nodes of the tiles' and the planes' warps, halo lanes too
   long long plane = 0;  // nodes of the largest xy plane (2D: row)
   bool pairs = true;
   bool few = false;     // blocks of small planes take fewer warps
@@ -368,7 +369,11 @@ StepSize step_size(const KernelTable& t, const Sims& sims, int by) {
     z.pairs = z.pairs && takes_pairs(t, s->kg);
   }
   const int nodes = z.pairs ? 2 : 1, span = node_threads(by, z.plane, nodes, z.few) * nodes;
-  for (const lbpf_sim* s : sims) z.slots += node_blocks(s->kg.nx, s->kg.ny, s->kg.nz, span) * span;
+  for (const lbpf_sim* s : sims) {
+    z.slots += node_blocks(s->kg.nx, s->kg.ny, s->kg.nz, span) * span;
+    z.tile_slots += (long long)((s->kg.nx + TILE_X - 1) / TILE_X) * 32 * s->kg.nz;
+    z.plane_slots += (long long)((s->kg.nx + 2 * TILE_X - 1) / (2 * TILE_X)) * 64 * s->kg.nz;
+  }
   return z;
 }
 
@@ -429,6 +434,47 @@ void adopt_plan(StepPlan& cur, OneLaunch& cur_ol, cudaGraphExec_t& gexec, bool& 
   cur_ol = ol;
 }
 
+// The form of a phase (0: phi, 1: U and theta) on the 2D lattices with FP32 arithmetic: node-wise while a step
+// is a matter of launches and of what stays in L2, then tiles or planes.  "a / b": measured, microseconds
+// per step as tiles or planes / node-wise unless said otherwise.  Small differences in the lines come from
+// the populations of the lattices (what L2 holds) and from the lanes that a row idles in each form.
+StepForm choose_form_2d(int phase, const KernelTable& t, const lbpf_lattice& l, const StepSize& z) {
+  const int q = l.q_u + l.q_theta, all = l.q_phi + q;
+  const bool half = t.sbytes == 2;
+  if (!z.pairs) {  // odd rows
+    const bool tiles_idle = z.tile_slots >= z.slots;  // tiles idle as many lanes
+    // narrow rows, whose tiles idle more lanes: FP32 31 x 22580 67.8 / 41.7, 91 x 16483 95.3 / 81.7; FP16 45 x 33333
+    // 131.5 / 103.3, 91 x 16483 123.8 / 87.4.  FP32 rows that idle the same only while small: D2Q5/D2Q9/D2Q9
+    // 15 x 60000 94.4 / 108
+    if (z.plane <= 96 && z.sites <= 4500000 && (half || z.tile_slots > z.slots || z.sites <= 700000)) return StepForm::node;
+    // FP16 841^2 49.9 / 45.6, 1301^2 94 / 101; D2Q5/D2Q5 201 x 3980 39.7 / 46.1 in 1.02 M slots, 0.89 M of tiles
+    if (half) return z.slots <= 1100000 && (z.sites <= 700000 || tiles_idle) ? StepForm::node : StepForm::tile;
+    // 701^2 31.6 / 31.3, 97 x 5154 in 0.66 M slots 39.3 / 35.2, 841^2 in 0.75 M 39.3 / 47.8; 97 x 6185 in 0.79 M D2Q9/D2Q9
+    // 46.8 / 40.3, D2Q9/D2Q5/D2Q5 44.5 / 45.9
+    return z.slots <= 670000 || (all <= 18 && tiles_idle && z.sites <= 660000) ? StepForm::node : StepForm::tile;
+  }
+  // rows of 61 to 64 and 121 to 128 nodes, which pairs fill while planes take half as many slots again: FP32 64 x 15625
+  // 60.7 / 50.3, 128 x 11718 72.9 / 69.6; FP16 64 x 23437 D2Q9 x 3 121 / 79, 128 x 11718 100 / 81
+  if (z.sites <= 4500000 && 2 * z.plane_slots >= 3 * z.slots) return StepForm::node_pairs;
+  if (half) {
+    // D2Q9 x 3 900^2 64.9 / 56.3, 300 x 2333 in 1.19 M slots 58.9 / 51.7, 1100^2 in 1.27 M 81 / 92; D2Q9/D2Q5/D2Q5 300 x 2333
+    // 40.3 / 42.2; FP16 2000^2 tiles 192, planes 134
+    return z.slots <= (q == 18 ? 1200000 : 1050000) ? StepForm::node_pairs : StepForm::plane;
+  }
+  // 500^2 24.6 / 14.1, 800^2 36.2 / 36.0, 900^2 42.6 / 46.2, 100000 x 8 36.7 / 42.2, 16 x 60000 in 3.8 M slots 88.7 / 112;
+  // D2Q5/D2Q5 300 x 1666 in 0.85 M 24.2 / 21.5, 1000 x 800 27.4 / 24.6, 500 x 1800 32.2 / 28.1; D2Q5/D2Q9/D2Q9
+  // 2000 x 400 48.8 / 46.5
+  const bool light = l.q_phi == 5 || all <= 15;
+  if (z.sites <= (light ? 950000 : 700000) && z.slots <= (light ? 1000000 : 900000)) return StepForm::node_pairs;
+  // tiles / planes: 2000^2 D2Q9/D2Q5/D2Q5 169 / 155, D2Q9/D2Q9/D2Q5 187 / 178, D2Q9 x 3 214 / 220
+  if (phase == 1 && q <= 14) return StepForm::plane;
+  // rows of up to 30 nodes, where planes idle twice the lanes: 24 x 291666 D2Q9/D2Q5/D2Q5 phi as a tile 381, as a plane 407
+  if (z.plane_slots >= 2 * z.tile_slots) return z.sites > (phase == 0 ? 12000000 : 4500000) ? StepForm::plane : StepForm::tile;
+  // tiles / planes: 2200^2 D2Q9/D2Q5/D2Q5 267 / 187, D2Q9 x 3 333 / 268; 48 x 83333 D2Q9 x 3 329 / 223; U and theta alone
+  // 120 x 35833 D2Q9 x 3 293 / 260 per step, phi alone 1000 x 4400 168 / 173
+  return z.tile_slots > (phase == 0 ? 4800000 : 4400000) ? StepForm::plane : StepForm::tile;
+}
+
 // The form of a phase (0: phi, 1: U and theta).  Tiles read the distributions once but spend 1.4
 // collisions per node, and small grids have too few tiles for the chip; the node-wise forms read
 // them twice.  Measured, microseconds per step (or of the phase):
@@ -441,26 +487,11 @@ void adopt_plan(StepPlan& cur, OneLaunch& cur_ol, cudaGraphExec_t& gexec, bool& 
 //   as pairs where rows are even (all tiled / all node-wise / phi as pairs, U and theta tiled): D3Q19/D3Q15/D3Q15
 //   256^3 1763 / 1630 / 1691, 301^3 2907 / 2885 / -; D3Q19 x 3 256^3 1938 / 1896 / 1865, 300^3 3026 / 3129 / 2984,
 //   301^3 3217 / 3409 / -, 512^3 14500 / 14737 / 14030 (with a gradient at most nodes 14580 / 15580 / 14710).
-//   2D FP32, FP16 and BF16 node-wise while a step is a matter of launches and of what stays in L2.
-//   Pairs FP32 to 0.7 M nodes and 0.85 M slots (D2Q9/D2Q5/D2Q5 as tiles, U and theta as planes / node-wise: 500^2
-//   24.6 / 14.1, 800^2 36.2 / 36.0, 900^2 42.6 / 46.2, 100000 x 8 36.7 / 42.2, 16 x 60000 in 3.8 M slots 88.7 / 112),
-//   16-bit to 1.05 M slots (all planes / node-wise: 900^2 D2Q9 x 3 64.9 / 56.3, 1100^2 81 / 92); odd rows FP32 to
-//   0.6 M slots (tiles / node-wise: 701^2 31.6 / 31.3, 841^2 39.3 / 47.8), 16-bit to 1.1 M (FP16 841^2 49.9 / 45.6,
-//   1301^2 94 / 101).
-//   Beyond, odd rows as tiles; even rows of 16 bits as planes (FP16 2000^2 tiles 192, planes 134).  FP32 even rows:
-//   planes from 4.5 M nodes on (2200^2 D2Q9/D2Q5/D2Q5 267 / 187, D2Q9 x 3 333 / 268; 3000^2 359 / 337, 485 / 505), below
-//   for U and theta of up to 14 populations (2000^2 D2Q9/D2Q5/D2Q5 169 / 155, D2Q9/D2Q9/D2Q5 187 / 178; D2Q9 x 3 214 / 220).
 StepForm choose_form(int phase, const KernelTable& t, const lbpf_lattice& l, const StepSize& z) {
   const StepForm node = z.pairs ? StepForm::node_pairs : StepForm::node;
-  const int q = l.q_u + l.q_theta;
   if (t.tbytes == 8) return node;
-  if (lattice_is_2d(l.q_phi)) {
-    if (!z.pairs) return z.slots <= (t.sbytes == 2 ? 1100000 : 600000) ? node : StepForm::tile;
-    if (t.sbytes == 2) return z.slots <= 1050000 ? node : StepForm::plane;
-    if (z.sites <= 700000 && z.slots <= 850000) return node;
-    return z.sites > 4500000 || (phase == 1 && q <= 14) ? StepForm::plane : StepForm::tile;
-  }
-  if (t.sbytes == 2 || z.sites <= 8000000 || q <= 26) return node;
+  if (lattice_is_2d(l.q_phi)) return choose_form_2d(phase, t, l, z);
+  if (t.sbytes == 2 || z.sites <= 8000000 || l.q_u + l.q_theta <= 26) return node;
   return phase == 0 && z.pairs ? node : StepForm::tile;
 }
 

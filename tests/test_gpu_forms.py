@@ -76,3 +76,20 @@ def test_short_blocks_equal_whole_ones(storage, shape, wide, lattices):
     alone.step(13)
     _same(batch.sims[0], alone, state=True)
     batch.close()
+
+
+# D2Q9 phi as planes in BF16, and narrow rows: phi tiled beside planes, node-wise beyond the lines of wide rows
+@pytest.mark.parametrize("storage,shape,lattices", [("bf16", (1030, 1100, 1), (9, 5, 5)), ("f32", (120, 36700, 1), (9, 9, 9)),
+                                                    ("f32", (24, 200000, 1), (9, 5, 5)), ("f32", (64, 15625, 1), (9, 9, 0)),
+                                                    ("f16", (31, 22580, 1), (5, 9, 5))])
+def test_narrow_forms_equal_tiles(storage, shape, lattices):
+    p = workloads.base_params(kappa=100.0)
+    shapes = [shape, (1101, 1100, 1)]
+    batch = lbpf.Batch.create(shapes, lattices, [lbpf.make_params(storage, **p) for _ in shapes])
+    alone = lbpf.Sim(shape, lattices, storage=storage, **p)
+    _init([batch.sims[0], alone])
+    _init([batch.sims[1]])
+    batch.step(7)
+    alone.step(7)
+    _same(batch.sims[0], alone, state=True)
+    batch.close()

@@ -244,3 +244,24 @@ def test_blocks_of_small_planes_stay_whole_where_few_of_them_run(fake):
         b.step(1)
         assert {int(l.split()[2]) for l in fake.launches()} == {threads}, (shapes, storage)
         b.close()
+
+
+# narrow rows beyond the lines of wide ones: node-wise where tiles or planes idle more lanes than node-wise blocks
+NARROW_FORMS = [((31, 22580, 1), (9, 5, 5), "f32", NODE, NODE), ((45, 33333, 1), (9, 9, 9), "bf16", NODE, NODE),
+                ((91, 60000, 1), (9, 5, 5), "f16", TILE, TILE), ((64, 15625, 1), (9, 9, 9), "f32", PAIR, PAIR),
+                ((128, 11718, 1), (5, 5, 0), "f16", PAIR, PAIR), ((128, 40000, 1), (9, 5, 5), "f32", PLANE, PLANE),
+                ((48, 20834, 1), (9, 5, 5), "f32", TILE, PLANE), ((160, 12500, 1), (9, 5, 5), "f16", PLANE, PLANE),
+                ((97, 5154, 1), (9, 5, 5), "f32", NODE, NODE), ((97, 7216, 1), (9, 5, 5), "f32", TILE, TILE),
+                ((300, 1666, 1), (5, 5, 0), "f32", PAIR, PAIR), ((300, 2333, 1), (9, 9, 9), "f16", PAIR, PAIR),
+                ((300, 2333, 1), (9, 5, 5), "f16", PLANE, PLANE), ((48, 83333, 1), (9, 9, 9), "f32", PLANE, PLANE),
+                ((24, 291666, 1), (9, 9, 9), "f32", TILE, PLANE), ((24, 180000, 1), (9, 9, 9), "f32", TILE, TILE),
+                ((201, 3980, 1), (5, 5, 0), "f16", TILE, TILE), ((201, 3400, 1), (5, 5, 0), "f16", NODE, NODE),
+                ((1000, 800, 1), (5, 5, 0), "f32", PAIR, PAIR), ((1000, 800, 1), (9, 5, 5), "f32", TILE, PLANE),
+                ((45, 66666, 1), (9, 9, 9), "f32", TILE, TILE), ((91, 16483, 1), (9, 5, 5), "f32", NODE, NODE),
+                ((120, 35833, 1), (9, 9, 9), "f32", TILE, PLANE), ((97, 6701, 1), (9, 9, 0), "f32", NODE, NODE),
+                ((15, 60000, 1), (5, 9, 9), "f32", TILE, TILE), ((1000, 800, 1), (5, 9, 9), "f32", PAIR, PAIR)]
+
+
+@pytest.mark.parametrize("shape,lattices,storage,phi,uth", NARROW_FORMS)
+def test_forms_of_narrow_rows(fake, shape, lattices, storage, phi, uth):
+    test_forms(fake, shape, lattices, storage, phi, uth)
